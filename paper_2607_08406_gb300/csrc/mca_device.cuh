@@ -50,11 +50,14 @@ __host__ __device__ __forceinline__ uint4 trial_words(uint64_t seed, uint64_t ta
 // u = (r3 + 1/2) 2^-32, r3 the fourth Philox word of its counter, that is u < exp(-beta dS / N),
 // i.e. dS <= -(N / beta) ln u. msc = N / beta > 0. Evaluated in fp64 (once per candidate and
 // batch) and rounded to the fp32 of the candidate's dS.
-__host__ __device__ __forceinline__ float metropolis_theta(uint64_t seed, uint64_t tau,
-                                                             double msc) {
-  const uint32_t r3 = trial_words(seed, tau).w;
+__host__ __device__ __forceinline__ float metropolis_theta_word(uint32_t r3, double msc) {
   const double u = ((double)r3 + 0.5) * 0x1p-32;
   return (float)(-msc * log(u));
+}
+
+__host__ __device__ __forceinline__ float metropolis_theta(uint64_t seed, uint64_t tau,
+                                                             double msc) {
+  return metropolis_theta_word(trial_words(seed, tau).w, msc);
 }
 
 // Acceptance of a candidate with loss-sum change d (Eq. 6, or Eq. 7 when metro != 0).
@@ -188,23 +191,44 @@ __device__ __forceinline__ int batch_width_fast(float acc, float trials, float c
 // ------------------------------------------------------------------------------------------------
 // Transfer functions (Section 2) and losses (Eq. 2 with R = 0). ACT < 0 selects at run time.
 //
-// exp and log use the hardware base-2 units (__expf, __logf: a few ulp). tanh is its exponential
-// form tanh|x| = (1 - e^{-2|x|}) / (1 + e^{-2|x|}) with the sign restored: absolute error below
+// exp and log use the hardware base-2 units (a few ulp). tanh is its exponential form
+// tanh|x| = (1 - e^{-2|x|}) / (1 + e^{-2|x|}) with the sign restored: absolute error below
 // ~2e-7, far inside the 1e-5 relative tolerance on the loss sum. Exactness where it matters does not
 // depend on accuracy: an unchanged field gives f(z) - f(z) = 0 exactly because both sides go through
 // the same function.
+//
+// The base-2 units are used in their flush-to-zero form: a result below 2^-126 becomes 0, which
+// changes no sum with a term near 1 (1 -+ t of tanh and sigmoid, the softmax's largest term) and
+// moves a Gaussian activation by less than 2^-126. The other form costs three more instructions per
+// call (a range test and two scalings), and these functions are most of what a batch executes.
 // ------------------------------------------------------------------------------------------------
+__device__ __forceinline__ float ex2_ftz(float x) {
+  float r;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
+__device__ __forceinline__ float rcp_ftz(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
+constexpr float kLog2e = 1.4426950408889634f;
+
+__device__ __forceinline__ float exp_fast(float x) { return ex2_ftz(x * kLog2e); }
+
 __device__ __forceinline__ float tanh_exp(float x) {
-  const float t = __expf(-2.0f * fabsf(x));
-  return copysignf(__fdividef(1.0f - t, 1.0f + t), x);
+  const float t = ex2_ftz(fabsf(x) * (-2.0f * kLog2e));
+  return copysignf((1.0f - t) * rcp_ftz(1.0f + t), x);
 }
 
 __device__ __forceinline__ float act_rt(int act, float z, float g) {
   switch (act) {
     case MCA_ACT_TANH: return tanh_exp(z);
-    case MCA_ACT_SIGMOID: return __fdividef(1.0f, 1.0f + __expf(-z));
+    case MCA_ACT_SIGMOID: return rcp_ftz(1.0f + exp_fast(-z));
     case MCA_ACT_RELU: return fmaxf(z, 0.0f);
-    case MCA_ACT_GAUSSIAN: return __expf(-g * z * z);
+    case MCA_ACT_GAUSSIAN: return exp_fast(-g * z * z);
     case MCA_ACT_GELU: return 0.5f * z * (1.0f + erff(z * 0.7071067811865476f));
     default: return z;
   }
@@ -214,6 +238,20 @@ template <int ACT>
 __device__ __forceinline__ float act(float z, float g, int act_runtime) {
   if constexpr (ACT < 0) {
     return act_rt(act_runtime, z, g);
+  } else {
+    return act_rt(ACT, z, g);
+  }
+}
+
+// The same for code that is executed once per batch or per sample: a run-time transfer function is
+// called, not expanded in place (six functions per use: an unrolled loop over the output fields would
+// not stay in the instruction cache).
+static __device__ __noinline__ float act_call(int act, float z, float g) { return act_rt(act, z, g); }
+
+template <int ACT>
+__device__ __forceinline__ float act_compact(float z, float g, int act_runtime) {
+  if constexpr (ACT < 0) {
+    return act_runtime == MCA_ACT_IDENTITY ? z : act_call(act_runtime, z, g);
   } else {
     return act_rt(ACT, z, g);
   }
@@ -229,7 +267,7 @@ __device__ __forceinline__ float sample_loss(const float (&z)[MAXC], int C, int 
 #pragma unroll
     for (int k = 0; k < MAXC; ++k) {
       if (k < C) {
-        const float d = act<ACT2>(z[k], g2, act2_rt) - (k == y ? 1.0f : 0.0f);
+        const float d = act_compact<ACT2>(z[k], g2, act2_rt) - (k == y ? 1.0f : 0.0f);
         s = fmaf(d, d, s);
       }
     }
@@ -240,7 +278,7 @@ __device__ __forceinline__ float sample_loss(const float (&z)[MAXC], int C, int 
 #pragma unroll
   for (int k = 0; k < MAXC; ++k) {
     if (k < C) {
-      a[k] = act<ACT2>(z[k], g2, act2_rt);
+      a[k] = act_compact<ACT2>(z[k], g2, act2_rt);
       m = fmaxf(m, a[k]);
     }
   }
@@ -248,7 +286,7 @@ __device__ __forceinline__ float sample_loss(const float (&z)[MAXC], int C, int 
 #pragma unroll
   for (int k = 0; k < MAXC; ++k) {
     if (k < C) {
-      s += __expf(a[k] - m);
+      s += exp_fast(a[k] - m);
       if (k == y) ay = a[k];
     }
   }

@@ -56,11 +56,14 @@ constexpr int kWS = 96;
 constexpr int kCap = 160;
 constexpr int kWinBatch = 64;
 // Per-batch accumulator buffer of the windowed loop: one packed word per candidate (arrival count
-// in bits 56..63, count of out-of-range shares in 48..55, fixed-point sum below), padding. Three
-// buffers rotate. One warp reads a batch's words, two per lane; the count fields cap the ranges at
-// 255.
-constexpr int kAccStride = 2 * kKmax + 32;
+// in bits 56..63, count of out-of-range shares in 48..55, fixed-point sum below), kAccWord words
+// apart, so that the CTAs' additions to a batch's candidates go to different lines (and L2 slices)
+// instead of queueing at one. Four buffers rotate. One warp reads a batch's words, two per lane; the
+// count fields cap the ranges at 255.
+constexpr int kAccWord = 32;
 constexpr int kArrivalWord = 64;   // count-only word of a batch without a live candidate
+constexpr int kAccStride = (kArrivalWord + 1) * kAccWord;
+constexpr int kAccBuffers = 4;
 constexpr int kWindowMaxRanges = 255;
 static_assert(kWinBatch <= 64 && kWinBatch < kWS, "a windowed batch is read by one warp, two per lane");
 
@@ -113,7 +116,7 @@ struct Mlp2Args {
   int K;
   int fixed_K;
   float* partial;            // [2 x kKmax x NR] per-candidate, per-range loss changes
-  unsigned long long* accum; // [3 x kAccStride] windowed loop: fixed-point sums, counts, arrivals
+  unsigned long long* accum; // [kAccBuffers x kAccStride] windowed loop: fixed-point sums, counts, arrivals
   GridBarrier* bar;
   DevState* st;
   mca_trace_rec* trace;
