@@ -456,6 +456,14 @@ mca::DeepArgs deep_args(mca_handle* h) {
     a.whi[l] = h->tc && l >= 1 && l + 1 < a.L ? h->whi[l - 1] : nullptr;
   }
   a.tc = h->tc ? 1 : 0;
+  a.tc_f16 = h->tc_f16 ? 1 : 0;
+  if (h->tc_f16) {                   // the dense weights' bound to at most 2^15
+    int e = 0;
+    std::frexp(h->wbound, &e);
+    e = std::max(-90, e);
+    a.tc_wscale = std::ldexp(1.0f, 15 - e);
+    a.tc_dscale = std::ldexp(1.0f / mca::kDeepDScale, e - 15);
+  }
   a.off[a.L] = h->P;
   a.XT = h->XT;
   a.ell = h->ell;
@@ -534,6 +542,13 @@ mca_status resync(mca_handle* h) {
   return MCA_OK;
 }
 
+// The power of two above x >= 0.
+float pow2_above(float x) {
+  int e = 0;
+  std::frexp(x, &e);
+  return std::ldexp(1.0f, std::min(e, 126));
+}
+
 // Load parameters in the init format into the per-layer weight arrays.
 mca_status load_params(mca_handle* h, const float* params, const signed char* codes) {
   const bool pdev = is_device_ptr(params);
@@ -551,11 +566,13 @@ mca_status load_params(mca_handle* h, const float* params, const signed char* co
   }
   const float* src = pdev ? params : tmp;
   const signed char* csrc = codes ? (cdev ? codes : ctmp) : nullptr;
-  mca_status rc = MCA_OK;
-  int* dflag = nullptr;
-  cudaError_t e = cudaMalloc(&dflag, sizeof(int));
-  if (e == cudaSuccess) e = cudaMemsetAsync(dflag, 0, sizeof(int), h->stream);
+  int* dflag = nullptr;              // [0] a non-finite value; [1] the dense weights' largest magnitude
+  cudaError_t e = cudaMalloc(&dflag, 2 * sizeof(int));
+  if (e == cudaSuccess) e = cudaMemsetAsync(dflag, 0, 2 * sizeof(int), h->stream);
   if (e == cudaSuccess) e = mca::launch_count_nonfinite(src, P, dflag, h->stream);
+  if (e == cudaSuccess && h->tc_f16)
+    e = mca::launch_abs_max(src + h->off[1], h->off[h->layers.size() - 1] - h->off[1], dflag + 1,
+                            h->stream);
   for (size_t l = 0; e == cudaSuccess && l < h->layers.size(); ++l) {
     const mca_layer& L = h->layers[l];
     const size_t n = (size_t)L.n_in * L.n_out;
@@ -563,16 +580,27 @@ mca_status load_params(mca_handle* h, const float* params, const signed char* co
                                n, h->w_eff[l], h->code[l], h->wfix[l], h->stream);
     h->launches++;
   }
-  int hflag = 0;
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&hflag, dflag, sizeof(int), cudaMemcpyDeviceToHost,
+  int hflag[2] = {0, 0};
+  if (e == cudaSuccess) e = cudaMemcpyAsync(hflag, dflag, sizeof(hflag), cudaMemcpyDeviceToHost,
                                             h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   cudaFree(dflag);
   if (tmp) cudaFree(tmp);
   if (ctmp) cudaFree(ctmp);
   CUDA_TRY(h, e);
-  if (hflag) rc = fail(h, MCA_ERR_NUMERIC, "non-finite parameter value");
-  return rc;
+  if (hflag[0]) return fail(h, MCA_ERR_NUMERIC, "non-finite parameter value");
+  if (h->tc_f16) {
+    float top = 0.0f;
+    std::memcpy(&top, &hflag[1], sizeof(top));
+    float sc = 1.0f;                 // ternary layers hold codes
+    for (const mca_layer& L : h->layers)
+      if (L.wkind == MCA_W_TERNARY_I8) sc = std::max(sc, std::fabs(L.scale));
+    top *= sc;
+    if (h->dom.op == MCA_OP_REPLACE)
+      top = std::max(top, std::max(std::fabs(h->dom.lo), std::fabs(h->dom.hi)));
+    h->wbound = pow2_above(top);
+  }
+  return MCA_OK;
 }
 
 mca_status read_state(mca_handle* h, DevState* out) {
@@ -937,6 +965,8 @@ mca_status mca_create(const mca_layer* layers, int32_t n_layers, int32_t loss,
   CTRY(cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, h->device));
   h->deep = is_deep(ls);
   h->tc = h->deep && deep_tc_ok(ls);
+  h->tc_f16 = h->tc;                 // fp16 operand parts: every layer of the dense chain is tanh
+  for (size_t m = 1; m + 1 < ls.size(); ++m) h->tc_f16 = h->tc_f16 && ls[m].act == MCA_ACT_TANH;
   h->ntiles = h->tc ? deep_tc_tiles(h->N) : deep_tiles(h->N);
   if (!h->deep) {
     long long nnz = 0;
@@ -1203,6 +1233,15 @@ mca_status mca_run(mca_handle* h, uint64_t n_trials, uint64_t seed, mca_run_stat
           h->rest_ns += (uint64_t)(ms_c * 1e6f);
           h->ev_c_pending = false;
         }
+      }
+      if (h->tc_f16 && ctl.kstar >= 0 && std::fabs(ctl.acc.neww) > h->wbound) {
+        // a kept weight beyond the operands' scale (perturbations): split again with a larger one
+        h->wbound = pow2_above(std::fabs(ctl.acc.neww));
+        const uint64_t sd = a.seed;
+        a = deep_args(h);
+        a.seed = sd;
+        CUDA_TRY(h, mca::launch_deep_split(a, h->stream));
+        h->launches += 1;
       }
       h->tau += (uint64_t)ctl.consumed;
       remaining -= (uint64_t)ctl.consumed;
@@ -1656,6 +1695,8 @@ mca_status mca_run_channels(mca_handle* h, uint64_t n_trials, uint64_t seed, int
                                 h->stream));
     CUDA_TRY(h, cudaStreamSynchronize(h->stream));
   }
+  for (int m = 0; m < L; ++m)         // He values
+    h->wbound = std::max(h->wbound, pow2_above((float)std::sqrt(6.0 / (double)h->layers[m].n_in)));
   std::vector<int> node(L + 1);
   std::vector<float> oldw(L), neww(L);
   std::vector<float*> at(L);

@@ -361,12 +361,8 @@ __global__ void __launch_bounds__(kKmax) deep_decide_kernel(DeepArgs a) {
     const unsigned long long off = c.idx - a.off[l];
     a.w[l][off] = c.neww;
     if (a.wk[l] != MCA_W_FP32) a.code[l][off] = (signed char)c.new_code;
-    if (a.whi[l] != nullptr) {                      // split image of the tensor-core chain
-      const float h = tf32_rna(c.neww);
-      const size_t o = deep_tc_image_index(c.row, c.col);
-      a.whi[l][o] = h;
-      a.whi[l][o + 4096] = tf32_rna(c.neww - h);
-    }
+    // split image of the tensor-core chain
+    if (a.whi[l] != nullptr) deep_tc_image_store(a, l, c.row, c.col, c.neww);
   } else {
     ctl->consumed = Kb;
     atomicAdd(&st->trials, (unsigned long long)Kb);

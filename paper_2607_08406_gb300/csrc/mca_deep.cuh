@@ -2,6 +2,8 @@
 // chain (mca_deep_tc.cu): the candidate of trial tau + k, and the loss change of one sample.
 #pragma once
 
+#include <cuda_fp16.h>
+
 #include "mca_device.cuh"
 #include "mca_internal.h"
 
@@ -12,6 +14,30 @@ namespace mca {
 // (columns 4g .. 4g+3 of 256 rows form a 4 KB block). The lo part is 4096 floats further on.
 __host__ __device__ __forceinline__ size_t deep_tc_image_index(int r, int k) {
   return (size_t)(k >> 4) * 8192 + (size_t)((k >> 2) & 3) * 1024 + (size_t)r * 4 + (size_t)(k & 3);
+}
+
+// The same for fp16 parts: 8 chunks of 32 columns, each 32 KB (hi 16 KB, then lo), columns 8g .. 8g+7
+// of 256 rows forming a 4 KB block. In halves; the lo part is 8192 halves further on.
+__host__ __device__ __forceinline__ size_t deep_tc_image_index_f16(int r, int k) {
+  return (size_t)(k >> 5) * 16384 + (size_t)((k >> 3) & 3) * 2048 + (size_t)r * 8 + (size_t)(k & 7);
+}
+
+// Weight w = W_m[r][k] of a dense layer into its split image.
+__device__ __forceinline__ void deep_tc_image_store(const DeepArgs& a, int m, int r, int k,
+                                                    float w) {
+  if (a.tc_f16) {
+    __half* img = reinterpret_cast<__half*>(a.whi[m]);
+    const size_t o = deep_tc_image_index_f16(r, k);
+    const float x = w * a.tc_wscale;
+    const __half h = __float2half_rn(x);
+    img[o] = h;
+    img[o + 8192] = __float2half_rn(x - __half2float(h));
+  } else {
+    const size_t o = deep_tc_image_index(r, k);
+    const float h = tf32_rna(w);
+    a.whi[m][o] = h;
+    a.whi[m][o + 4096] = tf32_rna(w - h);
+  }
 }
 
 // Flat index of trial tau's weight from its first Philox word r0 (Eq. 1): uniform over all

@@ -1,31 +1,39 @@
 // Deep MLP path on the 5th-generation tensor cores: the dense part of a candidate's chain,
 //   Z'_m = Z_m + W_m (f(Z'_{m-1}) - f(Z_{m-1})),   m = l+2 .. L-2   (Section 2.4),
-// as error-compensated 3xTF32 tcgen05 MMAs with the accumulator in tensor memory.
+// as error-compensated three-product tcgen05 MMAs with the accumulator in tensor memory.
 //
 // One CTA per (candidate, tile of kTcTS = 128 samples): 16 worker warps and one control warp. Per
 // dense layer the CTA computes the transposed change D^T[samples x 256] = A[samples x 256] W_m^T,
-// where A holds the previous layer's activation changes split as A = A_hi + A_lo (each rounded to
-// tf32) and W_m = W_hi + W_lo (kept split in global memory, updated with every commit):
+// where A holds the previous layer's activation changes split as A = A_hi + A_lo and W_m = W_hi + W_lo
+// (kept split in global memory, updated with every commit), each part with an 11-bit significand:
 //   D = A_lo W_hi^T + A_hi W_lo^T + A_hi W_hi^T      (the A_lo W_lo^T term, ~2^-22 relative, dropped)
+// Tanh layers use fp16 parts (kind::f16, K = 16 per MMA): |change| <= 2 and the largest weight's
+// magnitude are scaled by powers of two to at most 2^15, so that an element x is represented to 2^-22 of
+// itself or 2^-40 of the largest, whichever is larger, and D is scaled back exactly. Layers whose
+// changes have no bound (ReLU, GELU, identity) or another function use tf32 parts (K = 8 per MMA,
+// the same time per MMA, hence half the rate).
 //
-// The layers are pipelined chunk by chunk. The workers produce A in K chunks of 16 features (hi and
-// lo, 16 KB) into a ring of four shared-memory slots; the control thread issues each chunk's six
-// MMAs as soon as the chunk and its weight stage are there, so layer m+1's MMAs run while the
-// workers are still forming layer m's later chunks. Two accumulators in tensor memory (columns
+// The layers are pipelined chunk by chunk. The workers produce A in K chunks (32 fp16 or 16 tf32
+// features; hi and lo, 16 KB) into a ring of four shared-memory slots; the control thread issues each
+// chunk's six MMAs as soon as the chunk and its weight stage are there, so layer m+1's MMAs run while
+// the workers are still forming layer m's later chunks. Two accumulators in tensor memory (columns
 // [0, 256) and [256, 512)) alternate by layer: the workers read layer m's finished D while the
-// MMAs of layer m+1 fill the other one. W streams through four 32 KB stages of 16-wide K chunks
-// (hi + lo), each one bulk copy, reaching across layer boundaries. All operands are K-major without
-// swizzle: 8-row x 16-byte core matrices.
+// MMAs of layer m+1 fill the other one. W streams through four 32 KB stages (one chunk, hi + lo),
+// each one bulk copy, reaching across layer boundaries. All operands are K-major without swizzle:
+// 8-row x 16-byte core matrices. One elected thread of the converged control warp issues the MMAs.
+// 24 layers of 256 on 10000 samples, about two candidates per batch: 400 us per batch with tf32 parts,
+// two exponentials and two reciprocals per element and 16 features a step; 259 us with fp16 parts,
+// one reciprocal and 32 features a step.
 //
 // Worker warp w reads tensor-memory lanes 32 (w mod 4) .. + 31 (its samples) and, in every chunk,
-// the four features 4 (w / 4) .. + 3: the cached field + D gives the new field, the next activation
+// one quarter of the features (part w / 4): the cached field + D gives the new field, the next activation
 // change f(z') - f(z) (exactly 0 where a field did not change) goes into the ring, and after the
 // last dense layer the changes accumulate into the output layer instead. Every per-(candidate,
 // tile) loss change depends only on that pair: the trajectory does not depend on the batch width.
 // COMMIT writes the fields exactly as the evaluation computed them. Every wait is bounded (2 s); on a
 // time-out the CTA records MCA_ERR_TIMEOUT, lets its issued copies and MMAs complete (bounded) and
 // frees its tensor memory.
-#include <cstdio>
+#include <cuda_fp16.h>
 
 #include "mca_deep.cuh"
 #include "mca_device.cuh"
@@ -40,23 +48,35 @@ constexpr int kTcThreads = (kWorkWarps + 1) * 32;   // + one control warp
 constexpr int kCtl = kWorkWarps * 32;                // the control thread
 constexpr int kParts = 4;                            // feature parts per lane quarter
 constexpr int kTcW = 256;                            // width of the dense layers
-constexpr int kTcKC = 16;                            // K chunk
-constexpr int kTcChunks = kTcW / kTcKC;
-constexpr int kAHalf = kTcTS * kTcKC * 4;            // 8 KB: hi or lo of one A chunk
+constexpr int kChunkBytes = 64;                      // K chunk of one row: 16 tf32 or 32 fp16
+constexpr int kAHalf = kTcTS * kChunkBytes;          // 8 KB: hi or lo of one A chunk
 constexpr int kASlot = 2 * kAHalf;
 constexpr int kASlots = 4;
-constexpr int kWHalfBytes = kTcW * kTcKC * 4;        // 16 KB: hi or lo of one W chunk
+constexpr int kWHalfBytes = kTcW * kChunkBytes;      // 16 KB: hi or lo of one W chunk
 constexpr int kWStageBytes = 2 * kWHalfBytes;        // 32 KB
 constexpr int kStages = 4;
 constexpr int kTcSmem = kASlots * kASlot + kStages * kWStageBytes;
 // core-matrix strides (bytes): A chunk: K groups 2 KB apart, sample groups 128 B apart;
 // W stage: K groups 4 KB apart, row groups 128 B apart. The split weights of a layer are kept in
-// global memory as kTcChunks consecutive 32 KB stage images (hi then lo), so that one bulk copy
+// global memory as consecutive 32 KB stage images, one per chunk (hi then lo), so that one bulk copy
 // fills a stage.
 constexpr uint32_t kALBO = (kTcTS / 8) * 128, kASBO = 128;
 constexpr uint32_t kWLBO = (kTcW / 8) * 128, kWSBO = 128;
-// kind::tf32, D fp32, A and B tf32 K-major, M = 128, N = 256
-constexpr uint32_t kIdesc = tc_idesc_tf32(kTcTS, kTcW);
+
+// The operand split (see the head of this file). kKC: features per chunk; kNQ: those of one worker
+// thread (one 16-byte core-matrix row); M = 128, N = 256, D fp32, operands K-major.
+template <bool F16>
+struct Split;
+template <>
+struct Split<false> {
+  static constexpr int kKC = 16, kNQ = 4;
+  static constexpr uint32_t kIdesc = tc_idesc_tf32(kTcTS, kTcW);
+};
+template <>
+struct Split<true> {
+  static constexpr int kKC = 32, kNQ = 8;
+  static constexpr uint32_t kIdesc = tc_idesc_f16(kTcTS, kTcW);
+};
 
 static_assert(kTcSmem + 2048 <= 227 * 1024, "shared memory of the chain kernel");
 static_assert((kParts - 1) * kMaxC * kTcTS * 4 <= kStages * kWStageBytes, "output scratch");
@@ -77,18 +97,28 @@ __device__ __forceinline__ void prefetch_tile(const float* Zm, int Np, int n0, i
   prefetch_l2(r + 32);
 }
 
-// Four accumulator columns of this thread's lane into r, left in flight: the values may be read only
-// after tmem_wait4(r).
-__device__ __forceinline__ void tmem_issue4(uint32_t taddr, uint32_t (&r)[4]) {
+// N (4 or 8) accumulator columns of this thread's lane into r, left in flight: the values may be read
+// only after tmem_wait(r).
+__device__ __forceinline__ void tmem_issue(uint32_t taddr, uint32_t (&r)[4]) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(taddr) : "memory");
+}
+__device__ __forceinline__ void tmem_issue(uint32_t taddr, uint32_t (&r)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
+                 "=r"(r[6]), "=r"(r[7]) : "r"(taddr) : "memory");
 }
 
 // Wait for this thread's tensor-memory loads; r is tied to the wait so that no read of it moves
 // above it.
-__device__ __forceinline__ void tmem_wait4(uint32_t (&r)[4]) {
+__device__ __forceinline__ void tmem_wait(uint32_t (&r)[4]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;"
                : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]) :: "memory");
+}
+__device__ __forceinline__ void tmem_wait(uint32_t (&r)[8]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]),
+                 "+r"(r[6]), "+r"(r[7]) :: "memory");
 }
 
 // Every lane waits for the phase; true in every lane iff no lane timed out.
@@ -96,23 +126,41 @@ __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity) {
   return __all_sync(0xffffffffu, mbar_wait(bar, parity) ? 1 : 0) != 0;
 }
 
-// Worker: put four activation changes of sample s (features 4 fp .. + 3 of the chunk) into ring
-// slot ga % kASlots as hi and lo tf32 parts, once the MMAs of the chunk kASlots earlier are done
-// with the slot; then the warp's arrival on the slot's full barrier.
+// x (two values) as fp16 hi and lo parts.
+__device__ __forceinline__ void split_f16x2(float x0, float x1, uint32_t& hi, uint32_t& lo) {
+  const __half2 h = __floats2half2_rn(x0, x1);
+  const float2 f = __half22float2(h);
+  const __half2 l = __floats2half2_rn(x0 - f.x, x1 - f.y);
+  hi = *reinterpret_cast<const uint32_t*>(&h);
+  lo = *reinterpret_cast<const uint32_t*>(&l);
+}
+
+// Worker: put the activation changes d of sample s (part fp of the chunk's features) into ring slot
+// ga % kASlots as hi and lo parts, once the MMAs of the chunk kASlots earlier are done with the slot;
+// then the warp's arrival on the slot's full barrier.
+template <bool F16, int NQ>
 __device__ __forceinline__ bool produce_chunk(unsigned char* aring, uint64_t* afull,
                                               uint64_t* aempty, int ga, int fp, int s,
-                                              const float (&d)[4]) {
+                                              const float (&d)[NQ]) {
   const int as = ga % kASlots;
   if (ga >= kASlots && !warp_wait(&aempty[as], (uint32_t)((ga / kASlots) - 1) & 1u)) return false;
-  float hi[4], lo[4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    hi[q] = tf32_rna(d[q]);
-    lo[q] = tf32_rna(d[q] - hi[q]);
-  }
   unsigned char* slot = aring + (size_t)as * kASlot + (size_t)fp * kALBO + (size_t)s * 16;
-  *reinterpret_cast<float4*>(slot) = make_float4(hi[0], hi[1], hi[2], hi[3]);
-  *reinterpret_cast<float4*>(slot + kAHalf) = make_float4(lo[0], lo[1], lo[2], lo[3]);
+  if constexpr (F16) {
+    uint32_t hi[4], lo[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) split_f16x2(d[2 * q], d[2 * q + 1], hi[q], lo[q]);
+    *reinterpret_cast<uint4*>(slot) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+    *reinterpret_cast<uint4*>(slot + kAHalf) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+  } else {
+    float hi[4], lo[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      hi[q] = tf32_rna(d[q]);
+      lo[q] = tf32_rna(d[q] - hi[q]);
+    }
+    *reinterpret_cast<float4*>(slot) = make_float4(hi[0], hi[1], hi[2], hi[3]);
+    *reinterpret_cast<float4*>(slot + kAHalf) = make_float4(lo[0], lo[1], lo[2], lo[3]);
+  }
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   tc_fence_before();
   __syncwarp();
@@ -121,9 +169,33 @@ __device__ __forceinline__ bool produce_chunk(unsigned char* aring, uint64_t* af
   return true;
 }
 
+// e^{2z}, z cut at 20 from above.
+__device__ __forceinline__ float exp2z(float z) {
+  float m;
+  asm("min.NaN.f32 %0, %1, 0f41A00000;" : "=f"(m) : "f"(z));
+  return ex2_ftz(m * (2.0f * kLog2e));
+}
+
+// Change of one hidden activation. F16 (tanh layers): kDeepDScale (tanh(zn) - tanh(zo)), exactly 0 when
+// zn == zo, from u = e^{2z} as 2 (un - uo) / ((un + 1)(uo + 1)): three of the special-function unit's
+// operations instead of four, and no cancellation between two rounded tanh values. z is cut at 20
+// (tanh = 1 to 2e-17) so that the product stays finite; a NaN stays a NaN.
+template <int ACTH, bool F16>
+__device__ __forceinline__ float act_change(float zn, float zo, float g, int act_rt_) {
+  if constexpr (F16) {
+    const float un = exp2z(zn), uo = exp2z(zo);
+    const float t = uo + 1.0f;
+    return (un - uo) * rcp_ftz(fmaf(un, t, t)) * (2.0f * kDeepDScale);
+  } else {
+    return zn != zo ? act<ACTH>(zn, g, act_rt_) - act<ACTH>(zo, g, act_rt_) : 0.0f;
+  }
+}
+
 // ACTH: transfer function of the hidden layers (-1: read per layer at run time).
-template <bool COMMIT, int ACTH>
+template <bool COMMIT, int ACTH, bool F16>
 __global__ void __launch_bounds__(kTcThreads, 1) deep_chain_tc_kernel(DeepArgs a) {
+  constexpr int kKC = Split<F16>::kKC, NQ = Split<F16>::kNQ, kChunks = kTcW / kKC;
+  constexpr uint32_t kIdesc = Split<F16>::kIdesc;
   extern __shared__ __align__(1024) unsigned char tsm[];
   unsigned char* aring = tsm;                                 // A chunks
   unsigned char* wst = tsm + kASlots * kASlot;                // W stages
@@ -232,7 +304,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) deep_chain_tc_kernel(DeepArgs a
   } else if (l < L - 2) {
     const bool dense = l + 2 <= L - 2;
     const int nd = dense ? (L - 2) - (l + 2) + 1 : 0;      // dense layers of the chain
-    const int nchunks = nd * kTcChunks;
+    const int nchunks = nd * kChunks;
     const bool worker = warp < kWorkWarps;
     const int qd = warp & 3, fp = (warp >> 2) & 3;        // lane quarter, feature part
     const int s = qd * 32 + lane, n = n0 + s;
@@ -274,16 +346,25 @@ __global__ void __launch_bounds__(kTcThreads, 1) deep_chain_tc_kernel(DeepArgs a
     for (int q = 0; q < kMaxC; ++q) outp[q] = 0.0f;
     const float* Wout = a.w[L - 1];
     const int Kout = a.n_in[L - 1];
+    auto out_add = [&](const float (&d)[NQ], int f0) {   // the output layer's change, features f0 ..
+#pragma unroll
+      for (int q = 0; q < NQ; ++q)
+#pragma unroll
+        for (int o = 0; o < kMaxC; ++o)
+          if (o < a.C) outp[o] = fmaf(Wout[(size_t)o * Kout + f0 + q], d[q], outp[o]);
+    };
 
     if (!worker) {
-      // ---- control thread: every dense layer's MMAs, chunk by chunk as the workers produce A
-      if (dense && lane == 0) {
+      // ---- control warp, one elected thread: every dense layer's MMAs, chunk by chunk as the
+      // workers produce A
+      if (dense && elect_one()) {
         const uint32_t sw = smem_u32(wst), sa = smem_u32(aring);
+        const uint64_t a0 = umma_desc(sa, kALBO, kASBO), w0 = umma_desc(sw, kWLBO, kWSBO);
         int issued_w = kStages - 1 < nchunks ? kStages - 1 : nchunks;   // weight chunks requested
         int landed_w = 0;                                               // ... and waited for
         bool ok = true;
         for (int gc = 0; gc < nchunks && ok; ++gc) {
-          const int li = gc / kTcChunks, cc = gc % kTcChunks;
+          const int li = gc / kChunks, cc = gc % kChunks;
           const int as = gc % kASlots, st = gc % kStages;
           if (!mbar_wait(&s_wfull[st], (uint32_t)(gc / kStages) & 1u)) {
             ok = false;
@@ -296,21 +377,29 @@ __global__ void __launch_bounds__(kTcThreads, 1) deep_chain_tc_kernel(DeepArgs a
           }
           tc_fence_after();
           const uint32_t dt = tmem + (uint32_t)(li & 1) * 256u;
+          // descriptors count 16-byte units
+          const uint64_t ab = a0 + (uint64_t)(as * (kASlot / 16));
+          const uint64_t wb = w0 + (uint64_t)(st * (kWStageBytes / 16));
 #pragma unroll
-          for (int ks = 0; ks < kTcKC / 8; ++ks) {
-            const uint32_t ab = sa + (uint32_t)(as * kASlot) + (uint32_t)ks * 2u * kALBO;
-            const uint32_t wb = sw + (uint32_t)(st * kWStageBytes) + (uint32_t)ks * 2u * kWLBO;
-            const uint64_t dahi = umma_desc(ab, kALBO, kASBO);
-            const uint64_t dalo = umma_desc(ab + kAHalf, kALBO, kASBO);
-            const uint64_t dwhi = umma_desc(wb, kWLBO, kWSBO);
-            const uint64_t dwlo = umma_desc(wb + kWHalfBytes, kWLBO, kWSBO);
-            mma_ss(dt, dalo, dwhi, kIdesc, (cc > 0 || ks > 0) ? 1u : 0u);
-            mma_ss(dt, dahi, dwlo, kIdesc, 1u);
-            mma_ss(dt, dahi, dwhi, kIdesc, 1u);
+          for (int ks = 0; ks < 2; ++ks) {           // K steps of 8 tf32 / 16 fp16: two K groups each
+            const uint64_t dahi = ab + (uint64_t)(ks * 2 * (kALBO / 16));
+            const uint64_t dalo = dahi + kAHalf / 16;
+            const uint64_t dwhi = wb + (uint64_t)(ks * 2 * (kWLBO / 16));
+            const uint64_t dwlo = dwhi + kWHalfBytes / 16;
+            const uint32_t first = (cc > 0 || ks > 0) ? 1u : 0u;
+            if constexpr (F16) {
+              mma_ss_f16(dt, dalo, dwhi, kIdesc, first);
+              mma_ss_f16(dt, dahi, dwlo, kIdesc, 1u);
+              mma_ss_f16(dt, dahi, dwhi, kIdesc, 1u);
+            } else {
+              mma_ss(dt, dalo, dwhi, kIdesc, first);
+              mma_ss(dt, dahi, dwlo, kIdesc, 1u);
+              mma_ss(dt, dahi, dwhi, kIdesc, 1u);
+            }
           }
           umma_commit(&s_aempty[as]);
           umma_commit(&s_wempty[st]);
-          if (cc == kTcChunks - 1) umma_commit(&s_dfull[li & 1]);
+          if (cc == kChunks - 1) umma_commit(&s_dfull[li & 1]);
           // chunk gc + kStages - 1 goes to the stage chunk gc - 1 used, once its MMAs are done
           const int nc = gc + kStages - 1;
           if (nc < nchunks) {
@@ -319,7 +408,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) deep_chain_tc_kernel(DeepArgs a
               ok = false;
               break;
             }
-            const int nl = l + 2 + nc / kTcChunks, nci = nc % kTcChunks;
+            const int nl = l + 2 + nc / kChunks, nci = nc % kChunks;
             load_stage(sw + (uint32_t)(ns * kWStageBytes),
                        reinterpret_cast<const unsigned char*>(a.whi[nl]) +
                            (size_t)nci * kWStageBytes,
@@ -334,14 +423,15 @@ __global__ void __launch_bounds__(kTcThreads, 1) deep_chain_tc_kernel(DeepArgs a
         for (int q = landed_w; q < issued_w; ++q)
           if (!mbar_wait(&s_wfull[q % kStages], (uint32_t)(q / kStages) & 1u)) s_fail = 1;
       }
+      __syncwarp();
     } else {
       // ---- workers
       bool ok = true;
       int ga = 0;                                         // A chunks produced
-      float zo_n[4];                                      // cached fields one chunk ahead
-      if (dense) prefetch_tile(a.Z[l + 2], Np, n0, tid);
+      const float dsc = F16 ? a.tc_dscale : 1.0f;         // the products' scale
       // layer l+1: rank-1 change through column j of W_{l+1}; its activation change is the first
       // A (dense) or feeds the output layer directly (l = L-3)
+      if (dense) prefetch_tile(a.Z[l + 2], Np, n0, tid);
       {
         const int m1 = l + 1;
         const float* W1 = a.w[m1];
@@ -350,56 +440,51 @@ __global__ void __launch_bounds__(kTcThreads, 1) deep_chain_tc_kernel(DeepArgs a
         float* Zm = a.Z[m1];
         const bool moves = live && da != 0.0f;
         // loads one chunk ahead of their use (n < Np: always in the array)
-        float wv[4], zo[4], wv_n[4];
+        float wv[NQ], zo[NQ], wv_n[NQ], zo_n[NQ];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          wv_n[q] = W1[(size_t)(fp * 4 + q) * K1 + j];
-          zo_n[q] = Zm[(size_t)(fp * 4 + q) * Np + n];
+        for (int q = 0; q < NQ; ++q) {
+          wv_n[q] = W1[(size_t)(fp * NQ + q) * K1 + j];
+          zo_n[q] = Zm[(size_t)(fp * NQ + q) * Np + n];
         }
-        for (int cc = 0; cc < kTcChunks; ++cc) {
-          const int f0 = cc * kTcKC + fp * 4;
-          float d[4];
+#pragma unroll 1
+        for (int cc = 0; cc < kChunks; ++cc) {
+          const int f0 = cc * kKC + fp * NQ;
+          float d[NQ];
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {
+          for (int q = 0; q < NQ; ++q) {
             wv[q] = wv_n[q];
             zo[q] = zo_n[q];
           }
-          if (cc + 1 < kTcChunks) {
+          if (cc + 1 < kChunks) {
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              wv_n[q] = W1[(size_t)(f0 + kTcKC + q) * K1 + j];
-              zo_n[q] = Zm[(size_t)(f0 + kTcKC + q) * Np + n];
+            for (int q = 0; q < NQ; ++q) {
+              wv_n[q] = W1[(size_t)(f0 + kKC + q) * K1 + j];
+              zo_n[q] = Zm[(size_t)(f0 + kKC + q) * Np + n];
             }
           }
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const float zn = fmaf(wv[q], da, zo[q]);
-            const bool ch = moves && zn != zo[q];
-            const float an = act<ACTH>(zn, a.g[m1], a.act[m1]);
-            const float ao = act<ACTH>(zo[q], a.g[m1], a.act[m1]);
-            d[q] = ch ? an - ao : 0.0f;
-            if (COMMIT && ch) Zm[(size_t)(f0 + q) * Np + n] = zn;
-            if (sk) sk[m1][(size_t)(f0 + q) * Np + n] = ch ? zn : zo[q];
+          for (int q = 0; q < NQ; ++q) {
+            const float zn = moves ? fmaf(wv[q], da, zo[q]) : zo[q];
+            d[q] = act_change<ACTH, F16>(zn, zo[q], a.g[m1], a.act[m1]);
+            if (COMMIT && zn != zo[q]) Zm[(size_t)(f0 + q) * Np + n] = zn;
+            if (sk) sk[m1][(size_t)(f0 + q) * Np + n] = zn;
           }
           if (dense) {
-            if (!produce_chunk(aring, s_afull, s_aempty, ga, fp, s, d)) {
+            if (!produce_chunk<F16>(aring, s_afull, s_aempty, ga, fp, s, d)) {
               ok = false;
               break;
             }
             ++ga;
           } else {
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-#pragma unroll
-              for (int o = 0; o < kMaxC; ++o)
-                if (o < a.C) outp[o] = fmaf(Wout[(size_t)o * Kout + f0 + q], d[q], outp[o]);
+            out_add(d, f0);
           }
         }
       }
       // dense layers m = l+2 .. L-2: read D of layer m as its MMAs finish, form the next A
+      float zo_n[NQ];                                     // cached fields one chunk ahead
       if (dense) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) zo_n[q] = a.Z[l + 2][(size_t)(fp * 4 + q) * Np + n];
+        for (int q = 0; q < NQ; ++q) zo_n[q] = a.Z[l + 2][(size_t)(fp * NQ + q) * Np + n];
       }
       for (int li = 0; li < nd && ok; ++li) {
         const int m = l + 2 + li;
@@ -411,57 +496,55 @@ __global__ void __launch_bounds__(kTcThreads, 1) deep_chain_tc_kernel(DeepArgs a
         }
         tc_fence_after();
         float* Zm = a.Z[m];
+        float* Sm = sk ? sk[m] : nullptr;
+        const float* Zn = last ? Zm : a.Z[m + 1];
         const uint32_t dt = tmem + lane_base + (uint32_t)(li & 1) * 256u;
         // accumulator columns one chunk ahead: chunk cc + 1's load is in flight while chunk cc is
         // processed
-        uint32_t dr[4], dr_n[4];
-        tmem_issue4(dt + (uint32_t)(fp * 4), dr_n);
-        tmem_wait4(dr_n);
-        for (int cc = 0; cc < kTcChunks; ++cc) {
-          const int f0 = cc * kTcKC + fp * 4;
-          float zo[4], dv[4], d[4];
+        uint32_t dr_n[NQ];
+        tmem_issue(dt + (uint32_t)(fp * NQ), dr_n);
+        tmem_wait(dr_n);
+#pragma unroll 1
+        for (int cc = 0; cc < kChunks; ++cc) {
+          const int f0 = cc * kKC + fp * NQ;
+          float zo[NQ], zn[NQ], d[NQ];
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            dr[q] = dr_n[q];
-            dv[q] = __uint_as_float(dr[q]);
+          for (int q = 0; q < NQ; ++q) {
+            zo[q] = zo_n[q];
+            zn[q] = F16 ? fmaf(__uint_as_float(dr_n[q]), dsc, zo[q])
+                        : zo[q] + __uint_as_float(dr_n[q]);
           }
-          if (cc + 1 < kTcChunks) tmem_issue4(dt + (uint32_t)(f0 + kTcKC), dr_n);
+          if (cc + 1 < kChunks) tmem_issue(dt + (uint32_t)(f0 + kKC), dr_n);
+          {                                    // the next chunk's cached fields, one chunk ahead
+            const float* src = cc + 1 < kChunks ? Zm + (size_t)(f0 + kKC) * Np + n
+                                                : Zn + (size_t)(fp * NQ) * Np + n;
 #pragma unroll
-          for (int q = 0; q < 4; ++q) zo[q] = zo_n[q];
-          if (cc + 1 < kTcChunks) {            // the next chunk's cached fields, one chunk ahead
-#pragma unroll
-            for (int q = 0; q < 4; ++q) zo_n[q] = Zm[(size_t)(f0 + kTcKC + q) * Np + n];
-          } else if (!last) {                  // the next layer's first chunk
-#pragma unroll
-            for (int q = 0; q < 4; ++q) zo_n[q] = a.Z[m + 1][(size_t)(fp * 4 + q) * Np + n];
+            for (int q = 0; q < NQ; ++q) zo_n[q] = src[(size_t)q * Np];
           }
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const float zn = zo[q] + dv[q];
-            const bool ch = live && zn != zo[q];
-            const float an = act<ACTH>(zn, a.g[m], a.act[m]);
-            const float ao = act<ACTH>(zo[q], a.g[m], a.act[m]);
-            d[q] = ch ? an - ao : 0.0f;
-            if (COMMIT && ch) Zm[(size_t)(f0 + q) * Np + n] = zn;
-            if (sk) sk[m][(size_t)(f0 + q) * Np + n] = ch ? zn : zo[q];
+          for (int q = 0; q < NQ; ++q) {
+            if (!live) zn[q] = zo[q];
+            d[q] = act_change<ACTH, F16>(zn[q], zo[q], a.g[m], a.act[m]);
+            if (COMMIT && zn[q] != zo[q]) Zm[(size_t)(f0 + q) * Np + n] = zn[q];
+            if (Sm) Sm[(size_t)(f0 + q) * Np + n] = zn[q];
           }
           bool okc = true;
           if (!last) {
-            okc = produce_chunk(aring, s_afull, s_aempty, ga, fp, s, d);
+            okc = produce_chunk<F16>(aring, s_afull, s_aempty, ga, fp, s, d);
             ++ga;
           } else {
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-#pragma unroll
-              for (int o = 0; o < kMaxC; ++o)
-                if (o < a.C) outp[o] = fmaf(Wout[(size_t)o * Kout + f0 + q], d[q], outp[o]);
+            out_add(d, f0);
           }
-          tmem_wait4(dr_n);                    // chunk cc + 1's columns (none in flight at the end)
+          tmem_wait(dr_n);                     // chunk cc + 1's columns (none in flight at the end)
           if (!okc) {
             ok = false;
             break;
           }
         }
+      }
+      if constexpr (F16) {
+#pragma unroll
+        for (int o = 0; o < kMaxC; ++o) outp[o] *= 1.0f / kDeepDScale;
       }
       if (!ok) s_fail = 1;
     }
@@ -522,20 +605,14 @@ __global__ void __launch_bounds__(kTcThreads, 1) deep_chain_tc_kernel(DeepArgs a
   }
 }
 
-// W_hi = tf32(W), W_lo = tf32(W - W_hi) for every dense layer, stored as the stage images the
-// chain kernel copies (chunk c: hi then lo, core-matrix order).
+// W_hi and W_lo of every dense layer, stored as the stage images the chain kernel copies (chunk c:
+// hi then lo, core-matrix order).
 __global__ void deep_split_kernel(DeepArgs a) {
   const int m = blockIdx.y + 1;
   if (m > a.L - 2 || a.whi[m] == nullptr) return;
   const int n = kTcW * kTcW;
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
-    const int r = e / kTcW, k = e % kTcW;
-    const float w = a.w[m][e];
-    const float h = tf32_rna(w);
-    const size_t o = deep_tc_image_index(r, k);
-    a.whi[m][o] = h;
-    a.whi[m][o + kWHalfBytes / 4] = tf32_rna(w - h);
-  }
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x)
+    deep_tc_image_store(a, m, e / kTcW, e % kTcW, a.w[m][e]);
 }
 
 }  // namespace
@@ -546,18 +623,10 @@ cudaError_t launch_deep_split(const DeepArgs& a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-// The hidden layers' common transfer function, if every layer 1 .. L-2 has the same one.
-static int hidden_act(const DeepArgs& a) {
-  for (int m = 1; m <= a.L - 2; ++m)
-    if (a.act[m] != a.act[1]) return -1;
-  return a.act[1] == MCA_ACT_TANH ? MCA_ACT_TANH : -1;
-}
-
 template <bool COMMIT>
 static cudaError_t launch_tc(const DeepArgs& a, dim3 grid, cudaStream_t s) {
-  const void* fn = hidden_act(a) == MCA_ACT_TANH
-                       ? (const void*)deep_chain_tc_kernel<COMMIT, MCA_ACT_TANH>
-                       : (const void*)deep_chain_tc_kernel<COMMIT, -1>;
+  const void* fn = a.tc_f16 ? (const void*)deep_chain_tc_kernel<COMMIT, MCA_ACT_TANH, true>
+                            : (const void*)deep_chain_tc_kernel<COMMIT, -1, false>;
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmem);
   if (e != cudaSuccess) return e;
   DeepArgs args = a;

@@ -117,6 +117,15 @@ __global__ void count_nonfinite_kernel(const float* __restrict__ p, size_t n, in
   if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(out, 1);
 }
 
+__global__ void abs_max_kernel(const float* __restrict__ p, size_t n, int* out) {
+  int m = 0;                         // the bits of non-negative floats order like the floats
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
+       i += (size_t)gridDim.x * blockDim.x)
+    m = max(m, __float_as_int(fabsf(p[i])));
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0) atomicMax(out, m);
+}
+
 __global__ void init_layer_kernel(int wkind, float scale, const float* __restrict__ src,
                                   const signed char* __restrict__ mask, size_t n, float* w_eff,
                                   signed char* code, float* wfix) {
@@ -342,6 +351,13 @@ cudaError_t launch_count_nonfinite(const float* p, size_t n, int* out, cudaStrea
   if (n == 0) return cudaSuccess;
   const int grid = (int)std::min<size_t>(4096, (n + 255) / 256);
   count_nonfinite_kernel<<<grid, 256, 0, s>>>(p, n, out);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_abs_max(const float* p, size_t n, int* out, cudaStream_t s) {
+  if (n == 0) return cudaSuccess;
+  const int grid = (int)std::min<size_t>(1024, (n + 255) / 256);
+  abs_max_kernel<<<grid, 256, 0, s>>>(p, n, out);
   return cudaGetLastError();
 }
 

@@ -141,6 +141,7 @@ constexpr int kTcTS = 128;         // samples per tile of the tensor-core chain 
 constexpr int kDeepThreads = 256;
 constexpr int kDeepMaxWidth = 256; // widths of the layers inside the dense chain
 constexpr int kDeepKC = 16;        // weight-tile depth of the chain GEMM
+constexpr float kDeepDScale = 16384.0f;   // tanh changes (at most 2) as fp16 operands: scale
 constexpr int kDeepScrSlots = 16;  // candidates whose fields the tensor-core evaluation keeps
 constexpr int kTfmScrSlots = 16;   // candidates whose residual streams the evaluation keeps
 
@@ -170,6 +171,9 @@ struct DeepArgs {
   float* whi[kMaxLayers];    // tensor-core chain: tf32(W_m) and tf32(W_m - tf32(W_m)) of the
                              //   256 x 256 layers 1 .. L-2 as stage images (null otherwise)
   int tc;                    // 1: dense chain on the tensor cores, tiles of kTcTS samples
+  int tc_f16;                // tc = 1: operands as fp16 parts (tanh layers), else tf32 parts
+  float tc_wscale;           // tc_f16: power of two that scales the dense weights to at most 2^15
+  float tc_dscale;           // tc_f16: 1 / (tc_wscale kDeepDScale), the products' scale
   const float* XT;           // [D x Np]
   float* ell;                // [Np] per-sample loss
   const int* y;
@@ -302,6 +306,8 @@ cudaError_t launch_csr_sectors(const int* off, const int* xs_n, int D, int* sect
 cudaError_t launch_csr_range_offsets(const int* off, const int* xs_n, int D, int NR, int RS,
                                      int* roff, cudaStream_t s);
 cudaError_t launch_count_nonfinite(const float* p, size_t n, int* out, cudaStream_t s);
+// *out = max(*out, bits of max |p[i]|) (finite values; *out holds the bits of a float >= 0).
+cudaError_t launch_abs_max(const float* p, size_t n, int* out, cudaStream_t s);
 cudaError_t launch_init_layer(int wkind, float scale, const float* src, const signed char* mask,
                               size_t n, float* w_eff, signed char* code, float* wfix,
                               cudaStream_t s);
@@ -389,6 +395,8 @@ struct mca_handle {
   bool deep = false;
   bool tc = false;                   // deep: dense chain on the tensor cores; Transformer: the
                                      // tensor-core sequence kernels
+  bool tc_f16 = false;               // deep: the chain's operands as fp16 parts, scaled for weights
+  float wbound = 1.0f;               //   of magnitude at most wbound
   std::vector<float*> Z;
   std::vector<float*> whi;           // split-weight images of layers 1 .. L-2 (tensor-core chain)
   float* ell = nullptr;
