@@ -191,11 +191,16 @@ __device__ __forceinline__ float act_change(float zn, float zo, float g, int act
   }
 }
 
-// ACTH: transfer function of the hidden layers (-1: read per layer at run time).
-template <bool COMMIT, int ACTH, bool F16>
+// MODE: evaluation of a candidate, its commit, or the forward pass from Z_0 on (every later field and the
+// losses; the chain's "changes" are then the activations themselves). ACTH: transfer function of the
+// hidden layers (-1: read per layer at run time).
+enum ChainMode { kChainEval = 0, kChainCommit = 1, kChainForward = 2 };
+
+template <int MODE, int ACTH, bool F16>
 __global__ void __launch_bounds__(kTcThreads, 1) deep_chain_tc_kernel(DeepArgs a) {
   constexpr int kKC = Split<F16>::kKC, NQ = Split<F16>::kNQ, kChunks = kTcW / kKC;
   constexpr uint32_t kIdesc = Split<F16>::kIdesc;
+  constexpr bool COMMIT = MODE == kChainCommit, FWD = MODE == kChainForward;
   extern __shared__ __align__(1024) unsigned char tsm[];
   unsigned char* aring = tsm;                                 // A chunks
   unsigned char* wst = tsm + kASlots * kASlot;                // W stages
@@ -209,9 +214,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) deep_chain_tc_kernel(DeepArgs a
   __shared__ volatile int s_fail;
   __shared__ int s_k;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  int k = 0, tile = COMMIT ? blockIdx.x : 0;
+  int k = 0, tile = MODE != kChainEval ? blockIdx.x : 0;
   if (COMMIT && a.ctl->kstar < 0) return;
-  if (!COMMIT) {
+  if (MODE == kChainEval) {
     // Longest chains first: CTAs start in linear block order, so the linear index is mapped to
     // (candidate rank, tile) with the candidates ranked by the depth of their dense chain (the
     // mutated layer, from the proposal alone), ties by index. Every CTA computes the same ranking.
@@ -233,13 +238,17 @@ __global__ void __launch_bounds__(kTcThreads, 1) deep_chain_tc_kernel(DeepArgs a
   }
   const int n0 = tile * kTcTS;
   if (tid == 0) {
-    s_cand = COMMIT ? a.ctl->acc : deep_candidate(a, k);
+    if (FWD) {                       // the dense chain starts at layer 1
+      s_cand = DeepCand{0u, -1, 0, 0, 0.0f, 0.0f, 1.0f, 0, 1};
+    } else {
+      s_cand = COMMIT ? a.ctl->acc : deep_candidate(a, k);
+    }
     s_fail = 0;
   }
   __syncthreads();
   const DeepCand c = s_cand;
   float* part = a.partial + (size_t)k * a.ntiles + tile;
-  if (!c.valid || c.delta == 0.0f) {
+  if (!FWD && (!c.valid || c.delta == 0.0f)) {
     if (!COMMIT && tid == 0) *part = 0.0f;
     return;
   }
@@ -247,11 +256,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) deep_chain_tc_kernel(DeepArgs a
   const int Np = a.Np, N = a.N;
   float dl = 0.0f;
   // this candidate's scratch slot, when it has one and a dense chain (layer <= L-3)
-  float* const* sk = (!COMMIT && k < a.nscr && l <= L - 3) ? a.scr + (size_t)k * (L + 1) : nullptr;
+  float* const* sk = (MODE == kChainEval && k < a.nscr && l <= L - 3) ? a.scr + (size_t)k * (L + 1) : nullptr;
   if (l + 1 < L - 1 && a.n_out[l + 1] == kTcW && tid < kCtl) prefetch_tile(a.Z[l + 1], Np, n0, tid);
 
   // ---- row j of layer l (thread s = sample)
-  if (tid < kTcTS) {
+  if (!FWD && tid < kTcTS) {
     const int n = n0 + tid;
     float da = 0.0f;
     if (n < N) {
@@ -431,19 +440,19 @@ __global__ void __launch_bounds__(kTcThreads, 1) deep_chain_tc_kernel(DeepArgs a
       const float dsc = F16 ? a.tc_dscale : 1.0f;         // the products' scale
       // layer l+1: rank-1 change through column j of W_{l+1}; its activation change is the first
       // A (dense) or feeds the output layer directly (l = L-3)
-      if (dense) prefetch_tile(a.Z[l + 2], Np, n0, tid);
+      if (dense && !FWD) prefetch_tile(a.Z[l + 2], Np, n0, tid);
       {
         const int m1 = l + 1;
         const float* W1 = a.w[m1];
         const int K1 = a.n_in[m1];
-        const float da = s_da[s];
+        const float da = FWD ? 0.0f : s_da[s];
         float* Zm = a.Z[m1];
         const bool moves = live && da != 0.0f;
         // loads one chunk ahead of their use (n < Np: always in the array)
         float wv[NQ], zo[NQ], wv_n[NQ], zo_n[NQ];
 #pragma unroll
         for (int q = 0; q < NQ; ++q) {
-          wv_n[q] = W1[(size_t)(fp * NQ + q) * K1 + j];
+          wv_n[q] = FWD ? 0.0f : W1[(size_t)(fp * NQ + q) * K1 + j];
           zo_n[q] = Zm[(size_t)(fp * NQ + q) * Np + n];
         }
 #pragma unroll 1
@@ -458,12 +467,16 @@ __global__ void __launch_bounds__(kTcThreads, 1) deep_chain_tc_kernel(DeepArgs a
           if (cc + 1 < kChunks) {
 #pragma unroll
             for (int q = 0; q < NQ; ++q) {
-              wv_n[q] = W1[(size_t)(f0 + kKC + q) * K1 + j];
+              wv_n[q] = FWD ? 0.0f : W1[(size_t)(f0 + kKC + q) * K1 + j];
               zo_n[q] = Zm[(size_t)(f0 + kKC + q) * Np + n];
             }
           }
 #pragma unroll
           for (int q = 0; q < NQ; ++q) {
+            if (FWD) {
+              d[q] = tanh_exp(zo[q]) * kDeepDScale;
+              continue;
+            }
             const float zn = moves ? fmaf(wv[q], da, zo[q]) : zo[q];
             d[q] = act_change<ACTH, F16>(zn, zo[q], a.g[m1], a.act[m1]);
             if (COMMIT && zn != zo[q]) Zm[(size_t)(f0 + q) * Np + n] = zn;
@@ -484,12 +497,13 @@ __global__ void __launch_bounds__(kTcThreads, 1) deep_chain_tc_kernel(DeepArgs a
       float zo_n[NQ];                                     // cached fields one chunk ahead
       if (dense) {
 #pragma unroll
-        for (int q = 0; q < NQ; ++q) zo_n[q] = a.Z[l + 2][(size_t)(fp * NQ + q) * Np + n];
+        for (int q = 0; q < NQ; ++q)
+          zo_n[q] = FWD ? 0.0f : a.Z[l + 2][(size_t)(fp * NQ + q) * Np + n];
       }
       for (int li = 0; li < nd && ok; ++li) {
         const int m = l + 2 + li;
         const bool last = m == L - 2;
-        if (!last) prefetch_tile(a.Z[m + 1], Np, n0, tid);
+        if (!last && !FWD) prefetch_tile(a.Z[m + 1], Np, n0, tid);
         if (!warp_wait(&s_dfull[li & 1], (uint32_t)(li >> 1) & 1u)) {
           ok = false;
           break;
@@ -511,11 +525,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) deep_chain_tc_kernel(DeepArgs a
 #pragma unroll
           for (int q = 0; q < NQ; ++q) {
             zo[q] = zo_n[q];
-            zn[q] = F16 ? fmaf(__uint_as_float(dr_n[q]), dsc, zo[q])
-                        : zo[q] + __uint_as_float(dr_n[q]);
+            zn[q] = FWD ? __uint_as_float(dr_n[q]) * dsc
+                    : F16 ? fmaf(__uint_as_float(dr_n[q]), dsc, zo[q])
+                          : zo[q] + __uint_as_float(dr_n[q]);
           }
           if (cc + 1 < kChunks) tmem_issue(dt + (uint32_t)(f0 + kKC), dr_n);
-          {                                    // the next chunk's cached fields, one chunk ahead
+          if (!FWD) {                          // the next chunk's cached fields, one chunk ahead
             const float* src = cc + 1 < kChunks ? Zm + (size_t)(f0 + kKC) * Np + n
                                                 : Zn + (size_t)(fp * NQ) * Np + n;
 #pragma unroll
@@ -523,6 +538,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) deep_chain_tc_kernel(DeepArgs a
           }
 #pragma unroll
           for (int q = 0; q < NQ; ++q) {
+            if (FWD) {
+              d[q] = tanh_exp(zn[q]) * kDeepDScale;
+              Zm[(size_t)(f0 + q) * Np + n] = zn[q];
+              continue;
+            }
             if (!live) zn[q] = zo[q];
             d[q] = act_change<ACTH, F16>(zn[q], zo[q], a.g[m], a.act[m]);
             if (COMMIT && zn[q] != zo[q]) Zm[(size_t)(f0 + q) * Np + n] = zn[q];
@@ -565,7 +585,16 @@ __global__ void __launch_bounds__(kTcThreads, 1) deep_chain_tc_kernel(DeepArgs a
         for (int o = 0; o < kMaxC; ++o) outp[o] += xo[((p - 1) * kMaxC + o) * kTcTS + s];
     }
     const bool failed = s_fail != 0;                  // the same value in every thread here
-    if (worker && fp == 0 && live && !failed) {
+    if (FWD) {
+      if (worker && fp == 0 && !failed) {
+        const int Lo = L - 1;
+#pragma unroll
+        for (int o = 0; o < kMaxC; ++o)
+          if (o < a.C) a.Z[Lo][(size_t)o * Np + n] = outp[o];
+        if (live)
+          a.ell[n] = sample_loss<-1, -1, kMaxC>(outp, a.C, a.y[n], a.g[Lo], a.act[Lo], a.loss);
+      }
+    } else if (worker && fp == 0 && live && !failed) {
       float zz[kMaxC];
       bool changed = false;
 #pragma unroll
@@ -599,7 +628,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) deep_chain_tc_kernel(DeepArgs a
       if (tid == 0 && failed) atomicCAS(&a.st->err, 0, (int)MCA_ERR_TIMEOUT);
     }
   }
-  if (!COMMIT) {
+  if (MODE == kChainEval) {
     const float tot = block_sum(dl, s_red);
     if (tid == 0) *part = tot;
   }
@@ -623,10 +652,10 @@ cudaError_t launch_deep_split(const DeepArgs& a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-template <bool COMMIT>
+template <int MODE>
 static cudaError_t launch_tc(const DeepArgs& a, dim3 grid, cudaStream_t s) {
-  const void* fn = a.tc_f16 ? (const void*)deep_chain_tc_kernel<COMMIT, MCA_ACT_TANH, true>
-                            : (const void*)deep_chain_tc_kernel<COMMIT, -1, false>;
+  const void* fn = a.tc_f16 ? (const void*)deep_chain_tc_kernel<MODE, MCA_ACT_TANH, true>
+                            : (const void*)deep_chain_tc_kernel<MODE, -1, false>;
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmem);
   if (e != cudaSuccess) return e;
   DeepArgs args = a;
@@ -636,11 +665,21 @@ static cudaError_t launch_tc(const DeepArgs& a, dim3 grid, cudaStream_t s) {
 
 cudaError_t launch_deep_eval_tc(const DeepArgs& a, cudaStream_t s) {
   const int Kb = a.n_explicit > 0 ? a.n_explicit : a.Kb;
-  return launch_tc<false>(a, dim3(Kb, a.ntiles), s);
+  return launch_tc<kChainEval>(a, dim3(Kb, a.ntiles), s);
 }
 
 cudaError_t launch_deep_commit_tc(const DeepArgs& a, cudaStream_t s) {
-  return launch_tc<true>(a, dim3(a.ntiles), s);
+  return launch_tc<kChainCommit>(a, dim3(a.ntiles), s);
+}
+
+cudaError_t launch_deep_forward_tc(const DeepArgs& a, cudaStream_t s) {
+  if (!a.tc_f16) return cudaErrorInvalidValue;
+  const void* fn = (const void*)deep_chain_tc_kernel<kChainForward, MCA_ACT_TANH, true>;
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmem);
+  if (e != cudaSuccess) return e;
+  DeepArgs args = a;
+  void* params[] = {&args};
+  return cudaLaunchKernel(fn, dim3(a.ntiles), dim3(kTcThreads), params, kTcSmem, s);
 }
 
 }  // namespace mca

@@ -214,6 +214,7 @@ cudaError_t launch_deep_losses(const DeepArgs& a, cudaStream_t s);
 cudaError_t launch_deep_split(const DeepArgs& a, cudaStream_t s);     // W_hi / W_lo of all layers
 cudaError_t launch_deep_eval_tc(const DeepArgs& a, cudaStream_t s);   // grid (Kb, ntiles)
 cudaError_t launch_deep_commit_tc(const DeepArgs& a, cudaStream_t s); // grid ntiles
+cudaError_t launch_deep_forward_tc(const DeepArgs& a, cudaStream_t s);  // grid ntiles
 
 // ------------------------------------------------------------------------------------------------
 // Character-level Transformer path: pre-LN GPT blocks over B sequences of T tokens. All parameters
