@@ -498,7 +498,8 @@ mca_status resync(mca_handle* h) {
     const mca::TfmArgs a = tfm_args(h);
     if (a.tc) {
       CUDA_TRY(h, mca::launch_tfm_tc_split(a, h->stream));
-      h->launches += 1;
+      CUDA_TRY(h, mca::launch_tfm_f16_split(a, h->stream));
+      h->launches += 2;
     }
     CUDA_TRY(h, mca::launch_tfm_forward(a, h->stream));
     CUDA_TRY(h, mca::launch_sum_loss(h->ell, a.B, h->st, h->stream));
@@ -574,13 +575,16 @@ mca_status load_params(mca_handle* h, const float* params, const signed char* co
   }
   const float* src = pdev ? params : tmp;
   const signed char* csrc = codes ? (cdev ? codes : ctmp) : nullptr;
-  int* dflag = nullptr;              // [0] a non-finite value; [1] the dense weights' largest magnitude
+  // [0] a non-finite value; [1] the largest magnitude of a deep net's dense weights, or of the
+  // Transformer's parameters
+  int* dflag = nullptr;
   cudaError_t e = cudaMalloc(&dflag, 2 * sizeof(int));
   if (e == cudaSuccess) e = cudaMemsetAsync(dflag, 0, 2 * sizeof(int), h->stream);
   if (e == cudaSuccess) e = mca::launch_count_nonfinite(src, P, dflag, h->stream);
   if (e == cudaSuccess && h->tc_f16)
     e = mca::launch_abs_max(src + h->off[1], h->off[h->layers.size() - 1] - h->off[1], dflag + 1,
                             h->stream);
+  if (e == cudaSuccess && h->tfm && h->tc) e = mca::launch_abs_max(src, P, dflag + 1, h->stream);
   for (size_t l = 0; e == cudaSuccess && l < h->layers.size(); ++l) {
     const mca_layer& L = h->layers[l];
     const size_t n = (size_t)L.n_in * L.n_out;
@@ -597,9 +601,10 @@ mca_status load_params(mca_handle* h, const float* params, const signed char* co
   if (ctmp) cudaFree(ctmp);
   CUDA_TRY(h, e);
   if (hflag[0]) return fail(h, MCA_ERR_NUMERIC, "non-finite parameter value");
+  float top = 0.0f;
+  std::memcpy(&top, &hflag[1], sizeof(top));
+  h->pmax = top;
   if (h->tc_f16) {
-    float top = 0.0f;
-    std::memcpy(&top, &hflag[1], sizeof(top));
     float sc = 1.0f;                 // ternary layers hold codes
     for (const mca_layer& L : h->layers)
       if (L.wkind == MCA_W_TERNARY_I8) sc = std::max(sc, std::fabs(L.scale));
@@ -690,7 +695,7 @@ mca_status tfm_check(const mca_tfm_spec* t, int64_t n_seq) {
 
 struct TfmMem {
   size_t params, tokens, X, ell, partial, st, ctl, trace, ex_idx, ex_new, ex_out, prop, scratch,
-      wimg, Xmid, scrX, scr_ell, ctl2, tau_dev, total;
+      wimg, wimg16, Xmid, scrX, scr_ell, ctl2, tau_dev, total;
   int nscr;
 };
 
@@ -736,6 +741,7 @@ TfmMem tfm_plan(const mca_tfm_spec& t, long long B, int trace_cap, bool tc, int 
   M.prop = take(sizeof(mca_trace_rec) * mca::kKmax);
   M.scratch = take(sizeof(int) * 8);
   M.wimg = tc ? take(sizeof(float) * mca::tfm_tc_image_floats(t.d_ff, t.n_layer)) : 0;
+  M.wimg16 = tc ? take(mca::tfm_f16_image_bytes(t.d_ff, t.n_layer)) : 0;
   M.Xmid = take(tc ? sizeof(float) * (size_t)t.n_layer * B * t.ctx * t.d_model : 0);
   M.nscr = tfm_scratch_slots(t, B, K, tc);
   M.scrX = take(sizeof(float) * (size_t)M.nscr * (2 * t.n_layer + 1) * B * t.ctx * t.d_model);
@@ -744,6 +750,16 @@ TfmMem tfm_plan(const mca_tfm_spec& t, long long B, int trace_cap, bool tc, int 
   M.tau_dev = take(sizeof(unsigned long long));
   M.total = o;
   return M;
+}
+
+// The Transformer's parameters, and those of any trial drawn now, are within the range of the fp16
+// operands. Perturbations: the decision of the batch in flight may move a parameter by delta before
+// a trial moves it by delta again.
+bool tfm_f16_range(const mca_handle* h) {
+  const bool move = h->dom.op == MCA_OP_PERTURB;
+  const float step = move ? 2.0f * std::fabs(h->dom.delta) : 0.0f;
+  const float drawn = move ? 0.0f : std::max(std::fabs(h->dom.lo), std::fabs(h->dom.hi));
+  return h->pmax + step <= mca::kTfmF16Max && drawn <= mca::kTfmF16Max;
 }
 
 mca::TfmArgs tfm_args(mca_handle* h) {
@@ -800,6 +816,8 @@ mca::TfmArgs tfm_args(mca_handle* h) {
   a.nforce = h->nforce;
   a.tc = h->tc ? 1 : 0;
   a.wimg = h->tfm_img;
+  a.wimg16 = h->tfm_img16;
+  a.f16 = h->tc && tfm_f16_range(h) ? 1 : 0;
   return a;
 }
 
@@ -830,6 +848,7 @@ mca_status run_tfm_pipelined(mca_handle* h, mca::TfmArgs ta, uint64_t n_trials) 
                                   : mca::batch_width_cost(h->rate_acc, h->rate_trials,
                                                           mca::kBatchCostTfm, h->opt.K);
     ta.Kb = (int)std::min<uint64_t>(n_trials, (uint64_t)Kw);
+    ta.f16 = tfm_f16_range(h) ? 1 : 0;
     ta.ctl = h->ctl2 + p;
     CUDA_TRY(h, cudaEventRecord(h->ev_p[p][0], h->stream));
     CUDA_TRY(h, mca::launch_tfm_eval(ta, h->stream));
@@ -863,6 +882,7 @@ mca_status run_tfm_pipelined(mca_handle* h, mca::TfmArgs ta, uint64_t n_trials) 
       h->broken = true;
       return fail(h, MCA_ERR_NUMERIC, "non-finite loss change");
     }
+    if (ctl.kstar >= 0) h->pmax = std::max(h->pmax, std::fabs(ctl.acc.neww));
     done += (uint64_t)ctl.consumed;
     h->rate_acc = h->rate_acc * mca::kRateDecay + (ctl.kstar >= 0 ? 1.0f : 0.0f);
     h->rate_trials = h->rate_trials * mca::kRateDecay + (float)ctl.consumed;
@@ -1251,6 +1271,10 @@ mca_status mca_run(mca_handle* h, uint64_t n_trials, uint64_t seed, mca_run_stat
         CUDA_TRY(h, mca::launch_deep_split(a, h->stream));
         h->launches += 1;
       }
+      if (h->tfm && ctl.kstar >= 0) {
+        h->pmax = std::max(h->pmax, std::fabs(ctl.acc.neww));
+        ta.f16 = h->tc && tfm_f16_range(h) ? 1 : 0;
+      }
       h->tau += (uint64_t)ctl.consumed;
       remaining -= (uint64_t)ctl.consumed;
       h->rate_acc = h->rate_acc * mca::kRateDecay + (ctl.kstar >= 0 ? 1.0f : 0.0f);
@@ -1419,10 +1443,12 @@ mca_status mca_force_decisions(mca_handle* h, const uint64_t* tau, const uint8_t
 namespace {
 
 // Loss changes of the n candidates in h->ex_idx / h->ex_new against the current state, no commit,
-// into dS (host). The evaluation kernels of mca_run's evaluation step.
-mca_status eval_explicit(mca_handle* h, size_t n, double* dS) {
+// into dS (host); wmax: the candidates' largest magnitude. The evaluation kernels of mca_run's
+// evaluation step.
+mca_status eval_explicit(mca_handle* h, size_t n, float wmax, double* dS) {
   if (h->tfm) {
     mca::TfmArgs a = tfm_args(h);
+    if (wmax > mca::kTfmF16Max) a.f16 = 0;
     a.n_explicit = (int)n;
     a.ex_idx = h->ex_idx;
     a.ex_new = h->ex_new;
@@ -1478,7 +1504,9 @@ mca_status mca_eval_candidates(mca_handle* h, const uint32_t* flat_idx, const fl
                               h->stream));
   CUDA_TRY(h, cudaMemcpyAsync(h->ex_new, new_w, sizeof(float) * n, cudaMemcpyHostToDevice,
                               h->stream));
-  return eval_explicit(h, n, dS);
+  float wmax = 0.0f;
+  for (size_t m = 0; m < n; ++m) wmax = std::max(wmax, std::fabs(new_w[m]));
+  return eval_explicit(h, n, wmax, dS);
 }
 
 mca_status mca_eval_trials(mca_handle* h, uint64_t seed, uint64_t tau, size_t n,
@@ -1517,7 +1545,7 @@ mca_status mca_eval_trials(mca_handle* h, uint64_t seed, uint64_t tau, size_t n,
   CUDA_TRY(h, cudaMemcpyAsync(out, h->prop, sizeof(mca_trace_rec) * n, cudaMemcpyDeviceToHost,
                               h->stream));
   double dS[mca::kKmax];
-  mca_status rc = eval_explicit(h, n, dS);
+  mca_status rc = eval_explicit(h, n, 0.0f, dS);   // proposals are within tfm_f16_range's bound
   if (rc != MCA_OK) return rc;
   double S = 0.0;
   rc = mca_loss(h, &S);
@@ -1647,6 +1675,7 @@ mca_status mca_create_transformer(const mca_tfm_spec* spec, const mca_domain* do
   h->ex_out = reinterpret_cast<double*>(base + M.ex_out);
   h->prop = reinterpret_cast<mca_trace_rec*>(base + M.prop);
   h->tfm_img = h->tc ? reinterpret_cast<float*>(base + M.wimg) : nullptr;
+  h->tfm_img16 = h->tc ? base + M.wimg16 : nullptr;
   h->tfm_Xmid = h->tc ? reinterpret_cast<float*>(base + M.Xmid) : nullptr;
   h->ctl2 = reinterpret_cast<mca::DeepCtl*>(base + M.ctl2);
   h->tau_dev = reinterpret_cast<unsigned long long*>(base + M.tau_dev);

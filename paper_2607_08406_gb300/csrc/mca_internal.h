@@ -143,6 +143,7 @@ constexpr int kDeepMaxWidth = 256; // widths of the layers inside the dense chai
 constexpr int kDeepKC = 16;        // weight-tile depth of the chain GEMM
 constexpr float kDeepDScale = 16384.0f;   // tanh changes (at most 2) as fp16 operands: scale
 constexpr int kDeepScrSlots = 16;  // candidates whose fields the tensor-core evaluation keeps
+constexpr float kTfmF16Max = 4.0f;   // largest parameter magnitude of the fp16 Transformer kernels
 constexpr int kTfmScrSlots = 16;   // candidates whose residual streams the evaluation keeps
 
 struct DeepCand {
@@ -271,6 +272,9 @@ struct TfmArgs {
   double* ex_out;
   int tc;                    // 1: the tensor-core kernels (mca_tfm_tc.cu) run the sequences
   float* wimg;               // their split-weight images (mca_tc_layout.h), tc = 1 only
+  void* wimg16;              // the images with fp16 parts, kept beside them
+  int f16;                   // tc = 1: run the kernels with fp16 parts (every parameter, and every
+                             //   candidate's, at most kTfmF16Max in magnitude)
   // scratch slots (tc = 1, trial loop only): candidate k < nscr of a batch writes the residual
   // streams it recomputes to slot k of scrX ([nscr][(2 nL + 1) x B x T x d]: X, then Xmid) and its
   // sequence losses to scr_ell ([nscr][B]); an accepted candidate with a slot is adopted from it
@@ -292,6 +296,8 @@ cudaError_t launch_tfm_forward(const TfmArgs& a, cudaStream_t s);   // grid B, w
 // Tensor-core Transformer kernels (two sequences per CTA): the split-weight images from the
 // parameters, the three sequence modes, and the image entry of the accepted parameter after a commit.
 cudaError_t launch_tfm_tc_split(const TfmArgs& a, cudaStream_t s);
+cudaError_t launch_tfm_f16_split(const TfmArgs& a, cudaStream_t s);
+cudaError_t launch_tfm_f16(const TfmArgs& a, int mode, cudaStream_t s);   // the three modes, fp16 parts
 cudaError_t launch_tfm_tc_eval(const TfmArgs& a, cudaStream_t s);      // grid (Kb, B / 2)
 cudaError_t launch_tfm_tc_commit(const TfmArgs& a, cudaStream_t s);    // grid B / 2
 cudaError_t launch_tfm_tc_forward(const TfmArgs& a, cudaStream_t s);   // grid B / 2
@@ -447,6 +453,8 @@ struct mca_handle {
   int* tokens = nullptr;                 // [B x (ctx + 1)]
   float* X = nullptr;                    // cached residual stream at every stage
   float* tfm_img = nullptr;
+  void* tfm_img16 = nullptr;             // the same with fp16 operand parts
+  float pmax = 0.0f;                     // tensor-core Transformer: largest parameter magnitude
   float* tfm_Xmid = nullptr;             // its mid streams (after each block's attention)
   float* tfm_scrX = nullptr;             // Transformer tensor-core path: candidate scratch slots
   float* tfm_scr_ell = nullptr;          // (h->nscr of them)              // split-weight images of the tensor-core kernels (tc)

@@ -70,6 +70,14 @@ __device__ __forceinline__ void mma_ts(uint32_t d, uint32_t a, uint64_t b, uint3
                ::"r"(d), "r"(a), "l"(b), "r"(idesc), "r"(acc));
 }
 
+// The same with fp16 operands (A: two values per column).
+__device__ __forceinline__ void mma_ts_f16(uint32_t d, uint32_t a, uint64_t b, uint32_t idesc,
+                                           uint32_t acc) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+               "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n"
+               ::"r"(d), "r"(a), "l"(b), "r"(idesc), "r"(acc));
+}
+
 // Arrive on mbar once every MMA this thread issued before has completed.
 __device__ __forceinline__ void umma_commit(uint64_t* mbar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"

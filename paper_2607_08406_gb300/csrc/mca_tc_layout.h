@@ -59,6 +59,36 @@ MCA_HD size_t tfm_tc_image_offset(int mat, int b, int r, int k, int F, int nL) {
   return base + 131072 + (size_t)256 * F + tc_image_index(r, k, 128, F);
 }
 
+// Images with fp16 parts (two per weight as well, of a scaled weight): 16 KB chunks in the order in which
+// the fp16 kernels consume them. Per block: Wq, Wk, Wv, Wo, four chunks of 32 columns each; then, per
+// half h of 64 hidden units of the n = F / 64, W1's 64 rows as two chunks of 64 columns and W2's 64
+// columns as two chunks of 32, ordered W1(0), W1(1), and W2(h), W1(h + 2) for h = 0, 1, ... After the last
+// block the head, four chunks. Within a chunk the high parts (8 columns of all its rows after another,
+// 16 bytes a row), then the low parts.
+constexpr size_t kTfmF16Chunk = 16384;       // bytes
+MCA_HD int tfm_f16_block_chunks(int F) { return 16 + 4 * (F / kTcTfmHc); }
+MCA_HD size_t tfm_f16_image_bytes(int F, int nL) {
+  return ((size_t)nL * (size_t)tfm_f16_block_chunks(F) + 4) * kTfmF16Chunk;
+}
+MCA_HD int tfm_f16_w1_chunk(int h) { return 16 + (h < 2 ? 2 * h : 4 * h - 2); }
+MCA_HD int tfm_f16_w2_chunk(int h, int n) { return 16 + (h < n - 1 ? 4 + 4 * h : 4 * n - 2); }
+
+// Offset, in fp16 elements, of the high part of element (r, k) of matrix `mat` of block b; its low
+// part is kTfmF16Chunk / 4 elements further on.
+MCA_HD size_t tfm_f16_image_offset(int mat, int b, int r, int k, int F, int nL) {
+  const size_t chunk = kTfmF16Chunk / 2;
+  const int cpb = tfm_f16_block_chunks(F);
+  const int wide = ((k >> 3) & 3) * 1024 + r * 8 + (k & 7);      // 128 rows x 32 columns
+  if (mat == kTcHead) return ((size_t)nL * cpb + (size_t)(k >> 5)) * chunk + (size_t)wide;
+  const size_t blk = (size_t)b * cpb;
+  if (mat <= kTcO) return (blk + (size_t)(4 * mat + (k >> 5))) * chunk + (size_t)wide;
+  if (mat == kTcW1)
+    return (blk + (size_t)(tfm_f16_w1_chunk(r >> 6) + (k >> 6))) * chunk +
+           (size_t)(((k >> 3) & 7) * 512 + (r & 63) * 8 + (k & 7));
+  return (blk + (size_t)(tfm_f16_w2_chunk(k >> 6, F / kTcTfmHc) + ((k >> 5) & 1))) * chunk +
+         (size_t)wide;
+}
+
 // Shapes the tensor-core Transformer kernels handle: T = 64, d = 128, 4 heads of 32, d_ff a
 // multiple of 128 up to 1024, vocab <= 128, an even number of sequences (two per CTA).
 MCA_HD bool tfm_tc_shape_ok(int T, int d, int H, int F, int V, long long B) {

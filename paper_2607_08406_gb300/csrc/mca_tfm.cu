@@ -565,18 +565,18 @@ static cudaError_t launch_seq(const TfmArgs& a, dim3 grid, cudaStream_t s) {
 }
 
 cudaError_t launch_tfm_eval(const TfmArgs& a, cudaStream_t s) {
-  if (a.tc) return launch_tfm_tc_eval(a, s);
+  if (a.tc) return a.f16 ? launch_tfm_f16(a, kTfmEval, s) : launch_tfm_tc_eval(a, s);
   const int Kb = a.n_explicit > 0 ? a.n_explicit : a.Kb;
   return launch_seq<kTfmEval>(a, dim3(Kb, a.B), s);
 }
 
 cudaError_t launch_tfm_commit(const TfmArgs& a, cudaStream_t s) {
-  if (a.tc) return launch_tfm_tc_commit(a, s);
+  if (a.tc) return a.f16 ? launch_tfm_f16(a, kTfmCommit, s) : launch_tfm_tc_commit(a, s);
   return launch_seq<kTfmCommit>(a, dim3(a.B), s);
 }
 
 cudaError_t launch_tfm_forward(const TfmArgs& a, cudaStream_t s) {
-  if (a.tc) return launch_tfm_tc_forward(a, s);
+  if (a.tc) return a.f16 ? launch_tfm_f16(a, kTfmForward, s) : launch_tfm_tc_forward(a, s);
   return launch_seq<kTfmForward>(a, dim3(a.B), s);
 }
 

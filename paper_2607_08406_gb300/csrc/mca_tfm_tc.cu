@@ -35,23 +35,12 @@
 // the evaluation of candidate k < nscr also writes what the commit would write into scratch slot
 // k, and an accepted candidate with a slot is adopted by copying it (the commit kernel returns;
 // the copy kernel also refreshes the image entry).
-#include <cstdio>
-
-#include "mca_device.cuh"
-#include "mca_internal.h"
-#include "mca_tc.cuh"
-#include "mca_tc_layout.h"
-#include "mca_tfm.cuh"
+#include "mca_tfm_tc.cuh"
 
 namespace mca {
 namespace {
 
-constexpr int kThreads = 512;
-constexpr int kRows = 128;                       // token rows per CTA: two sequences
-constexpr int kD = kTcTfmD;
-constexpr int kT = kTcTfmT;
-constexpr int kHc = kTcTfmHc;
-constexpr int kXLd = kD + 4;                     // residual row stride: conflict-free row access
+constexpr int kThreads = kTfmWorkers;
 constexpr int kStages = 5;
 constexpr int kStageBytes = 16384;               // one chunk of 128 rows (64-row chunks use half)
 constexpr int kXsBytes = kRows * kXLd * 4;       // 67,584
@@ -73,83 +62,13 @@ static_assert(kSmem + 8 * 1024 <= 227 * 1024, "shared memory of the Transformer 
 // K and V (2 x 64 KB) overlay the lo part of A and the first four stages
 static_assert(2 * kRows * kD * 4 <= kAloBytes + 4 * kStageBytes, "K and V overlay");
 
-__device__ __forceinline__ float prm(const TfmArgs& a, unsigned long long i,
-                                     unsigned long long midx, float mval) {
-  return i == midx ? mval : a.params[i];
-}
-
-// The weight matrix entry a parameter is (kTcMatNone for biases, LN parameters, embeddings).
-struct Target {
-  int mat, row, col;
-};
-
-__device__ __forceinline__ Target tc_target(const TfmArgs& a, unsigned long long idx, int stage) {
-  Target t;
-  t.mat = kTcMatNone;
-  t.row = 0;
-  t.col = 0;
-  if (stage >= 0 && stage < a.nL) {
-    const unsigned long long off = idx - a.o_blk0 - (unsigned long long)stage * a.blk_size;
-    const unsigned long long dd = (unsigned long long)a.d * a.d, fd = (unsigned long long)a.F * a.d;
-    const unsigned int rq[4] = {a.r_wq, a.r_wk, a.r_wv, a.r_wo};
-#pragma unroll
-    for (int m = 0; m < 4; ++m)
-      if (off >= rq[m] && off < rq[m] + dd) {
-        t.mat = m;
-        t.row = (int)((off - rq[m]) / a.d);
-        t.col = (int)((off - rq[m]) % a.d);
-      }
-    if (off >= a.r_w1 && off < a.r_w1 + fd) {
-      t.mat = kTcW1;
-      t.row = (int)((off - a.r_w1) / a.d);
-      t.col = (int)((off - a.r_w1) % a.d);
-    }
-    if (off >= a.r_w2 && off < a.r_w2 + fd) {
-      t.mat = kTcW2;
-      t.row = (int)((off - a.r_w2) / a.F);
-      t.col = (int)((off - a.r_w2) % a.F);
-    }
-  } else if (stage == a.nL && idx >= a.o_wh && idx < a.o_wh + (unsigned long long)a.V * a.d) {
-    t.mat = kTcHead;
-    t.row = (int)((idx - a.o_wh) / a.d);
-    t.col = (int)((idx - a.o_wh) % a.d);
-  }
-  return t;
-}
-
-// Where candidate k's recomputation starts, from its proposal alone, as a key that orders the
-// recomputations by length: 4 stage, plus 2 for a block's feed-forward sub-block, plus 3 for one of
-// its hidden units (then block stage + 1, key 4 stage + 4, follows a short rank-1 step).
-__device__ __forceinline__ int candidate_stage(const TfmArgs& a, int k) {
-  unsigned int idx;
-  if (a.n_explicit > 0) {
-    idx = a.ex_idx[k];
-  } else {
-    const uint4 w = trial_words(a.seed, tfm_batch_tau(a) + (unsigned long long)k);
-    idx = (unsigned int)(((unsigned long long)w.x * a.P) >> 32);
-  }
-  const int st = tfm_stage(a, idx);
-  const int rs = tfm_restart(a, idx, st);
-  return 4 * st + (rs == kRestartFfn ? 2 : rs == kRestartUnit ? 3 : 0);
-}
-
-struct Ctx {
-  float* xs;                 // residual stream [128][kXLd]
+struct Ctx : RowCtx {
   unsigned char* alo;        // lo part of A, core-matrix order (element (r, k) at (k/4) kALBO + 16 r)
   unsigned char* wst;        // weight stages
-  float* ks;                 // K [128][128], 16-byte slots of a row swizzled by (row mod 8)
-  float* vs;                 // V, same
-  uint32_t tmem;             // tensor-memory base address
-  uint32_t trow;             // this warp's lane quarter in a tensor-memory address
-  int r, g, sl, t;           // token row, column part, sequence of the pair, position
   int b0s, nb, cpb, total;   // first block run, blocks run, chunks per block, chunks in all
   int q0, nbc;               // the first block's first chunk (its FFN's when ffn0), block chunks run
   bool ffn0;                 // the first block starts at its feed-forward sub-block
   bool unit0;                // a hidden unit of block cstage: rank-1 step, then block cstage + 1
-  unsigned long long midx;   // patched parameter (~0: none)
-  float mval, dlt;           // its value, and the change of a weight-matrix entry
-  int cstage;                // the stage the candidate feeds (-1 embeddings)
-  Target tg;
 };
 
 // State of the weight ring, in shared memory: nload belongs to the loading thread, nwait and
@@ -297,14 +216,6 @@ __device__ __forceinline__ void ld32(const Ctx& c, uint32_t col, float (&v)[32])
   }
 }
 
-// v[i] += val for the one i == at (none if at is outside the array).
-template <int N>
-__device__ __forceinline__ void add_at(float (&v)[N], int at, float val) {
-#pragma unroll
-  for (int i = 0; i < N; ++i)
-    if (i == at) v[i] += val;
-}
-
 // The A operand of row r, columns k0 .. k0 + 16 h - 1 (h = 1 or 2 halves): tf32 hi part into
 // tensor-memory columns col .., lo part into the shared-memory operand lo_base.
 template <int N>
@@ -383,164 +294,6 @@ __device__ void ln_to_a(const TfmArgs& a, const Ctx& c, unsigned long long og,
   for (int i = 0; i < 32; ++i)
     if (32 * c.g + i == stash) s_acol[c.r] = x[i];
   store_a<32>(c, x, kColA + 32u * (uint32_t)c.g, c.alo, 32 * c.g);
-}
-
-// A candidate in W1, b1, W2 or b2 of block b changes one hidden unit j of the block's feed-forward
-// network, so the block's output stream (cached) moves by a rank-1 term: by W2[:, j] (f(u'_j) -
-// f(u_j)) for W1[j][k] and b1[j], by delta f(u_j) on column i for W2[i][j], by delta on column i
-// for b2[i], with u_j = LN2(mid stream) . W1[j, :] + b1[j] recomputed here on the CUDA cores (the
-// candidate's own entry at its old value: in a commit the parameter already holds the new one).
-// The new output stream of this thread's row part goes to xr.
-__device__ void ffn_unit(const TfmArgs& a, const Ctx& c, const DeepCand& cd, int s0, float* xr,
-                         float* s_part, float* s_acol) {
-  const int b = cd.layer;
-  const unsigned long long base = a.o_blk0 + (unsigned long long)b * a.blk_size;
-  const unsigned long long off = (unsigned long long)cd.idx - base;
-  const size_t seq_floats = (size_t)kT * kD;
-  int kind, j = 0, i0 = -1, kcol = -1;       // kind: 0 W1[j][kcol], 1 b1[j], 2 W2[i0][j], 3 b2[i0]
-  if (off < a.r_b1) {
-    kind = 0;
-    j = (int)((off - a.r_w1) / kD);
-    kcol = (int)((off - a.r_w1) % kD);
-  } else if (off < a.r_w2) {
-    kind = 1;
-    j = (int)(off - a.r_b1);
-  } else if (off < a.r_b2) {
-    kind = 2;
-    i0 = (int)((off - a.r_w2) / (unsigned long long)a.F);
-    j = (int)((off - a.r_w2) % (unsigned long long)a.F);
-  } else {
-    kind = 3;
-    i0 = (int)(off - a.r_b2);
-  }
-  const size_t row = ((size_t)(s0 + c.sl)) * seq_floats + (size_t)c.t * kD + 32 * c.g;
-  float xn[32];
-  const float* xo = a.X + (size_t)(b + 1) * a.B * seq_floats + row;
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const float4 v = reinterpret_cast<const float4*>(xo)[i];
-    xn[4 * i] = v.x;
-    xn[4 * i + 1] = v.y;
-    xn[4 * i + 2] = v.z;
-    xn[4 * i + 3] = v.w;
-  }
-  if (kind == 3) {
-    add_at(xn, i0 - 32 * c.g, cd.delta);
-  } else {
-    float x[32];
-    const float* xm = a.Xmid + (size_t)b * a.B * seq_floats + row;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const float4 v = reinterpret_cast<const float4*>(xm)[i];
-      x[4 * i] = v.x;
-      x[4 * i + 1] = v.y;
-      x[4 * i + 2] = v.z;
-      x[4 * i + 3] = v.w;
-    }
-    float sm = 0.0f;
-#pragma unroll
-    for (int i = 0; i < 32; ++i) sm += x[i];
-    s_part[c.g * kRows + c.r] = sm;
-    __syncthreads();
-    const float mean = (((s_part[c.r] + s_part[kRows + c.r]) + s_part[2 * kRows + c.r]) +
-                        s_part[3 * kRows + c.r]) / (float)kD;
-    float v = 0.0f;
-#pragma unroll
-    for (int i = 0; i < 32; ++i) {
-      const float e = x[i] - mean;
-      v = fmaf(e, e, v);
-    }
-    s_part[(4 + c.g) * kRows + c.r] = v;
-    __syncthreads();
-    const float var = (((s_part[4 * kRows + c.r] + s_part[5 * kRows + c.r]) +
-                        s_part[6 * kRows + c.r]) + s_part[7 * kRows + c.r]) / (float)kD;
-    const float rstd = rsqrtf(var + a.eps);
-    const unsigned long long w1 = base + a.r_w1 + (unsigned long long)j * kD;
-    float p = 0.0f;
-#pragma unroll
-    for (int i = 0; i < 32; ++i) {
-      const int col = 32 * c.g + i;
-      const float ln = (x[i] - mean) * rstd * a.params[base + a.r_ln2g + col] +
-                       a.params[base + a.r_ln2b + col];
-      if (col == kcol) s_acol[c.r] = ln;
-      const float w = w1 + col == cd.idx ? cd.oldw : a.params[w1 + col];
-      p = fmaf(ln, w, p);
-    }
-    s_part[c.g * kRows + c.r] = p;           // every thread has read the means (barrier above)
-    __syncthreads();
-    const float bj = kind == 1 ? cd.oldw : a.params[base + a.r_b1 + j];
-    const float u = ((((s_part[c.r] + s_part[kRows + c.r]) + s_part[2 * kRows + c.r]) +
-                      s_part[3 * kRows + c.r])) + bj;
-    if (kind == 2) {
-      add_at(xn, i0 - 32 * c.g, cd.delta * act_rt(a.act, u, a.g));
-    } else {
-      const float un = kind == 0 ? fmaf(cd.delta, s_acol[c.r], u) : u + cd.delta;
-      const float da = act_rt(a.act, un, a.g) - act_rt(a.act, u, a.g);
-      const unsigned long long w2 = base + a.r_w2 + (unsigned long long)j;
-#pragma unroll
-      for (int i = 0; i < 32; ++i)
-        xn[i] = fmaf(a.params[w2 + (unsigned long long)(32 * c.g + i) * a.F], da, xn[i]);
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < 8; ++i)
-    *reinterpret_cast<float4*>(xr + 4 * i) =
-        make_float4(xn[4 * i], xn[4 * i + 1], xn[4 * i + 2], xn[4 * i + 3]);
-}
-
-// Causal attention of query row r with head g over the keys of its sequence (K and V in shared
-// memory), with a running maximum and sum over blocks of 8 keys.
-__device__ __forceinline__ void attention(const Ctx& c, const float (&q)[32], float (&o)[32]) {
-  const float scale = rsqrtf(32.0f);
-  const float* kb = c.ks + (size_t)(c.sl * kT) * kD + 32 * c.g;
-  const float* vb = c.vs + (size_t)(c.sl * kT) * kD + 32 * c.g;
-  float m = -INFINITY, l = 0.0f;
-#pragma unroll
-  for (int i = 0; i < 32; ++i) o[i] = 0.0f;
-  const int jend = (c.t | 31) + 1;               // the same for every lane of the warp
-  for (int j0 = 0; j0 < jend; j0 += 8) {
-    float sc[8];
-#pragma unroll
-    for (int jj = 0; jj < 8; ++jj) {
-      const float* kr = kb + (size_t)(j0 + jj) * kD;
-      float s = 0.0f;
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const float4 kv = *reinterpret_cast<const float4*>(kr + 4 * (i ^ jj));
-        s = fmaf(q[4 * i], kv.x, s);
-        s = fmaf(q[4 * i + 1], kv.y, s);
-        s = fmaf(q[4 * i + 2], kv.z, s);
-        s = fmaf(q[4 * i + 3], kv.w, s);
-      }
-      sc[jj] = j0 + jj <= c.t ? s * scale : -INFINITY;
-    }
-    float bm = sc[0];
-#pragma unroll
-    for (int jj = 1; jj < 8; ++jj) bm = fmaxf(bm, sc[jj]);
-    const float mn = fmaxf(m, bm);               // finite: key 0 is in the first block
-    const float corr = __expf(m - mn);
-    l *= corr;
-#pragma unroll
-    for (int i = 0; i < 32; ++i) o[i] *= corr;
-#pragma unroll
-    for (int jj = 0; jj < 8; ++jj) {
-      const float p = __expf(sc[jj] - mn);
-      l += p;
-      const float* vr = vb + (size_t)(j0 + jj) * kD;
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const float4 vv = *reinterpret_cast<const float4*>(vr + 4 * (i ^ jj));
-        o[4 * i] = fmaf(p, vv.x, o[4 * i]);
-        o[4 * i + 1] = fmaf(p, vv.y, o[4 * i + 1]);
-        o[4 * i + 2] = fmaf(p, vv.z, o[4 * i + 2]);
-        o[4 * i + 3] = fmaf(p, vv.w, o[4 * i + 3]);
-      }
-    }
-    m = mn;
-  }
-  const float inv = 1.0f / l;
-#pragma unroll
-  for (int i = 0; i < 32; ++i) o[i] *= inv;
 }
 
 template <int MODE>
@@ -944,18 +697,6 @@ __global__ void tfm_tc_split_kernel(TfmArgs a) {
     a.wimg[o] = hi;
     a.wimg[o + lo] = tf32_rna(w - hi);
   }
-}
-
-// The image entry of the accepted weight-matrix parameter (after the commit kernel, which reads the
-// old one).
-__device__ void image_update(const TfmArgs& a, const DeepCand& c) {
-  const Target tg = tc_target(a, c.idx, c.layer);
-  if (tg.mat == kTcMatNone) return;
-  const float w = a.params[c.idx];
-  const float hi = tf32_rna(w);
-  const size_t o = tfm_tc_image_offset(tg.mat, c.layer, tg.row, tg.col, a.F, a.nL);
-  a.wimg[o] = hi;
-  a.wimg[o + tc_image_lo(tfm_tc_rows(tg.mat))] = tf32_rna(w - hi);
 }
 
 // After the decision and the commit kernel: the image entry of the accepted weight (CTA (0, 0)),

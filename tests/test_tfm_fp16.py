@@ -1,0 +1,134 @@
+"""The Transformer kernels with fp16 operand parts: the range rule that chooses them (needs a GPU), and
+their weight images in the order of consumption (CPU).
+
+Tolerances: dS within TIE_REL * S of the fp64 oracle, as everywhere (parity.py)."""
+import dataclasses
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+from oracle import mca_tfm as T
+from paper_2607_08406_gb300 import workloads as W
+
+from parity import TIE_REL, compare, forced_from_oracle
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("layers,ff,vocab", [(1, 128, 2), (2, 384, 128), (3, 1024, 65)])
+@pytest.mark.parametrize("big", [1.0, 4.0, 30.0])
+def test_tfm_parameter_range(gpu_lib, layers, ff, vocab, big):
+    """Parameters up to `big`: the fp16 kernels up to 4, the tf32 kernels beyond; explicit candidates
+    of either size in every parameter tensor; the smallest and largest feed-forward width and
+    vocabulary. Both sides of the range answer alike."""
+    spec = W.TfmSpec(vocab=vocab, n_layer=layers, d_ff=ff)
+    wl = W.char_transformer(batch=2, text_len=4000, spec=spec, n_trials=8, K=8)
+    rng = np.random.default_rng(5)
+    init = wl.init.copy()
+    init[rng.integers(0, init.size, 40)] = rng.uniform(-1, 1, 40).astype(np.float32)
+    init[rng.integers(0, init.size)] = np.float32(big)
+    wl.init = init
+    h = gpu_lib.create_from_tfm_workload(wl)
+    assert gpu_lib.mca_get_stats(h)["tensor_cores"] == 1
+    flat = init.astype(np.float64)
+    S0 = T.tfm_seq_losses(spec, flat, wl.tokens).sum()
+    assert gpu_lib.mca_loss(h) * 2 * spec.ctx == pytest.approx(S0, rel=TIE_REL)
+    idx, o = [], 0
+    for _, shape in spec.blocks():
+        n = int(np.prod(shape))
+        idx.append(o + int(rng.integers(0, n)))
+        o += n
+    idx = np.array(idx[:128], np.uint32)
+    for amp in (1.0, 8.0):
+        new = rng.uniform(-amp, amp, len(idx)).astype(np.float32)
+        got = gpu_lib.mca_eval_candidates(h, idx, new)
+        for i, v, d in zip(idx, new, got):
+            old, flat[i] = flat[i], v
+            want = T.tfm_seq_losses(spec, flat, wl.tokens).sum() - S0
+            flat[i] = old
+            assert abs(d - want) <= TIE_REL * max(S0, S0 + want)
+
+
+@pytest.mark.gpu
+def test_tfm_perturbations_leave_the_fp16_range(gpu_lib):
+    """A run whose parameters grow past the fp16 kernels' bound continues on the tf32 kernels."""
+    spec = W.TfmSpec(n_layer=1, d_ff=128)
+    wl = W.char_transformer(batch=2, text_len=4000, spec=spec, n_trials=60, K=8)
+    wl.domain = dataclasses.replace(wl.domain, op="perturb", delta=1.2)
+    wl.init = wl.init.copy()
+    wl.init[::97] = np.float32(1.5)
+    tr, flat, S = T.run_full_tfm(spec, wl.tokens, wl.init, 60, 1, wl.domain)
+    h = gpu_lib.create_from_tfm_workload(wl, trace_cap=60)
+    gpu_lib.mca_force_decisions(h, *forced_from_oracle(tr))
+    gpu_lib.mca_run(h, 60, 1)
+    compare(gpu_lib.mca_get_trace(h, 60), tr)
+    assert np.array_equal(gpu_lib.mca_get_params(h, wl.n_params), flat)
+
+
+PROBE = r"""
+#include <cstdio>
+#include <cstdlib>
+#include "%s"
+int main(int, char** argv) {
+  const int F = atoi(argv[1]), nL = atoi(argv[2]);
+  printf("%%zu\n", mca::tfm_f16_image_bytes(F, nL));
+  for (int b = 0; b <= nL; ++b)
+    for (int m = 0; m < 7; ++m) {
+      if ((b == nL) != (m == mca::kTcHead)) continue;
+      const int rows = m == mca::kTcW1 ? F : 128, cols = m == mca::kTcW2 ? F : 128;
+      for (int r = 0; r < rows; ++r)
+        for (int k = 0; k < cols; ++k)
+          printf("%%d %%d %%d %%d %%zu\n", b, m, r, k, mca::tfm_f16_image_offset(m, b, r, k, F, nL));
+    }
+}
+"""
+
+
+@pytest.mark.parametrize("F,nL", [(128, 1), (512, 2), (1024, 1)])
+def test_tfm_f16_image_is_the_order_of_consumption(tmp_path, F, nL):
+    """Chunk by chunk as the control warp issues the MMAs, each chunk the canonical K-major layout (8
+    rows x 16 bytes core matrices, K groups of 8 columns after another), hi then lo."""
+    header = os.path.join(ROOT, "paper_2607_08406_gb300", "csrc", "mca_tc_layout.h")
+    (tmp_path / "p.cpp").write_text(PROBE % header)
+    subprocess.run(["g++", "-std=c++17", "-O1", str(tmp_path / "p.cpp"), "-o", str(tmp_path / "p")],
+                   check=True)
+    out = subprocess.run([str(tmp_path / "p"), str(F), str(nL)], capture_output=True, text=True,
+                         check=True).stdout.split("\n")
+    got = np.array([list(map(int, x.split())) for x in out[1:] if x])
+    want, chunk = {}, 0
+
+    def put(b, m, r0, rows, k0, cols):
+        nonlocal chunk
+        for r in range(rows):
+            for k in range(cols):
+                o = chunk * 8192 + (k // 8) * rows * 8 + r * 8 + k % 8
+                want[(b, m, r0 + r, k0 + k)] = o
+        chunk += 1
+
+    n = F // 64
+    for b in range(nL):
+        for m in range(4):
+            for q in range(4):
+                put(b, m, 0, 128, 32 * q, 32)
+
+        def w1(h):
+            for q in range(2):
+                put(b, 4, 64 * h, 64, 64 * q, 64)
+
+        w1(0), w1(1)
+        for h in range(n):
+            for q in range(2):
+                put(b, 5, 0, 128, 64 * h + 32 * q, 32)
+            if h + 2 < n:
+                w1(h + 2)
+    for q in range(4):
+        put(nL, 6, 0, 128, 32 * q, 32)
+    assert int(out[0]) == chunk * 16384
+    assert len(got) == len(want)
+    assert all(want[tuple(g[:4])] == g[4] for g in got.tolist())
+    # every high part's low part (4096 elements on) is in the same chunk and is no high part
+    offs = np.sort(got[:, 4])
+    assert np.all(offs % 8192 < 4096) and len(np.unique(offs)) == len(offs)
