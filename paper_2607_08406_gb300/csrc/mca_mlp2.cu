@@ -15,10 +15,10 @@ size_t mlp2_window_smem_bytes(int RS) { return window_smem_bytes(RS); }
 static LoopFn pick_loop(const Mlp2Args& a) {
   const bool window = a.window && a.n_explicit == 0;
   if (a.act2 == MCA_ACT_SIGMOID && a.loss == MCA_LOSS_MSE_ONEHOT)
-    return loop_variant_mse(window, a.act1, a.C == 10);
+    return loop_variant_mse(window, a.act1, a.C);
   if (a.act2 == MCA_ACT_IDENTITY && a.loss == MCA_LOSS_SOFTMAX_CE)
-    return loop_variant_ce(window, a.act1, a.C == 10);
-  return window ? mlp2_window_loop<-1, -1, -1, -1> : mlp2_trial_loop<-1, -1, -1, -1>;
+    return loop_variant_ce(window, a.act1, a.C);
+  return window ? mlp2_window_loop<-1, -1, -1, 14> : mlp2_trial_loop<-1, -1, -1, -1>;
 }
 
 size_t mlp2_loop_smem_bytes(const Mlp2Args& a) {

@@ -684,61 +684,262 @@ inline size_t window_smem_bytes(int RS) {
          (size_t)kWS * kCap * (sizeof(unsigned short) + 2 * sizeof(float));
 }
 
-// One cached entry: l' - l from the activation change da (COMMIT: also the new record).
-template <int ACT2, int LOSS, int NC, bool COMMIT>
-__device__ __forceinline__ float entry_cached(const Mlp2Args& a, Recs R,
-                                              const float (&w)[NC > 0 ? NC : kMaxC], int nl,
-                                              float da) {
-  if (da == 0.0f) return 0.0f;
-  constexpr int M = NC > 0 ? NC : kMaxC;
-  const int C = NC > 0 ? NC : a.C;
-  float zz[M];
-  float ell;
-  int y;
-  load_srec(R.rec, R.pitch, nl, zz, ell, y);
+// ------------------------------------------------------------------------------------------------
+// Sample records of the windowed loop, and the change of one sample. What bounds a batch is the number
+// of instructions that one warp has to execute one after another, so a record is a vector per sample
+// (read with three or four 16-byte loads), output fields come in pairs (one instruction for two), and
+// the fields past the class count hold -infinity, whose exponential and sigmoid are 0, instead of a
+// test per field. (One 4-byte load and one instruction per field took, per batch, 4.50 us for
+// 391-1001-7 masked nets with MSE on 12347 samples, 4.17 us for 784-2048-10 ReLU nets with
+// cross-entropy on 30000; now 3.70 and 4.03 us. 784-64-10, all of whose records fit a warp or two: 3.66
+// and 3.68.)
+//
+// M = 10 fields (up to 10 classes): 12 floats a sample, M = 14: 16 floats whose 16-byte parts are
+// permuted by the sample's number, so that the lanes of a warp, which read different samples, spread
+// over the banks (12 floats do by themselves). The loss and the label follow the fields.
+// ------------------------------------------------------------------------------------------------
+template <int M>
+struct VRecs {
+  static_assert(M == 10 || M == 14, "record sizes");
+  static constexpr int kStride = M + 2;
+  float* rec;
+  __device__ __forceinline__ float* part(int n, int q) const {
+    return rec + n * kStride + 4 * (M == 10 ? q : q ^ ((n >> 1) & 3));
+  }
+  __device__ __forceinline__ float& at(int n, int f) const { return part(n, f >> 2)[f & 3]; }
+  __device__ __forceinline__ void load(int n, float2 (&z)[M / 2], float& ell, int& y) const {
 #pragma unroll
-  for (int k = 0; k < M; ++k)
-    if (k < C) zz[k] = fmaf(w[k], da, zz[k]);
-  const float ln = sample_loss<ACT2, LOSS, M>(zz, C, y, a.g2, a.act2, a.loss);
-  if (COMMIT) store_srec(R.rec, R.pitch, nl, zz, ln, y);
+    for (int q = 0; q < kStride / 4; ++q) {
+      const float4 v = *reinterpret_cast<const float4*>(part(n, q));
+      z[2 * q] = make_float2(v.x, v.y);
+      if (2 * q + 1 < M / 2) {
+        z[2 * q + 1] = make_float2(v.z, v.w);
+      } else {
+        ell = v.z;
+        y = __float_as_int(v.w);
+      }
+    }
+  }
+  __device__ __forceinline__ void store(int n, const float2 (&z)[M / 2], float ell, int y) const {
+#pragma unroll
+    for (int q = 0; q < kStride / 4; ++q) {
+      const bool last = 2 * q + 1 == M / 2;
+      const float2 b = last ? make_float2(ell, __int_as_float(y)) : z[last ? 0 : 2 * q + 1];
+      *reinterpret_cast<float4*>(part(n, q)) = make_float4(z[2 * q].x, z[2 * q].y, b.x, b.y);
+    }
+  }
+};
+
+__device__ __forceinline__ unsigned long long pack2(float2 v) {
+  return *reinterpret_cast<const unsigned long long*>(&v);
+}
+__device__ __forceinline__ float2 unpack2(unsigned long long v) {
+  return *reinterpret_cast<const float2*>(&v);
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  unsigned long long d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(pack2(a)), "l"(pack2(b)), "l"(pack2(c)));
+  return unpack2(d);
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+  unsigned long long d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(pack2(a)), "l"(pack2(b)));
+  return unpack2(d);
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+  unsigned long long d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(pack2(a)), "l"(pack2(b)));
+  return unpack2(d);
+}
+
+// Loss of the fields z with label y; zy: field y; onehot: -[k == y] per field (MSE).
+template <int ACT2, int LOSS, int M>
+__device__ __forceinline__ float vloss(const Mlp2Args& a, const float2 (&z)[M / 2], int y, float zy,
+                                       const float* onehot) {
+  if constexpr (ACT2 == MCA_ACT_IDENTITY && LOSS == MCA_LOSS_SOFTMAX_CE) {
+    float m = fmaxf(z[0].x, z[0].y);
+#pragma unroll
+    for (int q = 1; q < M / 2; ++q) m = fmaxf(m, fmaxf(z[q].x, z[q].y));
+    float2 s = make_float2(0.0f, 0.0f);
+#pragma unroll
+    for (int q = 0; q < M / 2; ++q) {
+      const float2 t = mul2(add2(z[q], make_float2(-m, -m)), make_float2(kLog2e, kLog2e));
+      s = add2(s, make_float2(ex2_ftz(t.x), ex2_ftz(t.y)));
+    }
+    return (__logf(s.x + s.y) + m) - zy;
+  } else if constexpr (ACT2 == MCA_ACT_SIGMOID && LOSS == MCA_LOSS_MSE_ONEHOT) {
+    const float* oh = onehot + 16 * y;
+    float2 s = make_float2(0.0f, 0.0f);
+#pragma unroll
+    for (int q = 0; q < M / 2; ++q) {
+      const float2 t = mul2(z[q], make_float2(-kLog2e, -kLog2e));
+      const float2 u = add2(make_float2(ex2_ftz(t.x), ex2_ftz(t.y)), make_float2(1.0f, 1.0f));
+      const float2 d = add2(make_float2(rcp_ftz(u.x), rcp_ftz(u.y)),
+                            *reinterpret_cast<const float2*>(oh + 2 * q));
+      s = fma2(d, d, s);
+    }
+    return s.x + s.y;
+  } else {
+    float zz[M];
+#pragma unroll
+    for (int q = 0; q < M / 2; ++q) {
+      zz[2 * q] = z[q].x;
+      zz[2 * q + 1] = z[q].y;
+    }
+    return sample_loss<-1, -1, M>(zz, a.C, y, a.g2, a.act2, a.loss);
+  }
+}
+
+// The direction in which a candidate moves the output fields, per unit of its entries' numbers:
+// W2[:, j] for a first-layer weight (w2c), delta on field o for an output-layer weight W2[o, j].
+template <int M>
+struct Direction {
+  float2 w[M / 2];
+  const float* w2c;          // first layer: the column, in shared memory
+  int o;                     // output layer: the field (-1: first layer)
+  float delta;
+  __device__ __forceinline__ float at(int y) const { return o < 0 ? w2c[y] : y == o ? delta : 0.0f; }
+};
+
+template <int M>
+__device__ __forceinline__ Direction<M> direction(const Cand& c, const float* w2c) {
+  Direction<M> d;
+  d.w2c = w2c;
+  d.o = c.layer == 0 ? -1 : c.row;
+  d.delta = c.delta;
+#pragma unroll
+  for (int q = 0; q < M / 2; ++q)
+    d.w[q] = c.layer == 0 ? *reinterpret_cast<const float2*>(w2c + 2 * q)
+                          : make_float2(2 * q == c.row ? c.delta : 0.0f,
+                                        2 * q + 1 == c.row ? c.delta : 0.0f);
+  return d;
+}
+
+// The change of a sample whose activation change is not finite: 0 times it is no change of the fields
+// that the candidate does not touch. (A call: the same inline took 2 % of every batch.)
+template <int M, bool COMMIT>
+__device__ __noinline__ float vdelta_any(const Mlp2Args& a, VRecs<M> R, const float* w2c, int o,
+                                         float delta, int nl, float da) {
+  float zz[M];
+#pragma unroll
+  for (int f = 0; f < M; ++f) {
+    const float z = R.at(nl, f);
+    zz[f] = o >= 0 ? (f == o ? fmaf(delta, da, z) : z) : f < a.C ? fmaf(w2c[f], da, z) : z;
+  }
+  const float ell = R.at(nl, M);
+  const float ln = sample_loss<-1, -1, M>(zz, a.C, __float_as_int(R.at(nl, M + 1)), a.g2, a.act2,
+                                          a.loss);
+  if (COMMIT) {
+#pragma unroll
+    for (int f = 0; f < M; ++f) R.at(nl, f) = zz[f];
+    R.at(nl, M) = ln;
+  }
   return ln - ell;
 }
 
-// l' - l of one cached entry without branches (0 exactly when da == 0), so that a lane can keep
-// several entries in flight.
-template <int ACT2, int LOSS, int NC>
-__device__ __forceinline__ float cached_delta(const Mlp2Args& a, Recs R,
-                                              const float (&w)[NC > 0 ? NC : kMaxC], int nl,
-                                              float da) {
-  constexpr int M = NC > 0 ? NC : kMaxC;
-  const int C = NC > 0 ? NC : a.C;
-  float zz[M];
+// l' - l of sample nl whose fields move by da along dir; COMMIT also writes the new record (not when
+// nothing changes). Exactly 0 when da == 0, or when an output-layer weight moves no field. ANY: da may be
+// infinite or NaN.
+template <int ACT2, int LOSS, int M, bool COMMIT, bool ANY>
+__device__ __forceinline__ float vdelta(const Mlp2Args& a, const VRecs<M>& R, const float* onehot,
+                                        const Direction<M>& dir, int nl, float da) {
+  if (ANY && !(fabsf(da) < INFINITY))
+    return vdelta_any<M, COMMIT>(a, R, dir.w2c, dir.o, dir.delta, nl, da);
+  float2 z[M / 2];
   float ell;
   int y;
-  load_srec(R.rec, R.pitch, nl, zz, ell, y);
+  R.load(nl, z, ell, y);
+  const float zy = LOSS == MCA_LOSS_SOFTMAX_CE ? fmaf(dir.at(y), da, R.at(nl, y)) : 0.0f;
+  bool same = da == 0.0f;
+  if (dir.o >= 0) {
+    const float zo = R.at(nl, dir.o);
+    same = fmaf(dir.delta, da, zo) == zo;
+  }
 #pragma unroll
-  for (int k = 0; k < M; ++k)
-    if (k < C) zz[k] = fmaf(w[k], da, zz[k]);
-  const float ln = sample_loss<ACT2, LOSS, M>(zz, C, y, a.g2, a.act2, a.loss);
-  return da == 0.0f ? 0.0f : ln - ell;
+  for (int q = 0; q < M / 2; ++q) z[q] = fma2(dir.w[q], make_float2(da, da), z[q]);
+  const float ln = vloss<ACT2, LOSS, M>(a, z, y, zy, onehot);
+  if (COMMIT && !same) R.store(nl, z, ln, y);
+  return same ? 0.0f : ln - ell;
 }
 
 // Warp-level sum of l' - l over the cached entries e .. e + 31 of a slot (of n), one per lane.
-template <int ACT2, int LOSS, int NC>
-__device__ __forceinline__ float eval_cached(const Mlp2Args& a, Recs R,
-                                             const float (&w)[NC > 0 ? NC : kMaxC],
+template <int ACT2, int LOSS, int M>
+__device__ __forceinline__ float eval_cached(const Mlp2Args& a, const VRecs<M>& R,
+                                             const float* onehot, const Direction<M>& dir,
                                              const unsigned short* nl, const float* da, int e,
                                              int n) {
   e += threadIdx.x & 31;
   const bool in = e < n;
-  return warp_sum(
-      cached_delta<ACT2, LOSS, NC>(a, R, w, in ? (int)nl[e] : 0, in ? da[e] : 0.0f));
+  return warp_sum(vdelta<ACT2, LOSS, M, false, false>(a, R, onehot, dir, in ? (int)nl[e] : 0,
+                                                      in ? da[e] : 0.0f));
+}
+
+// The number that goes with an entry, from global memory: f(z + delta x) - f(z) (zn = z + delta x), or
+// f(z) for an output-layer weight.
+template <int ACT1>
+__device__ __forceinline__ float entry_step(const Mlp2Args& a, const Cand& c, float x, float z,
+                                            float& zn) {
+  const float f = act_compact<ACT1>(z, a.g1, a.act1);
+  zn = z;
+  if (c.layer != 0) return f;
+  zn = fmaf(c.delta, x, z);
+  return act_compact<ACT1>(zn, a.g1, a.act1) - f;
+}
+
+// Warp-level sum of l' - l over chunk q (of a.SUB entries) of a candidate that is not cached. Lane l
+// takes entries l, l + 32, ... in ascending order; the next entry's loads are in flight.
+template <int ACT1, int ACT2, int LOSS, int M>
+__device__ __forceinline__ float eval_global(const Mlp2Args& a, const VRecs<M> R,
+                                             const float* onehot, int s0, const Cand& c,
+                                             const float* w2c, int q) {
+  const int e_hi = min(q * a.SUB + a.SUB, c.ecnt);
+  const float* zrow = a.z1 + (size_t)(c.layer == 0 ? c.row : c.col) * a.Np;
+  const Direction<M> dir = direction<M>(c, w2c);
+  float acc = 0.0f, x1 = 0.0f, z1 = 0.0f;
+  int n1 = 0;
+  auto fetch = [&](int e) {
+    if (e < e_hi) {
+      n1 = c.layer == 0 ? __ldg(a.xs_n + c.ebeg + e) : s0 + e;
+      x1 = c.layer == 0 ? __ldg(a.xs_v + c.ebeg + e) : 0.0f;
+      z1 = zrow[n1];
+    }
+  };
+  const int e0 = q * a.SUB + (int)(threadIdx.x & 31);
+  fetch(e0);
+#pragma unroll 1
+  for (int e = e0; e < e_hi; e += 32) {
+    const int n = n1;
+    float zn;
+    const float da = entry_step<ACT1>(a, c, x1, z1, zn);
+    fetch(e + 32);
+    acc += vdelta<ACT2, LOSS, M, false, true>(a, R, onehot, dir, n - s0, da);
+  }
+  __syncwarp();
+  return warp_sum(acc);
+}
+
+// Commit of a candidate that is not cached to this CTA's samples: thread i0 of istride.
+template <int ACT1, int ACT2, int LOSS, int M>
+__device__ __forceinline__ void commit_global(const Mlp2Args& a, const VRecs<M> R,
+                                              const float* onehot, int s0, const Cand& c,
+                                              const float* w2c, int i0, int istride) {
+  float* zrow = a.z1 + (size_t)(c.layer == 0 ? c.row : c.col) * a.Np;
+  const Direction<M> dir = direction<M>(c, w2c);
+#pragma unroll 1
+  for (int e = i0; e < c.ecnt; e += istride) {
+    const int n = c.layer == 0 ? __ldg(a.xs_n + c.ebeg + e) : s0 + e;
+    const float x = c.layer == 0 ? __ldg(a.xs_v + c.ebeg + e) : 0.0f;
+    float zn;
+    const float da = entry_step<ACT1>(a, c, x, zrow[n], zn);
+    if (c.layer == 0) zrow[n] = zn;
+    (void)vdelta<ACT2, LOSS, M, true, true>(a, R, onehot, dir, n - s0, da);
+  }
 }
 
 // Warp prepares slot sl for trial t: proposal, W2 column, and (cacheable first-layer candidates)
 // the gathered entries; then publishes it. `epoch` was read before any of the data.
 template <int ACT1>
-__device__ __forceinline__ void prepare_slot(const Mlp2Args& a, WSlot* slots, float (*w2c)[kMaxC],
+__device__ __forceinline__ void prepare_slot(const Mlp2Args& a, WSlot* slots, float (*w2c)[16],
                                              unsigned short* e_nl, float* e_da, float* e_zn,
                                              int sl, unsigned long long t, int epoch, int r, int s0,
                                              int s1) {
@@ -755,10 +956,10 @@ __device__ __forceinline__ void prepare_slot(const Mlp2Args& a, WSlot* slots, fl
   __syncwarp();
   const Cand c = slots[sl].c;
   if (c.layer == 0 && c.gcnt > 0) {
-    for (int q = lane; q < kMaxC; q += 32)
-      w2c[sl][q] = q < a.C ? a.w2[(size_t)q * a.H + c.row] : 0.0f;
+    if (lane < 16) w2c[sl][lane] = lane < a.C ? a.w2[(size_t)lane * a.H + c.row] : 0.0f;
   }
-  int state = 2;
+  int state = 2;             // not cached: does not fit, or activation changes that are not finite
+  bool finite = true;
   if (c.gcnt == 0) {
     state = 1;
   } else if (c.layer == 0 && c.ecnt <= kCap) {
@@ -788,10 +989,12 @@ __device__ __forceinline__ void prepare_slot(const Mlp2Args& a, WSlot* slots, fl
         const float z2 = fmaf(c.delta, xv[u], zv[u]);
         nl[e] = (unsigned short)(nn[u] - s0);
         zn[e] = z2;
-        da[e] = act_compact<ACT1>(z2, a.g1, a.act1) - act_compact<ACT1>(zv[u], a.g1, a.act1);
+        const float d = act_compact<ACT1>(z2, a.g1, a.act1) - act_compact<ACT1>(zv[u], a.g1, a.act1);
+        da[e] = d;
+        finite &= fabsf(d) < INFINITY;
       }
     }
-    state = 1;
+    state = __all_sync(0xffffffffu, finite) ? 1 : 2;
   }
   __syncwarp();
   if (lane == 0) {
@@ -917,11 +1120,13 @@ __device__ __forceinline__ unsigned long long batch_bytes(const WSlot* slots, un
   return bytes;
 }
 
-template <int ACT1, int ACT2, int LOSS, int NC>
+// M: fields of a sample's record (10 for up to 10 classes, else 14).
+template <int ACT1, int ACT2, int LOSS, int M>
 __global__ void __launch_bounds__(kLoopThreads, 1) mlp2_window_loop(Mlp2Args a) {
   extern __shared__ __align__(16) float s_dyn[];
   __shared__ WSlot s_slot[kWS];
-  __shared__ float s_w2c[kWS][kMaxC];
+  __shared__ __align__(16) float s_w2c[kWS][16];
+  __shared__ __align__(16) float s_onehot[16][16];   // -[k == y]
   __shared__ float s_sub[kWinBatch][kMaxSubs];        // sums of a candidate's chunks
   __shared__ CommitLog s_log[kLogLen];
   __shared__ float s_dS[kWinBatch];
@@ -941,18 +1146,24 @@ __global__ void __launch_bounds__(kLoopThreads, 1) mlp2_window_loop(Mlp2Args a) 
   unsigned short* e_nl = reinterpret_cast<unsigned short*>(s_dyn + kRecFields * a.RS);
   float* e_da = reinterpret_cast<float*>(e_nl + kWS * kCap);
   float* e_zn = e_da + kWS * kCap;
-  constexpr int M = NC > 0 ? NC : kMaxC;
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int r = blockIdx.x;
   const int s0 = min(r * a.RS, a.N), s1 = min(s0 + a.RS, a.N);
-  const Recs R{s_records, a.RS};
+  const VRecs<M> R{s_records};
+  const float* onehot = &s_onehot[0][0];
   {
+    // the records: fields past the class count hold -infinity
     const int ns = s1 - s0;
-    for (int t = tid; t < kRecFields * ns; t += kLoopThreads) {
-      const int f = t / ns, nl = t - f * ns;
-      s_records[f * a.RS + nl] = a.srec[(size_t)f * a.Np + s0 + nl];
-    }
+#pragma unroll 1
+    for (int f = 0; f < M + 2; ++f)
+#pragma unroll 1
+      for (int nl = tid; nl < ns; nl += kLoopThreads)
+        R.at(nl, f) = f < M && f >= a.C
+                          ? -INFINITY
+                          : a.srec[(size_t)(f < M ? f : f - M + kRecLoss) * a.Np + s0 + nl];
+    for (int q = tid; q < 256; q += kLoopThreads)
+      s_onehot[q >> 4][q & 15] = (q >> 4) == (q & 15) ? -1.0f : 0.0f;
   }
   for (int q = tid; q < kWS; q += kLoopThreads) s_slot[q].ticket = 0ull;
   for (int q = tid; q < kRedoLen; q += kLoopThreads) s_redo_q[q] = 0ull;
@@ -1184,30 +1395,18 @@ __global__ void __launch_bounds__(kLoopThreads, 1) mlp2_window_loop(Mlp2Args a) 
         const int i0 = tid - 32, istride = kConsThreads - 32;
         if (c.gcnt > 0) {
           if (s_slot[sl].state == 1) {
-            float w[M];
-            load_w2c<NC>(s_w2c[sl], a.C, w);
+            const Direction<M> dir = direction<M>(c, s_w2c[sl]);
             float* zrow = a.z1 + (size_t)c.row * a.Np + s0;
             const unsigned short* nl = e_nl + (size_t)sl * kCap;
             const float* da = e_da + (size_t)sl * kCap;
             const float* zn = e_zn + (size_t)sl * kCap;
+#pragma unroll 1
             for (int e = i0; e < c.ecnt; e += istride) {
               zrow[nl[e]] = zn[e];
-              (void)entry_cached<ACT2, LOSS, NC, true>(a, R, w, nl[e], da[e]);
-            }
-          } else if (c.layer == 0) {
-            float* zrow = a.z1 + (size_t)c.row * a.Np;
-            float w[M];
-            load_w2c<NC>(s_w2c[sl], a.C, w);
-            for (int e = i0; e < c.ecnt; e += istride) {
-              const int n = __ldg(a.xs_n + c.ebeg + e);
-              const float x = __ldg(a.xs_v + c.ebeg + e);
-              (void)entry_l1<ACT1, ACT2, LOSS, NC, true>(a, R, c.delta, w, n - s0, x, zrow[n],
-                                                        zrow + n);
+              (void)vdelta<ACT2, LOSS, M, true, false>(a, R, onehot, dir, nl[e], da[e]);
             }
           } else {
-            const float* zrow = a.z1 + (size_t)c.col * a.Np;
-            for (int e = i0; e < c.ecnt; e += istride)
-              (void)entry_l2<ACT1, ACT2, LOSS, NC, true>(a, R, c.delta, c.row, e, zrow[s0 + e]);
+            commit_global<ACT1, ACT2, LOSS, M>(a, R, onehot, s0, c, s_w2c[sl], i0, istride);
           }
         }
         if (tid == 32) {
@@ -1347,19 +1546,19 @@ __global__ void __launch_bounds__(kLoopThreads, 1) mlp2_window_loop(Mlp2Args a) 
           const bool alone = wpc == 1 || nc == 1;
           float v = 0.0f;
           if (cached) {
-            float w[M];
-            load_w2c<NC>(s_w2c[sl], a.C, w);
+            const Direction<M> dir = direction<M>(c, s_w2c[sl]);
 #pragma unroll 1
             for (int q = j; q < nc; q += wpc) {
-              const float t = eval_cached<ACT2, LOSS, NC>(a, R, w, e_nl + (size_t)sl * kCap,
-                                                          e_da + (size_t)sl * kCap, 32 * q, c.ecnt);
+              const float t =
+                  eval_cached<ACT2, LOSS, M>(a, R, onehot, dir, e_nl + (size_t)sl * kCap,
+                                             e_da + (size_t)sl * kCap, 32 * q, c.ecnt);
               v += t;
               if (!alone && lane == 0) s_sub[k][q] = t;
             }
           } else {
 #pragma unroll 1
             for (int q = j; q < nc; q += wpc) {
-              const float t = eval_sub<ACT1, ACT2, LOSS, NC>(a, R, s0, c, s_w2c[sl], q);
+              const float t = eval_global<ACT1, ACT2, LOSS, M>(a, R, onehot, s0, c, s_w2c[sl], q);
               v += t;
               if (!alone && lane == 0) s_sub[k][q] = t;
             }
@@ -1621,34 +1820,36 @@ __global__ void __launch_bounds__(kLoopThreads, 1) mlp2_window_loop(Mlp2Args a) 
   __syncthreads();
   {
     const int ns = s1 - s0;
-    for (int t = tid; t < kRecFields * ns; t += kLoopThreads) {
-      const int f = t / ns, nl = t - f * ns;
-      a.srec[(size_t)f * a.Np + s0 + nl] = s_records[f * a.RS + nl];
+#pragma unroll 1
+    for (int f = 0; f < M + 1; ++f) {              // (the labels do not change)
+      if (f < M && f >= a.C) continue;
+#pragma unroll 1
+      for (int nl = tid; nl < ns; nl += kLoopThreads)
+        a.srec[(size_t)(f < M ? f : kRecLoss) * a.Np + s0 + nl] = R.at(nl, f);
     }
   }
 }
 
-// Trial-loop kernels (windowed or not) by hidden transfer function and class count (ten: exactly 10
-// classes) for sigmoid outputs with MSE (mca_mlp2_mse.cu) and identity outputs with cross-entropy
-// (mca_mlp2_ce.cu).
+// Trial-loop kernels (windowed or not) by hidden transfer function and class count C, for sigmoid
+// outputs with MSE (mca_mlp2_mse.cu) and identity outputs with cross-entropy (mca_mlp2_ce.cu).
 using LoopFn = void (*)(Mlp2Args);
-LoopFn loop_variant_mse(bool window, int act1, bool ten);
-LoopFn loop_variant_ce(bool window, int act1, bool ten);
+LoopFn loop_variant_mse(bool window, int act1, int C);
+LoopFn loop_variant_ce(bool window, int act1, int C);
 
-template <int ACT2, int LOSS, int NC>
+template <int ACT2, int LOSS, int NC, int M>
 LoopFn loop_variant(bool window, int act1) {
   switch (act1) {
     case MCA_ACT_TANH:
-      return window ? mlp2_window_loop<MCA_ACT_TANH, ACT2, LOSS, NC>
+      return window ? mlp2_window_loop<MCA_ACT_TANH, ACT2, LOSS, M>
                     : mlp2_trial_loop<MCA_ACT_TANH, ACT2, LOSS, NC>;
     case MCA_ACT_GAUSSIAN:
-      return window ? mlp2_window_loop<MCA_ACT_GAUSSIAN, ACT2, LOSS, NC>
+      return window ? mlp2_window_loop<MCA_ACT_GAUSSIAN, ACT2, LOSS, M>
                     : mlp2_trial_loop<MCA_ACT_GAUSSIAN, ACT2, LOSS, NC>;
     case MCA_ACT_RELU:
-      return window ? mlp2_window_loop<MCA_ACT_RELU, ACT2, LOSS, NC>
+      return window ? mlp2_window_loop<MCA_ACT_RELU, ACT2, LOSS, M>
                     : mlp2_trial_loop<MCA_ACT_RELU, ACT2, LOSS, NC>;
     default:
-      return window ? mlp2_window_loop<-1, ACT2, LOSS, NC> : mlp2_trial_loop<-1, ACT2, LOSS, NC>;
+      return window ? mlp2_window_loop<-1, ACT2, LOSS, M> : mlp2_trial_loop<-1, ACT2, LOSS, NC>;
   }
 }
 

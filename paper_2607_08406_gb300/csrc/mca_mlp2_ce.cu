@@ -3,9 +3,10 @@
 
 namespace mca {
 
-LoopFn loop_variant_ce(bool window, int act1, bool ten) {
-  return ten ? loop_variant<MCA_ACT_IDENTITY, MCA_LOSS_SOFTMAX_CE, 10>(window, act1)
-             : loop_variant<MCA_ACT_IDENTITY, MCA_LOSS_SOFTMAX_CE, -1>(window, act1);
+LoopFn loop_variant_ce(bool window, int act1, int C) {
+  if (C == 10) return loop_variant<MCA_ACT_IDENTITY, MCA_LOSS_SOFTMAX_CE, 10, 10>(window, act1);
+  if (C < 10) return loop_variant<MCA_ACT_IDENTITY, MCA_LOSS_SOFTMAX_CE, -1, 10>(window, act1);
+  return loop_variant<MCA_ACT_IDENTITY, MCA_LOSS_SOFTMAX_CE, -1, 14>(window, act1);
 }
 
 }  // namespace mca

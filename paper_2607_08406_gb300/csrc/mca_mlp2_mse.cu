@@ -3,9 +3,10 @@
 
 namespace mca {
 
-LoopFn loop_variant_mse(bool window, int act1, bool ten) {
-  return ten ? loop_variant<MCA_ACT_SIGMOID, MCA_LOSS_MSE_ONEHOT, 10>(window, act1)
-             : loop_variant<MCA_ACT_SIGMOID, MCA_LOSS_MSE_ONEHOT, -1>(window, act1);
+LoopFn loop_variant_mse(bool window, int act1, int C) {
+  if (C == 10) return loop_variant<MCA_ACT_SIGMOID, MCA_LOSS_MSE_ONEHOT, 10, 10>(window, act1);
+  if (C < 10) return loop_variant<MCA_ACT_SIGMOID, MCA_LOSS_MSE_ONEHOT, -1, 10>(window, act1);
+  return loop_variant<MCA_ACT_SIGMOID, MCA_LOSS_MSE_ONEHOT, -1, 14>(window, act1);
 }
 
 }  // namespace mca
