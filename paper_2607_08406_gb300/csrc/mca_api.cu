@@ -77,7 +77,7 @@ bool is_device_ptr(const void* p) {
 
 struct Layout {
   size_t XT, y, xs_off, xs_n, xs_v, xs_sect, xs_roff, z1, srec, partial, accum, bar, st, trace,
-      ex_idx, ex_new, ex_out, prop, scratch, ell, ctl, gimg, scr_tab, total;
+      ex_idx, ex_new, scratch, ell, ctl, gimg, scr_tab, total;
   std::vector<size_t> w_eff, code, wfix, Z, whi, scr;
 };
 
@@ -184,8 +184,6 @@ Layout plan(const std::vector<mca_layer>& layers, long long N, int D, long long 
   L.trace = take(sizeof(mca_trace_rec) * (size_t)std::max(trace_cap, 0));
   L.ex_idx = take(sizeof(unsigned int) * mca::kKmax);
   L.ex_new = take(sizeof(float) * mca::kKmax);
-  L.ex_out = take(sizeof(double) * mca::kKmax);
-  L.prop = take(sizeof(mca_trace_rec) * mca::kKmax);
   L.scratch = take(sizeof(int) * (size_t)(D + 8));
   const size_t gb = forward_tc_image_bytes(layers, Np);
   L.gimg = gb ? take(gb) : SIZE_MAX;
@@ -694,7 +692,7 @@ mca_status tfm_check(const mca_tfm_spec* t, int64_t n_seq) {
 }
 
 struct TfmMem {
-  size_t params, tokens, X, ell, partial, st, ctl, trace, ex_idx, ex_new, ex_out, prop, scratch,
+  size_t params, tokens, X, ell, partial, st, ctl, trace, ex_idx, ex_new, scratch,
       wimg, wimg16, Xmid, scrX, scr_ell, ctl2, tau_dev, total;
   int nscr;
 };
@@ -737,8 +735,6 @@ TfmMem tfm_plan(const mca_tfm_spec& t, long long B, int trace_cap, bool tc, int 
   M.trace = take(sizeof(mca_trace_rec) * (size_t)std::max(trace_cap, 0));
   M.ex_idx = take(sizeof(unsigned int) * mca::kKmax);
   M.ex_new = take(sizeof(float) * mca::kKmax);
-  M.ex_out = take(sizeof(double) * mca::kKmax);
-  M.prop = take(sizeof(mca_trace_rec) * mca::kKmax);
   M.scratch = take(sizeof(int) * 8);
   M.wimg = tc ? take(sizeof(float) * mca::tfm_tc_image_floats(t.d_ff, t.n_layer)) : 0;
   M.wimg16 = tc ? take(mca::tfm_f16_image_bytes(t.d_ff, t.n_layer)) : 0;
@@ -1072,8 +1068,6 @@ mca_status mca_create(const mca_layer* layers, int32_t n_layers, int32_t loss,
   h->trace = o.trace_cap > 0 ? reinterpret_cast<mca_trace_rec*>(base + L.trace) : nullptr;
   h->ex_idx = reinterpret_cast<unsigned int*>(base + L.ex_idx);
   h->ex_new = reinterpret_cast<float*>(base + L.ex_new);
-  h->ex_out = reinterpret_cast<double*>(base + L.ex_out);
-  h->prop = reinterpret_cast<mca_trace_rec*>(base + L.prop);
   h->gimg = L.gimg != SIZE_MAX ? reinterpret_cast<float*>(base + L.gimg) : nullptr;
   int* scratch = reinterpret_cast<int*>(base + L.scratch);
   CTRY(cudaMemsetAsync(h->st, 0, sizeof(DevState), h->stream));
@@ -1132,6 +1126,8 @@ mca_status mca_create(const mca_layer* layers, int32_t n_layers, int32_t loss,
     CTRY(cudaMemcpyAsync(h->y, yh.data(), sizeof(int) * h->N, cudaMemcpyHostToDevice, h->stream));
     CTRY(cudaStreamSynchronize(h->stream));
   }
+  CTRY(cudaMallocHost(reinterpret_cast<void**>(&h->ev_host), sizeof(*h->ev_host)));
+  std::memset(h->ev_host, 0, sizeof(*h->ev_host));
   TRY(load_params(h, init_params, nullptr));
   TRY(resync(h));
   DevState ds;
@@ -1443,16 +1439,19 @@ mca_status mca_force_decisions(mca_handle* h, const uint64_t* tau, const uint8_t
 namespace {
 
 // Loss changes of the n candidates in h->ex_idx / h->ex_new against the current state, no commit,
-// into dS (host); wmax: the candidates' largest magnitude. The evaluation kernels of mca_run's
-// evaluation step.
-mca_status eval_explicit(mca_handle* h, size_t n, float wmax, double* dS) {
+// into h->ev_host; wmax: the candidates' largest magnitude. The evaluation kernels of mca_run's
+// evaluation step. The kernels write the results to pinned memory, so one synchronisation ends the
+// call.
+mca_status eval_explicit(mca_handle* h, size_t n, float wmax) {
+  auto* ev = h->ev_host;
   if (h->tfm) {
     mca::TfmArgs a = tfm_args(h);
     if (wmax > mca::kTfmF16Max) a.f16 = 0;
     a.n_explicit = (int)n;
     a.ex_idx = h->ex_idx;
     a.ex_new = h->ex_new;
-    a.ex_out = h->ex_out;
+    a.ex_out = ev->dS;
+    a.ex_tail = &ev->tail;
     CUDA_TRY(h, mca::launch_tfm_eval(a, h->stream));
     CUDA_TRY(h, mca::launch_tfm_decide(a, h->stream));
     h->launches += 2;
@@ -1461,7 +1460,8 @@ mca_status eval_explicit(mca_handle* h, size_t n, float wmax, double* dS) {
     a.n_explicit = (int)n;
     a.ex_idx = h->ex_idx;
     a.ex_new = h->ex_new;
-    a.ex_out = h->ex_out;
+    a.ex_out = ev->dS;
+    a.ex_tail = &ev->tail;
     CUDA_TRY(h, mca::launch_deep_eval(a, h->stream));
     CUDA_TRY(h, mca::launch_deep_decide(a, h->stream));
     h->launches += 2;
@@ -1470,18 +1470,15 @@ mca_status eval_explicit(mca_handle* h, size_t n, float wmax, double* dS) {
     a.n_explicit = (int)n;
     a.ex_idx = h->ex_idx;
     a.ex_new = h->ex_new;
-    a.ex_out = h->ex_out;
-    CUDA_TRY(h, cudaMemsetAsync(h->bar, 0, sizeof(GridBarrier), h->stream));
+    a.ex_out = ev->dS;
+    a.ex_tail = &ev->tail;
+    if (!h->smem_records)            // the trial loop's grid barrier counts generations from 0
+      CUDA_TRY(h, cudaMemsetAsync(h->bar, 0, sizeof(GridBarrier), h->stream));
     CUDA_TRY(h, mca::launch_mlp2_loop(a, h->stream));
     h->launches++;
   }
-  CUDA_TRY(h, cudaMemcpyAsync(dS, h->ex_out, sizeof(double) * n, cudaMemcpyDeviceToHost,
-                              h->stream));
   CUDA_TRY(h, cudaStreamSynchronize(h->stream));
-  DevState ds;
-  mca_status rc = read_state(h, &ds);
-  if (rc != MCA_OK) return rc;
-  if (ds.err == MCA_ERR_TIMEOUT) {
+  if (ev->tail.err == MCA_ERR_TIMEOUT) {
     h->broken = true;
     return fail(h, MCA_ERR_TIMEOUT, "device-side wait timed out");
   }
@@ -1496,17 +1493,22 @@ mca_status mca_eval_candidates(mca_handle* h, const uint32_t* flat_idx, const fl
   if (n > (size_t)mca::kKmax) return fail(h, MCA_ERR_INVALID, "n = %zu > %d", n, mca::kKmax);
   if (h->broken) return fail(h, MCA_ERR_CUDA, "handle unusable after an earlier device error");
   if (n == 0) return MCA_OK;
+  float wmax = 0.0f;
   for (size_t m = 0; m < n; ++m) {
     if (flat_idx[m] >= h->P) return fail(h, MCA_ERR_INVALID, "flat_idx[%zu] >= P", m);
     if (!std::isfinite(new_w[m])) return fail(h, MCA_ERR_INVALID, "new_w[%zu] not finite", m);
+    wmax = std::max(wmax, std::fabs(new_w[m]));
   }
-  CUDA_TRY(h, cudaMemcpyAsync(h->ex_idx, flat_idx, sizeof(unsigned int) * n, cudaMemcpyHostToDevice,
+  std::memcpy(h->ev_host->idx, flat_idx, sizeof(unsigned int) * n);
+  std::memcpy(h->ev_host->new_w, new_w, sizeof(float) * n);
+  // ex_idx and ex_new lie one after the other, as in EvalHost
+  CUDA_TRY(h, cudaMemcpyAsync(h->ex_idx, h->ev_host->idx,
+                              sizeof(h->ev_host->idx) + sizeof(float) * n, cudaMemcpyHostToDevice,
                               h->stream));
-  CUDA_TRY(h, cudaMemcpyAsync(h->ex_new, new_w, sizeof(float) * n, cudaMemcpyHostToDevice,
-                              h->stream));
-  float wmax = 0.0f;
-  for (size_t m = 0; m < n; ++m) wmax = std::max(wmax, std::fabs(new_w[m]));
-  return eval_explicit(h, n, wmax, dS);
+  const mca_status rc = eval_explicit(h, n, wmax);
+  if (rc != MCA_OK) return rc;
+  std::memcpy(dS, h->ev_host->dS, sizeof(double) * n);
+  return MCA_OK;
 }
 
 mca_status mca_eval_trials(mca_handle* h, uint64_t seed, uint64_t tau, size_t n,
@@ -1537,22 +1539,17 @@ mca_status mca_eval_trials(mca_handle* h, uint64_t seed, uint64_t tau, size_t n,
   a.stretch = h->dom.layer_stretch;
   a.seed = seed;
   a.tau0 = tau;
-  a.rec = h->prop;
+  a.rec = h->ev_host->prop;
   a.ex_idx = h->ex_idx;
   a.ex_new = h->ex_new;
   CUDA_TRY(h, mca::launch_propose(a, h->stream));
   h->launches++;
-  CUDA_TRY(h, cudaMemcpyAsync(out, h->prop, sizeof(mca_trace_rec) * n, cudaMemcpyDeviceToHost,
-                              h->stream));
-  double dS[mca::kKmax];
-  mca_status rc = eval_explicit(h, n, 0.0f, dS);   // proposals are within tfm_f16_range's bound
+  const mca_status rc = eval_explicit(h, n, 0.0f);    // proposals are within tfm_f16_range's bound
   if (rc != MCA_OK) return rc;
-  double S = 0.0;
-  rc = mca_loss(h, &S);
-  if (rc != MCA_OK) return rc;
-  S *= (double)h->N;
+  const double S = h->ev_host->tail.S;
   for (size_t k = 0; k < n; ++k) {
-    out[k].dS = out[k].valid ? dS[k] : std::nan("");
+    out[k] = h->ev_host->prop[k];
+    out[k].dS = out[k].valid ? h->ev_host->dS[k] : std::nan("");
     out[k].S = S;
   }
   return MCA_OK;
@@ -1672,8 +1669,6 @@ mca_status mca_create_transformer(const mca_tfm_spec* spec, const mca_domain* do
   h->trace = o.trace_cap > 0 ? reinterpret_cast<mca_trace_rec*>(base + M.trace) : nullptr;
   h->ex_idx = reinterpret_cast<unsigned int*>(base + M.ex_idx);
   h->ex_new = reinterpret_cast<float*>(base + M.ex_new);
-  h->ex_out = reinterpret_cast<double*>(base + M.ex_out);
-  h->prop = reinterpret_cast<mca_trace_rec*>(base + M.prop);
   h->tfm_img = h->tc ? reinterpret_cast<float*>(base + M.wimg) : nullptr;
   h->tfm_img16 = h->tc ? base + M.wimg16 : nullptr;
   h->tfm_Xmid = h->tc ? reinterpret_cast<float*>(base + M.Xmid) : nullptr;
@@ -1698,6 +1693,9 @@ mca_status mca_create_transformer(const mca_tfm_spec* spec, const mca_domain* do
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) return bail(fail(h, MCA_ERR_CUDA, "%s", cudaGetErrorString(e)));
   }
+  e = cudaMallocHost(reinterpret_cast<void**>(&h->ev_host), sizeof(*h->ev_host));
+  if (e != cudaSuccess) return bail(fail(h, MCA_ERR_OOM, "%s", cudaGetErrorString(e)));
+  std::memset(h->ev_host, 0, sizeof(*h->ev_host));
   rc = load_params(h, init_params, nullptr);
   if (rc != MCA_OK) return bail(rc);
   rc = resync(h);
@@ -1833,6 +1831,7 @@ void mca_destroy(mca_handle* h) {
     for (auto& e : b)
       if (e) cudaEventDestroy(e);
   if (h->pipe_host) cudaFreeHost(h->pipe_host);
+  if (h->ev_host) cudaFreeHost(h->ev_host);
   if (h->ws_owned && h->ws) cudaFree(h->ws);
   if (h->ftau) cudaFree(h->ftau);
   if (h->facc) cudaFree(h->facc);

@@ -282,7 +282,13 @@ __global__ void __launch_bounds__(kKmax) deep_decide_kernel(DeepArgs a) {
       }
     }
   }
-  if (a.n_explicit > 0) return;
+  if (a.n_explicit > 0) {
+    if (k == 0 && a.ex_tail != nullptr) {
+      a.ex_tail->S = a.st->S;
+      a.ex_tail->err = a.st->err;
+    }
+    return;
+  }
   const unsigned int ma = __ballot_sync(0xffffffffu, acc);
   const unsigned int mb = __ballot_sync(0xffffffffu, bad);
   const unsigned int mf = __ballot_sync(0xffffffffu, forced);

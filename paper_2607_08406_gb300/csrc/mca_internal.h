@@ -80,6 +80,12 @@ struct DevState {
   int pad;
 };
 
+// What an explicit evaluation reports beside its loss changes.
+struct ExTail {
+  double S;                  // loss sum of the cached state
+  int err;                   // first device-side error
+};
+
 // Arguments of the two-layer trial loop (input -> hidden -> output). The samples are split into NR
 // contiguous ranges of RS samples (RS a multiple of 8); CTA r owns range r.
 struct Mlp2Args {
@@ -128,6 +134,7 @@ struct Mlp2Args {
   const unsigned int* ex_idx;
   const float* ex_new;
   double* ex_out;
+  ExTail* ex_tail;           // nullable
 };
 
 // ------------------------------------------------------------------------------------------------
@@ -199,6 +206,7 @@ struct DeepArgs {
   const unsigned int* ex_idx;
   const float* ex_new;
   double* ex_out;
+  ExTail* ex_tail;           // nullable
   // tensor-core evaluation of candidate k < nscr with a dense chain (layer <= L-3): every field it
   // computes goes to scr[k * (L + 1) + m] (layer m: row j of the mutated layer, the full layers
   // after it; m = L: the per-sample losses), so that an accepted candidate's fields are adopted
@@ -270,6 +278,7 @@ struct TfmArgs {
   const unsigned int* ex_idx;
   const float* ex_new;
   double* ex_out;
+  ExTail* ex_tail;           // nullable
   int tc;                    // 1: the tensor-core kernels (mca_tfm_tc.cu) run the sequences
   float* wimg;               // their split-weight images (mca_tc_layout.h), tc = 1 only
   void* wimg16;              // the images with fp16 parts, kept beside them
@@ -418,8 +427,15 @@ struct mca_handle {
   int trace_cap = 0;
   unsigned int* ex_idx = nullptr;
   float* ex_new = nullptr;
-  double* ex_out = nullptr;
-  mca_trace_rec* prop = nullptr;         // [kKmax] proposals of mca_eval_trials
+  // explicit evaluations: pinned host memory that the candidates are copied from and the kernels
+  // write the results to
+  struct EvalHost {
+    unsigned int idx[mca::kKmax];
+    float new_w[mca::kKmax];
+    double dS[mca::kKmax];
+    mca_trace_rec prop[mca::kKmax];
+    mca::ExTail tail;
+  }* ev_host = nullptr;
   float* gimg = nullptr;                 // operand images of the tensor-core forward pass
   int nscr = 0;                          // tensor-core paths: candidate scratch slots
   std::vector<float*> scr;               // [nscr x (L + 1)] layer m of slot k (m = L: losses)

@@ -12,13 +12,18 @@ size_t mlp2_window_smem_bytes(int RS) { return window_smem_bytes(RS); }
 // Gaussian net of 1001 hidden neurons and 17.0 us for 2048 ReLU neurons under the Metropolis rule;
 // the variants (with the producers computing the rule's threshold) take 4.5 and 4.2 us. The
 // variants of each loss are compiled in their own file.
+static LoopKind loop_kind(const Mlp2Args& a) {
+  if (a.n_explicit > 0) return a.smem_records ? kLoopEval : kLoopTrial;
+  return a.window ? kLoopWindow : kLoopTrial;
+}
+
 static LoopFn pick_loop(const Mlp2Args& a) {
-  const bool window = a.window && a.n_explicit == 0;
+  const LoopKind kind = loop_kind(a);
   if (a.act2 == MCA_ACT_SIGMOID && a.loss == MCA_LOSS_MSE_ONEHOT)
-    return loop_variant_mse(window, a.act1, a.C);
+    return loop_variant_mse(kind, a.act1, a.C);
   if (a.act2 == MCA_ACT_IDENTITY && a.loss == MCA_LOSS_SOFTMAX_CE)
-    return loop_variant_ce(window, a.act1, a.C);
-  return window ? mlp2_window_loop<-1, -1, -1, 14> : mlp2_trial_loop<-1, -1, -1, -1>;
+    return loop_variant_ce(kind, a.act1, a.C);
+  return loop_kernel<-1, -1, -1, -1, 14>(kind);
 }
 
 size_t mlp2_loop_smem_bytes(const Mlp2Args& a) {
@@ -50,6 +55,8 @@ cudaError_t launch_mlp2_loop(const Mlp2Args& a, cudaStream_t s) {
   }
   Mlp2Args args = a;
   void* params[] = {&args};
+  if (loop_kind(a) == kLoopEval)     // no CTA waits for another
+    return cudaLaunchKernel((const void*)loop, dim3(a.NR), dim3(kEvalThreads), params, smem, s);
   return cudaLaunchCooperativeKernel((const void*)loop, dim3(a.NR), dim3(kLoopThreads), params,
                                      smem, s);
 }
