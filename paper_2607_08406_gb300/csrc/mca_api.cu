@@ -82,7 +82,10 @@ struct Layout {
 };
 
 bool is_deep(const std::vector<mca_layer>& layers) { return layers.size() > 2; }
-int deep_tiles(long long N) { return (int)((N + mca::kDeepTS - 1) / mca::kDeepTS); }
+// Samples per tile of the SIMT chain: 32 while 64 would leave SMs without a tile.
+int deep_tile_samples(long long N, int sms) {
+  return N <= (long long)mca::kDeepTS * sms ? mca::kDeepSmallTS : mca::kDeepTS;
+}
 
 // The dense chain runs on the tensor cores when every layer between the first and the output layer
 // is 256 x 256 (the kernel's fixed width).
@@ -92,7 +95,6 @@ bool deep_tc_ok(const std::vector<mca_layer>& layers) {
     if (layers[l].n_in != 256 || layers[l].n_out != 256) return false;
   return true;
 }
-int deep_tc_tiles(long long N) { return (int)((N + mca::kTcTS - 1) / mca::kTcTS); }
 
 // Accepted candidates are adopted from scratch slots written by their evaluation (deep and
 // Transformer tensor-core paths) unless the process sets MCA_ADOPT=0: then the commit kernels
@@ -171,7 +173,8 @@ Layout plan(const std::vector<mca_layer>& layers, long long N, int D, long long 
     L.ell = take(sizeof(float) * (size_t)Np);
     L.ctl = take(sizeof(mca::DeepCtl));
     L.z1 = L.srec = SIZE_MAX;
-    L.partial = take(sizeof(float) * (size_t)mca::kKmax * deep_tiles(N));
+    L.partial = take(sizeof(float) * (size_t)mca::kKmax *
+                     (size_t)((N + mca::kDeepSmallTS - 1) / mca::kDeepSmallTS));
   } else {
     L.ell = L.ctl = SIZE_MAX;
     L.z1 = take(sizeof(float) * (size_t)H * Np);
@@ -438,6 +441,7 @@ mca::DeepArgs deep_args(mca_handle* h) {
   a.D = h->D;
   a.C = h->C;
   a.ntiles = h->ntiles;
+  a.tile = h->tile;
   for (int l = 0; l < a.L; ++l) {
     const mca_layer& L = h->layers[l];
     a.n_in[l] = L.n_in;
@@ -991,7 +995,8 @@ mca_status mca_create(const mca_layer* layers, int32_t n_layers, int32_t loss,
   h->tc = h->deep && deep_tc_ok(ls);
   h->tc_f16 = h->tc;                 // fp16 operand parts: every layer of the dense chain is tanh
   for (size_t m = 1; m + 1 < ls.size(); ++m) h->tc_f16 = h->tc_f16 && ls[m].act == MCA_ACT_TANH;
-  h->ntiles = h->tc ? deep_tc_tiles(h->N) : deep_tiles(h->N);
+  h->tile = h->tc ? mca::kTcTS : deep_tile_samples(h->N, h->num_sms);
+  h->ntiles = (int)((h->N + h->tile - 1) / h->tile);
   if (!h->deep) {
     long long nnz = 0;
     mca_status s = count_nnz(data, h->stream, &nnz);

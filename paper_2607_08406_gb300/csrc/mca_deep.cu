@@ -9,7 +9,7 @@
 // change contributes exactly zero, and the commit writes exactly what the evaluation computed.
 //
 // Per batch the host launches three kernels:
-//   deep_eval     grid (K, tiles): CTA (k, t) runs candidate k's chain over tile t's kDeepTS samples,
+//   deep_eval     grid (K, tiles): CTA (k, t) runs candidate k's chain over tile t's samples (32 or 64),
 //                 the change matrix staying in shared memory from layer to layer, and writes one
 //                 partial loss change per (candidate, tile) -- a fixed computation, independent of K
 //   deep_decide   one CTA: fixed-order (compensated fp32) sums, lowest-index candidate with
@@ -25,18 +25,50 @@
 
 namespace mca {
 
-template <bool COMMIT>
+// Transfer function of a hidden layer: tanh in place, any other called.
+__device__ __forceinline__ float hidden_act(int act, float z, float g) {
+  return act == MCA_ACT_TANH ? tanh_exp(z) : act_call(act, z, g);
+}
+
+// Chunk of kDeepKC weights W[row][k0 ..] of one row into registers (0 past the last column).
+__device__ __forceinline__ void load_row_chunk(const float* W, int row, int K, int k0,
+                                               float (&w)[kDeepKC]) {
+  const float* src = W + (size_t)row * K + k0;
+  if (k0 + kDeepKC <= K && (K & 3) == 0) {
+#pragma unroll
+    for (int v = 0; v < kDeepKC / 4; ++v) {
+      const float4 w4 = *reinterpret_cast<const float4*>(src + 4 * v);
+      w[4 * v] = w4.x;
+      w[4 * v + 1] = w4.y;
+      w[4 * v + 2] = w4.z;
+      w[4 * v + 3] = w4.w;
+    }
+  } else {
+#pragma unroll
+    for (int v = 0; v < kDeepKC; ++v) w[v] = k0 + v < K ? src[v] : 0.0f;
+  }
+}
+
+// One CTA per (candidate, tile of 16 S samples): thread (ty, tx) computes R rows x S samples of a dense
+// layer, so that 16 R >= the widest layer. What bounds a chain is the latency of its layers, one after
+// another: the next weight chunk is in flight (in registers) while one is multiplied, a layer's
+// cached fields are loaded before its product, and small nets (fewer than one 64-sample tile per SM)
+// use tiles of 32. (With 256 rows and 64 samples whatever the widths, no load ahead of its use and
+// one thread per sample in the output layer, five layers of 100 on 3001 samples took 156 us per batch;
+// now 74 us.)
+template <bool COMMIT, int R, int S>
 __global__ void __launch_bounds__(kDeepThreads) deep_chain_kernel(DeepArgs a) {
+  constexpr int TS = 16 * S, ROWS = 16 * R;
   extern __shared__ __align__(16) float sm[];
-  float* Ds = sm;                                   // [kDeepMaxWidth][kDeepTS] activation changes
-  float* Ws = sm + kDeepMaxWidth * kDeepTS;         // [kDeepKC][kDeepMaxWidth] weight tile
+  float* Ds = sm;                                   // [kDeepMaxWidth][TS] activation changes
+  float* Ws = sm + kDeepMaxWidth * TS;              // two weight chunks [kDeepKC][ROWS]
   __shared__ DeepCand s_cand;
-  __shared__ float s_da[kDeepTS];
+  __shared__ float s_da[TS];
   __shared__ float s_red[32];
   const int tid = threadIdx.x;
   const int k = COMMIT ? 0 : blockIdx.x;
   const int tile = COMMIT ? blockIdx.x : blockIdx.y;
-  const int n0 = tile * kDeepTS;
+  const int n0 = tile * TS;
   if (COMMIT && a.ctl->kstar < 0) return;
   if (tid == 0) s_cand = COMMIT ? a.ctl->acc : deep_candidate(a, k);
   __syncthreads();
@@ -51,12 +83,12 @@ __global__ void __launch_bounds__(kDeepThreads) deep_chain_kernel(DeepArgs a) {
   float dl = 0.0f;
 
   // ---- row j of layer l
-  if (tid < kDeepTS) {
+  if (tid < TS) {
     const int n = n0 + tid;
     float da = 0.0f;
     if (n < N) {
       const float v = l == 0 ? a.XT[(size_t)i * Np + n]
-                             : act_rt(a.act[l - 1], a.Z[l - 1][(size_t)i * Np + n], a.g[l - 1]);
+                             : hidden_act(a.act[l - 1], a.Z[l - 1][(size_t)i * Np + n], a.g[l - 1]);
       float* zp = a.Z[l] + (size_t)j * Np + n;
       const float z = *zp;
       const float zn = fmaf(c.delta, v, z);
@@ -70,7 +102,7 @@ __global__ void __launch_bounds__(kDeepThreads) deep_chain_kernel(DeepArgs a) {
           if (q == j) zz[q] = zn;
         dl = out_delta<COMMIT>(a, n, zz, zn != z);
       } else {
-        da = act_rt(a.act[l], zn, a.g[l]) - act_rt(a.act[l], z, a.g[l]);
+        da = hidden_act(a.act[l], zn, a.g[l]) - hidden_act(a.act[l], z, a.g[l]);
         if (COMMIT) *zp = zn;
       }
     }
@@ -84,7 +116,7 @@ __global__ void __launch_bounds__(kDeepThreads) deep_chain_kernel(DeepArgs a) {
     const float* W1 = a.w[m1];
     const int K1 = a.n_in[m1];
     if (m1 == L - 1) {
-      if (tid < kDeepTS) {
+      if (tid < TS) {
         const int n = n0 + tid;
         const float da = s_da[tid];
         if (n < N && da != 0.0f) {
@@ -104,124 +136,167 @@ __global__ void __launch_bounds__(kDeepThreads) deep_chain_kernel(DeepArgs a) {
         }
       }
     } else {
-      const int M = a.n_out[m1];
-      for (int e = tid; e < M * kDeepTS; e += kDeepThreads) {
-        const int r = e / kDeepTS, t = e - r * kDeepTS, n = n0 + t;
-        const float da = s_da[t];
-        float d = 0.0f;
-        if (n < N && da != 0.0f) {
-          float* zp = a.Z[m1] + (size_t)r * Np + n;
-          const float zo = *zp;
-          const float zn = fmaf(W1[(size_t)r * K1 + j], da, zo);
-          if (COMMIT) *zp = zn;
-          d = act_rt(a.act[m1], zn, a.g[m1]) - act_rt(a.act[m1], zo, a.g[m1]);
+      const int M = a.n_out[m1], act1 = a.act[m1];
+      const float g1 = a.g[m1];
+      float* Z1 = a.Z[m1];
+#pragma unroll 1
+      for (int e0 = tid; e0 < M * TS; e0 += 4 * kDeepThreads) {
+        float zo[4], w[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {               // n < Np: always in the arrays
+          const int e = e0 + u * kDeepThreads, r = min(e / TS, M - 1);
+          zo[u] = Z1[(size_t)r * Np + n0 + e % TS];
+          w[u] = W1[(size_t)r * K1 + j];
         }
-        Ds[r * kDeepTS + t] = d;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int e = e0 + u * kDeepThreads, r = e / TS, t = e % TS, n = n0 + t;
+          if (e >= M * TS) break;
+          const float da = s_da[t];
+          float d = 0.0f;
+          if (n < N && da != 0.0f) {
+            const float zn = fmaf(w[u], da, zo[u]);
+            if (COMMIT) Z1[(size_t)r * Np + n] = zn;
+            d = hidden_act(act1, zn, g1) - hidden_act(act1, zo[u], g1);
+          }
+          Ds[e] = d;
+        }
       }
       __syncthreads();
 
       // ---- layers l+2 .. L-2: Z'_m = Z_m + W_m D, D <- f(Z'_m) - f(Z_m)
       const int ty = tid >> 4, tx = tid & 15;
+      const int wrow = tid < ROWS ? tid : 0;         // the row whose weights this thread stages
       for (int m = l + 2; m < L - 1; ++m) {
         const float* Wm = a.w[m];
         const int Mm = a.n_out[m], Km = a.n_in[m];
-        float acc[16][4];
+        float* Zm = a.Z[m];
+        constexpr bool kAhead = R * S <= 32;         // registers for the cached fields meanwhile
+        float zf[kAhead ? R : 1][S];
+        if (kAhead) {
 #pragma unroll
-        for (int q = 0; q < 16; ++q)
+          for (int q = 0; q < R; ++q)
 #pragma unroll
-          for (int cc = 0; cc < 4; ++cc) acc[q][cc] = 0.0f;
+            for (int cc = 0; cc < S; ++cc)
+              zf[kAhead ? q : 0][cc] =
+                  Zm[(size_t)min(ty * R + q, Mm - 1) * Np + n0 + tx * S + cc];
+        }
+        float acc[R][S];
+#pragma unroll
+        for (int q = 0; q < R; ++q)
+#pragma unroll
+          for (int cc = 0; cc < S; ++cc) acc[q][cc] = 0.0f;
+        float wn[kDeepKC];
+        const bool stage = tid < Mm;                 // Mm <= ROWS
+        if (stage) load_row_chunk(Wm, wrow, Km, 0, wn);
+        int buf = 0;
+#pragma unroll 1
         for (int k0 = 0; k0 < Km; k0 += kDeepKC) {
           const int kn = min(kDeepKC, Km - k0);
-          if (tid < Mm) {
-            const float* src = Wm + (size_t)tid * Km + k0;
-            if (kn == kDeepKC && (Km & 3) == 0) {
+          float* Wb = Ws + buf * kDeepKC * ROWS;
+          if (stage) {
 #pragma unroll
-              for (int v4 = 0; v4 < kDeepKC / 4; ++v4) {
-                const float4 w4 = *reinterpret_cast<const float4*>(src + 4 * v4);
-                Ws[(4 * v4 + 0) * kDeepMaxWidth + tid] = w4.x;
-                Ws[(4 * v4 + 1) * kDeepMaxWidth + tid] = w4.y;
-                Ws[(4 * v4 + 2) * kDeepMaxWidth + tid] = w4.z;
-                Ws[(4 * v4 + 3) * kDeepMaxWidth + tid] = w4.w;
+            for (int v = 0; v < kDeepKC; ++v) Wb[v * ROWS + tid] = wn[v];
+          }
+          __syncthreads();
+          if (stage && k0 + kDeepKC < Km) load_row_chunk(Wm, wrow, Km, k0 + kDeepKC, wn);
+          if (ty * R < Mm) {
+#pragma unroll 4
+            for (int kk = 0; kk < kn; ++kk) {
+              float b[S], av[R];
+              const float* dr = &Ds[(k0 + kk) * TS + tx * S];
+              if constexpr (S == 4) {
+                const float4 v = *reinterpret_cast<const float4*>(dr);
+                b[0] = v.x;
+                b[1] = v.y;
+                b[2] = v.z;
+                b[3] = v.w;
+              } else {
+                const float2 v = *reinterpret_cast<const float2*>(dr);
+                b[0] = v.x;
+                b[1] = v.y;
               }
-            } else {
-              for (int kk = 0; kk < kn; ++kk) Ws[kk * kDeepMaxWidth + tid] = src[kk];
+              const float* wr = &Wb[kk * ROWS + ty * R];
+#pragma unroll
+              for (int v4 = 0; v4 < R / 4; ++v4) {
+                const float4 w4 = *reinterpret_cast<const float4*>(wr + 4 * v4);
+                av[4 * v4] = w4.x;
+                av[4 * v4 + 1] = w4.y;
+                av[4 * v4 + 2] = w4.z;
+                av[4 * v4 + 3] = w4.w;
+              }
+#pragma unroll
+              for (int q = 0; q < R; ++q)
+#pragma unroll
+                for (int cc = 0; cc < S; ++cc) acc[q][cc] = fmaf(av[q], b[cc], acc[q][cc]);
             }
           }
-          __syncthreads();
-          for (int kk = 0; kk < kn; ++kk) {
-            const float4 b = *reinterpret_cast<const float4*>(&Ds[(k0 + kk) * kDeepTS + tx * 4]);
-            const float* wr = &Ws[kk * kDeepMaxWidth + ty * 16];
-            float av[16];
-#pragma unroll
-            for (int v4 = 0; v4 < 4; ++v4) {
-              const float4 w4 = *reinterpret_cast<const float4*>(wr + 4 * v4);
-              av[4 * v4 + 0] = w4.x;
-              av[4 * v4 + 1] = w4.y;
-              av[4 * v4 + 2] = w4.z;
-              av[4 * v4 + 3] = w4.w;
-            }
-#pragma unroll
-            for (int q = 0; q < 16; ++q) {
-              acc[q][0] = fmaf(av[q], b.x, acc[q][0]);
-              acc[q][1] = fmaf(av[q], b.y, acc[q][1]);
-              acc[q][2] = fmaf(av[q], b.z, acc[q][2]);
-              acc[q][3] = fmaf(av[q], b.w, acc[q][3]);
-            }
-          }
-          __syncthreads();
+          buf ^= 1;
         }
-        // epilogue: new fields and the next change matrix (rows >= Mm are never read)
-        float* Zm = a.Z[m];
+        __syncthreads();                             // every thread is done with Ds
+        // new fields and the next change matrix (rows >= Mm are never read)
+        const int actm = a.act[m];
+        const float gm = a.g[m];
 #pragma unroll
-        for (int q = 0; q < 16; ++q) {
-          const int r = ty * 16 + q;
+        for (int q = 0; q < R; ++q) {
+          const int r = ty * R + q;
           if (r < Mm) {
-            const int t0 = tx * 4;
-            const float4 zo4 = *reinterpret_cast<const float4*>(Zm + (size_t)r * Np + n0 + t0);
-            const float zo[4] = {zo4.x, zo4.y, zo4.z, zo4.w};
 #pragma unroll
-            for (int cc = 0; cc < 4; ++cc) {
-              const int n = n0 + t0 + cc;
-              const float zn = zo[cc] + acc[q][cc];
+            for (int cc = 0; cc < S; ++cc) {
+              const int t = tx * S + cc, n = n0 + t;
+              const float zo = kAhead ? zf[kAhead ? q : 0][cc] : Zm[(size_t)r * Np + n];
+              const float zn = zo + acc[q][cc];
               float d = 0.0f;
-              if (n < N && zn != zo[cc]) {
-                d = act_rt(a.act[m], zn, a.g[m]) - act_rt(a.act[m], zo[cc], a.g[m]);
+              if (n < N && zn != zo) {
+                d = hidden_act(actm, zn, gm) - hidden_act(actm, zo, gm);
                 if (COMMIT) Zm[(size_t)r * Np + n] = zn;
               }
-              Ds[r * kDeepTS + t0 + cc] = d;
+              Ds[r * TS + t] = d;
             }
           }
         }
         __syncthreads();
       }
 
-      // ---- output layer: Z'_{L-1} = Z_{L-1} + W_{L-1} D, loss
+      // ---- output layer: Z'_{L-1} = Z_{L-1} + W_{L-1} D, loss. The features are cut into
+      // 256 / TS parts per sample, added in part order.
       {
+        constexpr int PARTS = kDeepThreads / TS;
         const int mo = L - 1;
         const int Ko = a.n_in[mo];
         const float* Wo = a.w[mo];
-        for (int e = tid; e < a.C * Ko; e += kDeepThreads) Ws[e] = Wo[e];
-        __syncthreads();
-        if (tid < kDeepTS) {
-          const int n = n0 + tid;
-          if (n < N) {
-            float zz[kMaxC];
-            bool changed = false;
+        const int t = tid % TS, p = tid / TS, n = n0 + t;
+        const int per = (Ko + PARTS - 1) / PARTS;
+        float s[kMaxC];
 #pragma unroll
-            for (int q = 0; q < kMaxC; ++q) {
-              if (q < a.C) {
-                float s = 0.0f;
-                const float* wq = Ws + q * Ko;
-                for (int kk = 0; kk < Ko; ++kk) s = fmaf(wq[kk], Ds[kk * kDeepTS + tid], s);
-                const float zo = a.Z[mo][(size_t)q * Np + n];
-                zz[q] = zo + s;
-                changed |= zz[q] != zo;
-              } else {
-                zz[q] = 0.0f;
-              }
+        for (int q = 0; q < kMaxC; ++q) s[q] = 0.0f;
+#pragma unroll 2
+        for (int kk = p * per; kk < min(Ko, p * per + per); ++kk) {
+          const float d = Ds[kk * TS + t];
+#pragma unroll
+          for (int q = 0; q < kMaxC; ++q)
+            if (q < a.C) s[q] = fmaf(__ldg(Wo + (size_t)q * Ko + kk), d, s[q]);
+        }
+        __syncthreads();                             // Ds takes the parts
+#pragma unroll
+        for (int q = 0; q < kMaxC; ++q) Ds[(p * kMaxC + q) * TS + t] = s[q];
+        __syncthreads();
+        if (p == 0 && n < N) {
+          float zz[kMaxC];
+          bool changed = false;
+#pragma unroll
+          for (int q = 0; q < kMaxC; ++q) {
+            zz[q] = 0.0f;
+            if (q < a.C) {
+              float v = 0.0f;
+#pragma unroll
+              for (int u = 0; u < PARTS; ++u) v += Ds[(u * kMaxC + q) * TS + t];
+              const float zo = a.Z[mo][(size_t)q * Np + n];
+              zz[q] = zo + v;
+              changed |= zz[q] != zo;
             }
-            dl = out_delta<COMMIT>(a, n, zz, changed);
           }
+          dl = out_delta<COMMIT>(a, n, zz, changed);
         }
       }
     }
@@ -386,18 +461,36 @@ __global__ void deep_losses_kernel(DeepArgs a) {
   a.ell[n] = sample_loss<-1, -1, kMaxC>(zz, a.C, a.y[n], a.g[Lo], a.act[Lo], a.loss);
 }
 
-static size_t chain_smem() {
-  return sizeof(float) * (size_t)(kDeepMaxWidth * kDeepTS + kDeepKC * kDeepMaxWidth);
+// The SIMT chain's variant: rows per thread from the widest layer behind the first, samples per
+// thread from the handle's tile.
+using ChainFn = void (*)(DeepArgs);
+
+template <bool COMMIT, int S>
+static ChainFn chain_rows(int width, size_t* smem) {
+  const int R = width <= 64 ? 4 : width <= 128 ? 8 : 16;
+  *smem = sizeof(float) * (size_t)(kDeepMaxWidth * 16 * S + 2 * kDeepKC * 16 * R);
+  return R == 4   ? deep_chain_kernel<COMMIT, 4, S>
+         : R == 8 ? deep_chain_kernel<COMMIT, 8, S>
+                  : deep_chain_kernel<COMMIT, 16, S>;
+}
+
+template <bool COMMIT>
+static cudaError_t chain_variant(const DeepArgs& a, ChainFn* fn, size_t* smem) {
+  int width = 0;
+  for (int m = 1; m < a.L - 1; ++m) width = std::max(width, a.n_out[m]);
+  *fn = a.tile == 32 ? chain_rows<COMMIT, 2>(width, smem) : chain_rows<COMMIT, 4>(width, smem);
+  return cudaFuncSetAttribute((const void*)*fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)*smem);
 }
 
 cudaError_t launch_deep_eval(const DeepArgs& a, cudaStream_t s) {
   if (a.tc) return launch_deep_eval_tc(a, s);
   const int Kb = a.n_explicit > 0 ? a.n_explicit : a.Kb;
-  cudaError_t e = cudaFuncSetAttribute((const void*)deep_chain_kernel<false>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)chain_smem());
+  ChainFn fn;
+  size_t smem;
+  cudaError_t e = chain_variant<false>(a, &fn, &smem);
   if (e != cudaSuccess) return e;
-  deep_chain_kernel<false><<<dim3(Kb, a.ntiles), kDeepThreads, chain_smem(), s>>>(a);
+  fn<<<dim3(Kb, a.ntiles), kDeepThreads, smem, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -408,11 +501,11 @@ cudaError_t launch_deep_decide(const DeepArgs& a, cudaStream_t s) {
 
 cudaError_t launch_deep_commit(const DeepArgs& a, cudaStream_t s) {
   if (a.tc) return launch_deep_commit_tc(a, s);
-  cudaError_t e = cudaFuncSetAttribute((const void*)deep_chain_kernel<true>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)chain_smem());
+  ChainFn fn;
+  size_t smem;
+  cudaError_t e = chain_variant<true>(a, &fn, &smem);
   if (e != cudaSuccess) return e;
-  deep_chain_kernel<true><<<a.ntiles, kDeepThreads, chain_smem(), s>>>(a);
+  fn<<<a.ntiles, kDeepThreads, smem, s>>>(a);
   return cudaGetLastError();
 }
 

@@ -143,7 +143,8 @@ struct Mlp2Args {
 // from l+2 on as  Z'_m = Z_m + W_m (f(Z'_{m-1}) - f(Z_{m-1}))  over tiles of kDeepTS samples.
 // ------------------------------------------------------------------------------------------------
 constexpr int kMaxLayers = 32;
-constexpr int kDeepTS = 64;        // samples per tile
+constexpr int kDeepTS = 64;        // samples per tile of the SIMT chain, or
+constexpr int kDeepSmallTS = 32;   //   of small nets (deep_tile_samples)
 constexpr int kTcTS = 128;         // samples per tile of the tensor-core chain (one MMA M)
 constexpr int kDeepThreads = 256;
 constexpr int kDeepMaxWidth = 256; // widths of the layers inside the dense chain
@@ -178,6 +179,7 @@ struct DeepArgs {
   float* Z[kMaxLayers];      // [n_out[l] x Np] fields of layer l; Z[L-1] are the output fields
   float* whi[kMaxLayers];    // tensor-core chain: tf32(W_m) and tf32(W_m - tf32(W_m)) of the
                              //   256 x 256 layers 1 .. L-2 as stage images (null otherwise)
+  int tile;                  // samples per tile
   int tc;                    // 1: dense chain on the tensor cores, tiles of kTcTS samples
   int tc_f16;                // tc = 1: operands as fp16 parts (tanh layers), else tf32 parts
   float tc_wscale;           // tc_f16: power of two that scales the dense weights to at most 2^15
@@ -417,7 +419,7 @@ struct mca_handle {
   std::vector<float*> whi;           // split-weight images of layers 1 .. L-2 (tensor-core chain)
   float* ell = nullptr;
   mca::DeepCtl* ctl = nullptr;
-  int ntiles = 0;
+  int ntiles = 0, tile = 0;          // deep: tiles, and their samples
   float* partial = nullptr;
   unsigned long long* accum = nullptr;
   int NR = 0, RS = 0, SUB = 0, smem_records = 0, window = 0;
