@@ -845,8 +845,8 @@ mca_status run_tfm_pipelined(mca_handle* h, mca::TfmArgs ta, uint64_t n_trials) 
   auto launch = [&](int i) -> mca_status {
     const int p = i & 1;
     const int Kw = h->opt.fixed_K ? h->opt.K
-                                  : mca::batch_width_cost(h->rate_acc, h->rate_trials,
-                                                          mca::kBatchCostTfm, h->opt.K);
+                                  : mca::batch_width_waves(h->rate_acc, h->rate_trials, h->wave,
+                                                           mca::kWaveTailTfm, h->opt.K);
     ta.Kb = (int)std::min<uint64_t>(n_trials, (uint64_t)Kw);
     ta.f16 = tfm_f16_range(h) ? 1 : 0;
     ta.ctl = h->ctl2 + p;
@@ -1140,6 +1140,9 @@ mca_status mca_create(const mca_layer* layers, int32_t n_layers, int32_t loss,
   if (ds.err == MCA_ERR_TIMEOUT)
     return bail(fail(h, MCA_ERR_TIMEOUT, "device-side wait timed out in the forward pass"));
   if (!std::isfinite(ds.S)) return bail(fail(h, MCA_ERR_NUMERIC, "initial loss is not finite"));
+  if (h->deep)
+    h->wave = (float)h->ntiles /
+              (float)(h->num_sms * mca::deep_eval_ctas_per_sm(deep_args(h)));
 #undef TRY
 #undef CTRY
   *out = h;
@@ -1166,10 +1169,10 @@ mca_status mca_run(mca_handle* h, uint64_t n_trials, uint64_t seed, mca_run_stat
     while (remaining > 0) {
       NvtxRange nv_batch(h->tfm ? "mca batch (transformer)" : "mca batch (deep)");
       const int Kw = h->opt.fixed_K ? h->opt.K
-                                    : mca::batch_width_cost(h->rate_acc, h->rate_trials,
-                                                            h->tfm ? mca::kBatchCostTfm
-                                                                   : mca::kBatchCostDeep,
-                                                            h->opt.K);
+                                    : mca::batch_width_waves(h->rate_acc, h->rate_trials, h->wave,
+                                                             h->tfm ? mca::kWaveTailTfm
+                                                                    : mca::kWaveTailDeep,
+                                                             h->opt.K);
       uint64_t kb = std::min<uint64_t>(remaining, (uint64_t)Kw);
       if (R > 0) kb = std::min<uint64_t>(kb, R - h->tau % R);
       if (!h->ev[0]) {
@@ -1709,6 +1712,11 @@ mca_status mca_create_transformer(const mca_tfm_spec* spec, const mca_domain* do
   rc = read_state(h, &ds);
   if (rc != MCA_OK) return bail(rc);
   if (!std::isfinite(ds.S)) return bail(fail(h, MCA_ERR_NUMERIC, "initial loss is not finite"));
+  {
+    const mca::TfmArgs a = tfm_args(h);
+    h->wave = (float)(h->tc ? a.B / 2 : a.B) /
+              (float)(h->num_sms * mca::tfm_eval_ctas_per_sm(a));
+  }
   *out = h;
   return MCA_OK;
 }

@@ -494,6 +494,20 @@ cudaError_t launch_deep_eval(const DeepArgs& a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+// Evaluation CTAs that run at the same time on one SM.
+int deep_eval_ctas_per_sm(const DeepArgs& a) {
+  if (a.tc) return 1;
+  ChainFn fn;
+  size_t smem;
+  int occ = 0;
+  if (chain_variant<false>(a, &fn, &smem) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, kDeepThreads, smem) != cudaSuccess) {
+    cudaGetLastError();
+    return 1;
+  }
+  return std::max(1, occ);
+}
+
 cudaError_t launch_deep_decide(const DeepArgs& a, cudaStream_t s) {
   deep_decide_kernel<<<1, kKmax, 0, s>>>(a);
   return cudaGetLastError();

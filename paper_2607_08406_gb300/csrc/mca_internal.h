@@ -28,12 +28,7 @@ constexpr float kWidthMlp2 = 2.0f;
 // Host-driven batches (deep nets, the Transformer): a batch of K candidates consumes
 // (1 - (1 - p)^K) / p trials on average and costs about r + K candidate evaluations, r being its
 // fixed part (decision, adoption or commit, launch gaps, the last partial wave of CTAs). The width
-// maximises trials per cost. r was fitted to fixed-width runs on GB300 (batch time against K):
-// about 1.9 candidate-times for the 24 x 256 chain at N = 10000, 0.5 for the d_model 128
-// Transformer on 256 sequences.
-constexpr float kBatchCostDeep = 1.9f;
-constexpr float kBatchCostTfm = 0.5f;
-
+// maximises trials per cost.
 inline int batch_width_cost(float acc, float trials, float r, int K) {
   const double p = ((double)acc + 0.5) / ((double)trials + 1.0);
   double qk = 1.0, best = -1.0;
@@ -41,6 +36,35 @@ inline int batch_width_cost(float acc, float trials, float r, int K) {
   for (int k = 1; k <= K; ++k) {
     qk *= 1.0 - p;
     const double v = (1.0 - qk) / ((double)r + (double)k);
+    if (v > best) {
+      best = v;
+      kb = k;
+    }
+  }
+  return kb;
+}
+
+// The same with the grid's size: a candidate's CTAs fill the fraction u of the GPU, so that candidates
+// cost nothing more until the GPU is full, and then u each (a: what the last, partial wave costs).
+// In units of one CTA's chain: r + max(1, a + K u). Measured on GB300 with fixed widths: for 24 x 256
+// tanh nets on 10000 samples (u = 0.52) 177, 283, 362, 431, 575 us per batch at K = 1, 2, 3, 4, 6, that
+// is 135 (0.3 + max(1, 0.7 + K u)) within 5 %; for the d_model 128 Transformer on 256 sequences (u = 0.84) 116,
+// 200, 274, 350, 491, that is 89 (0.3 + max(1, 0.15 + K u)). Small nets (u < 1/4) gain most: at an
+// acceptance of one half they consume 1.9 trials per batch instead of 1 to 1.5.
+constexpr float kWaveFixed = 0.3f;
+constexpr float kWaveTailDeep = 0.7f;
+constexpr float kWaveTailTfm = 0.15f;
+
+inline int batch_width_waves(float acc, float trials, float u, float tail, int K) {
+  if (u > 1.0f) return batch_width_cost(acc, trials, (kWaveFixed + tail) / u, K);
+  const double p = ((double)acc + 0.5) / ((double)trials + 1.0);
+  double qk = 1.0, best = -1.0;
+  int kb = 1;
+  for (int k = 1; k <= K; ++k) {
+    qk *= 1.0 - p;
+    const double fill = (double)k * (double)u;
+    const double t = (double)kWaveFixed + (fill <= 1.0 ? 1.0 : (double)tail + fill);
+    const double v = (1.0 - qk) / t;
     if (v > best) {
       best = v;
       kb = k;
@@ -218,6 +242,7 @@ struct DeepArgs {
 };
 
 cudaError_t launch_deep_eval(const DeepArgs& a, cudaStream_t s);    // grid (Kb, ntiles)
+int deep_eval_ctas_per_sm(const DeepArgs& a);
 cudaError_t launch_deep_decide(const DeepArgs& a, cudaStream_t s);  // one CTA
 cudaError_t launch_deep_commit(const DeepArgs& a, cudaStream_t s);  // grid ntiles
 cudaError_t launch_deep_forward_layer(const DeepArgs& a, int l, cudaStream_t s);
@@ -300,6 +325,7 @@ struct TfmArgs {
 };
 
 size_t tfm_smem_bytes(int T, int d, int dh, int V);
+int tfm_eval_ctas_per_sm(const TfmArgs& a);
 cudaError_t launch_tfm_eval(const TfmArgs& a, cudaStream_t s);      // grid (Kb, B)
 cudaError_t launch_tfm_decide(const TfmArgs& a, cudaStream_t s);    // one CTA
 cudaError_t launch_tfm_commit(const TfmArgs& a, cudaStream_t s);    // grid B
@@ -420,6 +446,7 @@ struct mca_handle {
   float* ell = nullptr;
   mca::DeepCtl* ctl = nullptr;
   int ntiles = 0, tile = 0;          // deep: tiles, and their samples
+  float wave = 1.0f;                 // host-driven batches: CTAs per candidate / CTAs that run at once
   float* partial = nullptr;
   unsigned long long* accum = nullptr;
   int NR = 0, RS = 0, SUB = 0, smem_records = 0, window = 0;

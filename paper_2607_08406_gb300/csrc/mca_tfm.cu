@@ -639,6 +639,21 @@ static cudaError_t launch_seq(const TfmArgs& a, dim3 grid, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+// Evaluation CTAs that run at the same time on one SM.
+int tfm_eval_ctas_per_sm(const TfmArgs& a) {
+  int occ = 0;
+  if (a.tc) return 1;
+  if (cudaFuncSetAttribute((const void*)tfm_seq_kernel<kTfmEval>,
+                           cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)a.smem) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, tfm_seq_kernel<kTfmEval>, kTfmThreads,
+                                                    a.smem) != cudaSuccess) {
+    cudaGetLastError();
+    return 1;
+  }
+  return std::max(1, occ);
+}
+
 cudaError_t launch_tfm_eval(const TfmArgs& a, cudaStream_t s) {
   if (a.tc) return a.f16 ? launch_tfm_f16(a, kTfmEval, s) : launch_tfm_tc_eval(a, s);
   const int Kb = a.n_explicit > 0 ? a.n_explicit : a.Kb;
