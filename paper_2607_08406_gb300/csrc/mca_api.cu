@@ -96,20 +96,25 @@ bool deep_tc_ok(const std::vector<mca_layer>& layers) {
   return true;
 }
 
-// Accepted candidates are adopted from scratch slots written by their evaluation (deep and
-// Transformer tensor-core paths) unless the process sets MCA_ADOPT=0: then the commit kernels
+// Accepted candidates are adopted from scratch slots written by their evaluation unless the process sets MCA_ADOPT=0: then the commit kernels
 // recompute them. Read by the workspace-size calls and creation, so it must not change between them.
 bool adopt_enabled() {
   const char* e = std::getenv("MCA_ADOPT");
   return !(e && std::strcmp(e, "0") == 0);
 }
 
-// Candidate scratch slots of the deep tensor-core path (min(K, kDeepScrSlots)); none elsewhere.
-int deep_scratch_slots(const std::vector<mca_layer>& layers, int K) {
-  return deep_tc_ok(layers) && adopt_enabled() ? std::min(K, mca::kDeepScrSlots) : 0;
-}
-
 int pad_n(long long N) { return (int)((N + 127) / 128 * 128); }
+
+// Candidate scratch slots of deep nets: min(K, kDeepScrSlots), on the SIMT chain (any width of the
+// first layer) within kSimtScrBytes.
+int deep_scratch_slots(const std::vector<mca_layer>& layers, long long N, int K) {
+  if (!is_deep(layers) || !adopt_enabled()) return 0;
+  const size_t slots = (size_t)std::min(K, mca::kDeepScrSlots);
+  if (deep_tc_ok(layers)) return (int)slots;
+  size_t rows = 1;
+  for (const auto& ly : layers) rows += (size_t)ly.n_out;
+  return (int)std::min(slots, mca::kSimtScrBytes / (sizeof(float) * rows * (size_t)pad_n(N)));
+}
 
 // The forward pass (creation, resync) computes the fields of a layer on the tensor cores
 // (mca_gemm_tc.cu) when its shape allows, unless the process sets MCA_FORWARD_TENSOR_CORES=0 (then
@@ -710,13 +715,15 @@ bool tfm_use_tc(const mca_tfm_spec& t, long long B) {
   return mca::tfm_tc_shape_ok(t.ctx, t.d_model, t.n_head, t.d_ff, t.vocab, B);
 }
 
-// Scratch slots of the tensor-core Transformer kernels: candidate k < nscr of a batch writes its
-// residual streams (X and the mid streams) and sequence losses to slot k, min(K, kTfmScrSlots)
-// slots within 8 GiB.
+// Residual streams of a Transformer: X, and the tensor-core kernels' mid streams.
+int tfm_streams(const mca_tfm_spec& t, bool tc) { return (tc ? 2 : 1) * t.n_layer + 1; }
+
+// Scratch slots of the Transformer kernels: candidate k < nscr of a batch writes its residual streams
+// and sequence losses to slot k, min(K, kTfmScrSlots) slots within 8 GiB (SIMT: kSimtScrBytes).
 int tfm_scratch_slots(const mca_tfm_spec& t, long long B, int K, bool tc) {
-  if (!tc || !adopt_enabled()) return 0;
-  const size_t slot = sizeof(float) * ((size_t)(2 * t.n_layer + 1) * B * t.ctx * t.d_model + B);
-  const size_t cap = (size_t)8 << 30;
+  if (!adopt_enabled()) return 0;
+  const size_t slot = sizeof(float) * ((size_t)tfm_streams(t, tc) * B * t.ctx * t.d_model + B);
+  const size_t cap = tc ? (size_t)8 << 30 : mca::kSimtScrBytes;
   return (int)std::min<size_t>((size_t)std::min(K, mca::kTfmScrSlots), cap / slot);
 }
 
@@ -744,7 +751,7 @@ TfmMem tfm_plan(const mca_tfm_spec& t, long long B, int trace_cap, bool tc, int 
   M.wimg16 = tc ? take(mca::tfm_f16_image_bytes(t.d_ff, t.n_layer)) : 0;
   M.Xmid = take(tc ? sizeof(float) * (size_t)t.n_layer * B * t.ctx * t.d_model : 0);
   M.nscr = tfm_scratch_slots(t, B, K, tc);
-  M.scrX = take(sizeof(float) * (size_t)M.nscr * (2 * t.n_layer + 1) * B * t.ctx * t.d_model);
+  M.scrX = take(sizeof(float) * (size_t)M.nscr * tfm_streams(t, tc) * B * t.ctx * t.d_model);
   M.scr_ell = take(sizeof(float) * (size_t)M.nscr * B);
   M.ctl2 = take(2 * sizeof(mca::DeepCtl));
   M.tau_dev = take(sizeof(unsigned long long));
@@ -914,7 +921,8 @@ mca_status mca_workspace_size(const mca_layer* layers, int32_t n_layers, int32_t
   if (!bytes) return fail(nullptr, MCA_ERR_INVALID, "bytes is NULL");
   const mca_options o = opt ? *opt : default_options();
   if (is_deep(ls)) {
-    *bytes = plan(ls, data->n, data->d, 0, o.trace_cap, 0, deep_scratch_slots(ls, o.K)).total;
+    *bytes = plan(ls, data->n, data->d, 0, o.trace_cap, 0, deep_scratch_slots(ls, data->n, o.K))
+                 .total;
     return MCA_OK;
   }
   long long nnz = 0;
@@ -923,7 +931,7 @@ mca_status mca_workspace_size(const mca_layer* layers, int32_t n_layers, int32_t
   Ranges R;
   rc = choose_ranges(ls, loss, data->n, o.grid, &R);
   if (rc != MCA_OK) return rc;
-  *bytes = plan(ls, data->n, data->d, nnz, o.trace_cap, R.NR, deep_scratch_slots(ls, o.K)).total;
+  *bytes = plan(ls, data->n, data->d, nnz, o.trace_cap, R.NR, 0).total;
   return MCA_OK;
 }
 
@@ -1019,7 +1027,7 @@ mca_status mca_create(const mca_layer* layers, int32_t n_layers, int32_t loss,
     h->smem_records = R.smem_records;
     h->window = R.window;
   }
-  h->nscr = h->deep ? deep_scratch_slots(ls, o.K) : 0;
+  h->nscr = deep_scratch_slots(ls, h->N, o.K);
   const Layout L = plan(ls, h->N, h->D, h->nnz, o.trace_cap, h->NR, h->nscr);
   if (o.workspace) {
     if (o.workspace_bytes < L.total)
@@ -1188,9 +1196,9 @@ mca_status mca_run(mca_handle* h, uint64_t n_trials, uint64_t seed, mca_run_stat
         CUDA_TRY(h, mca::launch_tfm_eval(ta, h->stream));
         CUDA_TRY(h, cudaEventRecord(h->ev[1], h->stream));
         CUDA_TRY(h, mca::launch_tfm_decide(ta, h->stream));
-        // the commit kernel recomputes an accepted candidate beyond the scratch slots (and
-        // returns at once otherwise); then the accepted weight's image entry and, for a
-        // candidate with a slot, its adoption
+        // the commit kernel recomputes an accepted candidate beyond the scratch slots (SIMT: or
+        // copies its slot); then, on the tensor cores, the accepted weight's image entry and, for
+        // a candidate with a slot, its adoption
         CUDA_TRY(h, mca::launch_tfm_commit(ta, h->stream));
         if (ta.tc) {
           CUDA_TRY(h, mca::launch_tfm_tc_adopt(ta, h->stream));
@@ -1204,8 +1212,8 @@ mca_status mca_run(mca_handle* h, uint64_t n_trials, uint64_t seed, mca_run_stat
         CUDA_TRY(h, mca::launch_deep_eval(a, h->stream));
         CUDA_TRY(h, cudaEventRecord(h->ev[1], h->stream));
         CUDA_TRY(h, mca::launch_deep_decide(a, h->stream));
-        // with scratch slots the commit follows the decision on the host (below)
-        if (h->nscr == 0) CUDA_TRY(h, mca::launch_deep_commit(a, h->stream));
+        // tensor-core chain with scratch slots: the commit follows the decision on the host (below)
+        if (!h->tc || h->nscr == 0) CUDA_TRY(h, mca::launch_deep_commit(a, h->stream));
         else h->launches -= 1;
       }
       CUDA_TRY(h, cudaEventRecord(h->ev[2], h->stream));
@@ -1228,7 +1236,7 @@ mca_status mca_run(mca_handle* h, uint64_t n_trials, uint64_t seed, mca_run_stat
         h->broken = true;
         return fail(h, MCA_ERR_NUMERIC, "non-finite loss change");
       }
-      if (!h->tfm && h->nscr > 0 && ctl.kstar >= 0) {
+      if (h->deep && h->tc && h->nscr > 0 && ctl.kstar >= 0) {
         // The accepted candidate's fields: adopted from its scratch slot (row j of its layer
         // copied, the later layers' arrays and the losses swapped with the slot's), or, for a
         // candidate without a dense chain or beyond the slots, recomputed by the commit kernel.

@@ -96,19 +96,27 @@ __device__ __forceinline__ DeepCand deep_candidate(const DeepArgs& a, int k) {
 }
 
 // Loss change of sample n whose output fields become zz (changed: any field differs from the cached
-// one). COMMIT writes the new output fields and loss.
+// one). COMMIT writes the new output fields and loss. zout, lout (nullable): the fields and losses of
+// the candidate's scratch slot, written changed or not.
 template <bool COMMIT>
 __device__ __forceinline__ float out_delta(const DeepArgs& a, int n, const float (&zz)[kMaxC],
-                                           bool changed) {
-  if (!changed) return 0.0f;
+                                           bool changed, float* zout = nullptr,
+                                           float* lout = nullptr) {
   const int Lo = a.L - 1;
-  const float ln = sample_loss<-1, -1, kMaxC>(zz, a.C, a.y[n], a.g[Lo], a.act[Lo], a.loss);
-  const float dl = ln - a.ell[n];
-  if (COMMIT) {
+  float ln = 0.0f, dl = 0.0f;
+  if (changed) {
+    ln = sample_loss<-1, -1, kMaxC>(zz, a.C, a.y[n], a.g[Lo], a.act[Lo], a.loss);
+    dl = ln - a.ell[n];
+  }
+  if (COMMIT && changed) {
+    zout = a.Z[Lo];
+    lout = a.ell;
+  }
+  if (lout != nullptr) {
 #pragma unroll
     for (int c = 0; c < kMaxC; ++c)
-      if (c < a.C) a.Z[Lo][(size_t)c * a.Np + n] = zz[c];
-    a.ell[n] = ln;
+      if (c < a.C) zout[(size_t)c * a.Np + n] = zz[c];
+    lout[n] = changed ? ln : a.ell[n];
   }
   return dl;
 }

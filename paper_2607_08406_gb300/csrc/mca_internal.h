@@ -177,6 +177,7 @@ constexpr float kDeepDScale = 16384.0f;   // tanh changes (at most 2) as fp16 op
 constexpr int kDeepScrSlots = 16;  // candidates whose fields the tensor-core evaluation keeps
 constexpr float kTfmF16Max = 4.0f;   // largest parameter magnitude of the fp16 Transformer kernels
 constexpr int kTfmScrSlots = 16;   // candidates whose residual streams the evaluation keeps
+constexpr size_t kSimtScrBytes = (size_t)1 << 30;   // all slots of a SIMT evaluation
 
 struct DeepCand {
   unsigned int idx;
