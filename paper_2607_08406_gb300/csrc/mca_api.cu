@@ -861,12 +861,15 @@ mca_status run_tfm_pipelined(mca_handle* h, mca::TfmArgs ta, uint64_t n_trials) 
     CUDA_TRY(h, mca::launch_tfm_eval(ta, h->stream));
     CUDA_TRY(h, cudaEventRecord(h->ev_p[p][1], h->stream));
     CUDA_TRY(h, mca::launch_tfm_decide(ta, h->stream));
-    CUDA_TRY(h, mca::launch_tfm_commit(ta, h->stream));
+    if (ta.Kb > ta.nscr) {             // a candidate beyond the slots may be accepted
+      CUDA_TRY(h, mca::launch_tfm_commit(ta, h->stream));
+      h->launches += 1;
+    }
     CUDA_TRY(h, mca::launch_tfm_tc_adopt(ta, h->stream));
     CUDA_TRY(h, cudaMemcpyAsync(&ph->ctl[p], h->ctl2 + p, sizeof(mca::DeepCtl),
                                 cudaMemcpyDeviceToHost, h->stream));
     CUDA_TRY(h, cudaEventRecord(h->ev_p[p][2], h->stream));
-    h->launches += 4;
+    h->launches += 3;
     return MCA_OK;
   };
   uint64_t done = 0;
