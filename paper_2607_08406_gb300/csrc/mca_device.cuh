@@ -528,4 +528,27 @@ __device__ __forceinline__ float warp_sum_comp(float hi, float lo) {
   return hi + lo;
 }
 
+// Two fp32 operations in one instruction.
+__device__ __forceinline__ unsigned long long pack2(float2 v) {
+  return *reinterpret_cast<const unsigned long long*>(&v);
+}
+__device__ __forceinline__ float2 unpack2(unsigned long long v) {
+  return *reinterpret_cast<const float2*>(&v);
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  unsigned long long d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(pack2(a)), "l"(pack2(b)), "l"(pack2(c)));
+  return unpack2(d);
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+  unsigned long long d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(pack2(a)), "l"(pack2(b)));
+  return unpack2(d);
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+  unsigned long long d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(pack2(a)), "l"(pack2(b)));
+  return unpack2(d);
+}
+
 }  // namespace mca

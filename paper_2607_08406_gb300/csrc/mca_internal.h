@@ -389,8 +389,8 @@ struct ProposeArgs {
 cudaError_t launch_propose(const ProposeArgs& a, cudaStream_t s);
 
 // Fields of a layer on the tensor cores (mca_gemm_tc.cu): Z[M x Np] = W[M x K] act(B)[K x Np]
-// (act < 0: B as it is), three MMAs per product of fp16 or tf32 parts. img: scratch of gemm_tc_image_bytes(M, K, Np) bytes, 256-byte
-// aligned; err: device status word (MCA_ERR_TIMEOUT when a bounded wait ran out).
+// (act < 0: B as it is), three MMAs per product of fp16 or tf32 parts. img: scratch of
+// gemm_tc_image_bytes(M, K, Np) bytes, 256-byte aligned; err: device status word (MCA_ERR_TIMEOUT when a bounded wait ran out).
 bool gemm_tc_ok(int M, int K, int Np);
 size_t gemm_tc_image_bytes(int M, int K, int Np);
 cudaError_t launch_gemm_tc(const float* W, int M, int K, const float* B, int act, float g,

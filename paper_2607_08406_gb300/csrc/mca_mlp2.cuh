@@ -734,28 +734,6 @@ struct VRecs {
   }
 };
 
-__device__ __forceinline__ unsigned long long pack2(float2 v) {
-  return *reinterpret_cast<const unsigned long long*>(&v);
-}
-__device__ __forceinline__ float2 unpack2(unsigned long long v) {
-  return *reinterpret_cast<const float2*>(&v);
-}
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
-  unsigned long long d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(pack2(a)), "l"(pack2(b)), "l"(pack2(c)));
-  return unpack2(d);
-}
-__device__ __forceinline__ float2 add2(float2 a, float2 b) {
-  unsigned long long d;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(pack2(a)), "l"(pack2(b)));
-  return unpack2(d);
-}
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
-  unsigned long long d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(pack2(a)), "l"(pack2(b)));
-  return unpack2(d);
-}
-
 // Loss of the fields z with label y; zy: field y; onehot: -[k == y] per field (MSE).
 template <int ACT2, int LOSS, int M>
 __device__ __forceinline__ float vloss(const Mlp2Args& a, const float2 (&z)[M / 2], int y, float zy,
