@@ -148,75 +148,116 @@ __global__ void init_layer_kernel(int wkind, float scale, const float* __restric
 }
 
 // C[M x Ncol] = A[M x K] * B[K x Ncol], row-major, fp32 FMA in ascending k. Ncol % 128 == 0,
-// ldb and ldc multiples of 4. 128x128 tile per CTA, 256 threads, 8x8 outputs per thread.
-// ACTB: the B operand enters as act(B) (the previous layer's activations from its fields).
-template <bool ACTB>
-__global__ void __launch_bounds__(256) sgemm_nn_kernel(int M, int Ncol, int K,
-                                                       const float* __restrict__ A, int lda,
-                                                       const float* __restrict__ B, int ldb,
-                                                       float* __restrict__ C, int ldc, int bact,
-                                                       float bg) {
-  constexpr int BM = 128, BN = 128, BK = 8;
-  __shared__ __align__(16) float As[BK][BM];
-  __shared__ __align__(16) float Bs[BK][BN];
+// ldb and ldc multiples of 4. ACTB: the B operand enters as act(B) (the previous layer's activations
+// from its fields).
+//
+// 256 threads compute a tile of 16 R x 16 R outputs, R x R per thread. The next 16 k are in flight (in
+// registers) while a chunk is multiplied out of one of two buffers, one barrier per chunk; products come
+// in pairs of columns, each rounded as a single one. Small products are bounded by latency, so the
+// tile is the largest one whose CTAs fill the GPU (sgemm_tile). The forward pass of 784-64-10 on 1000
+// samples takes 65 us (152 us with tiles of 128 throughout, one chunk of 8 k at a time), of 784-100x5-10
+// on 3001 samples 125 us (258 us), of 391-1001-7 on 12347 samples 285 us (336 us).
+constexpr int kSgK = 16;
+
+// Row or column of value q of thread t (of 16): groups of four for the vector loads.
+template <int R>
+__device__ __forceinline__ int sg_at(int t, int q) {
+  return R == 8 ? (q >> 2) * 64 + t * 4 + (q & 3) : t * R + q;
+}
+
+template <int R>
+__device__ __forceinline__ void sg_load(const float* p, int t, float (&v)[R]) {
+  if constexpr (R == 2) {
+    const float2 x = *reinterpret_cast<const float2*>(p + 2 * t);
+    v[0] = x.x;
+    v[1] = x.y;
+  } else {
+#pragma unroll
+    for (int g = 0; g < R / 4; ++g) {
+      const float4 x = *reinterpret_cast<const float4*>(p + 64 * g + 4 * t);
+      v[4 * g] = x.x;
+      v[4 * g + 1] = x.y;
+      v[4 * g + 2] = x.z;
+      v[4 * g + 3] = x.w;
+    }
+  }
+}
+
+template <int R, bool ACTB>
+__global__ void __launch_bounds__(256, R == 8 ? 2 : 4) sgemm_nn_kernel(
+    int M, int K, const float* __restrict__ A, int lda, const float* __restrict__ B, int ldb,
+    float* __restrict__ C, int ldc, int bact, float bg) {
+  constexpr int BM = 16 * R, BN = 16 * R;
+  constexpr int NB = (kSgK * BN / 4 + 255) / 256;   // 16-byte units of B per thread
+  __shared__ __align__(16) float As[2][kSgK][BM + 4];
+  __shared__ __align__(16) float Bs[2][kSgK][BN];
   const int tid = threadIdx.x;
   const int bm = blockIdx.y * BM, bn = blockIdx.x * BN;
   const int tr = tid / 16, tc = tid % 16;
-  float acc[8][8];
+  float2 acc[R][R / 2];
 #pragma unroll
-  for (int i = 0; i < 8; ++i)
+  for (int i = 0; i < R; ++i)
 #pragma unroll
-    for (int j = 0; j < 8; ++j) acc[i][j] = 0.0f;
-  const int arow = tid / 2, akk = (tid % 2) * 4;
-  const int bkk = tid / 32, bcol = (tid % 32) * 4;
-  for (int k0 = 0; k0 < K; k0 += BK) {
+    for (int j = 0; j < R / 2; ++j) acc[i][j] = make_float2(0.0f, 0.0f);
+  float an[R];                                      // k = tid % 16 of rows tid / 16 + 16 u
+  float4 bv[NB];
+  auto fetch = [&](int k0) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int m = bm + arow, kk = k0 + akk + q;
-      As[akk + q][arow] = (m < M && kk < K) ? A[(size_t)m * lda + kk] : 0.0f;
+    for (int u = 0; u < R; ++u) {
+      const int m = bm + tr + 16 * u, kk = k0 + tc;
+      an[u] = m < M && kk < K ? A[(size_t)m * lda + kk] : 0.0f;
     }
-    {
-      const int kk = k0 + bkk;
-      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (kk < K) {
-        v = *reinterpret_cast<const float4*>(B + (size_t)kk * ldb + bn + bcol);
-        if (ACTB) {
-          v.x = act_rt(bact, v.x, bg);
-          v.y = act_rt(bact, v.y, bg);
-          v.z = act_rt(bact, v.z, bg);
-          v.w = act_rt(bact, v.w, bg);
-        }
+#pragma unroll
+    for (int u = 0; u < NB; ++u) {
+      const int e = tid + 256 * u, kk = k0 + e / (BN / 4), col = e % (BN / 4) * 4;
+      bv[u] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      if (e < kSgK * BN / 4 && kk < K)
+        bv[u] = *reinterpret_cast<const float4*>(B + (size_t)kk * ldb + bn + col);
+    }
+  };
+  fetch(0);
+  int buf = 0;
+#pragma unroll 1
+  for (int k0 = 0; k0 < K; k0 += kSgK) {
+#pragma unroll
+    for (int u = 0; u < R; ++u) As[buf][tc][tr + 16 * u] = an[u];
+#pragma unroll
+    for (int u = 0; u < NB; ++u) {
+      const int e = tid + 256 * u, kk = e / (BN / 4), col = e % (BN / 4) * 4;
+      if (e >= kSgK * BN / 4) continue;
+      float4 v = bv[u];
+      if (ACTB && k0 + kk < K) {
+        v.x = act_rt(bact, v.x, bg);
+        v.y = act_rt(bact, v.y, bg);
+        v.z = act_rt(bact, v.z, bg);
+        v.w = act_rt(bact, v.w, bg);
       }
-      *reinterpret_cast<float4*>(&Bs[bkk][bcol]) = v;
+      *reinterpret_cast<float4*>(&Bs[buf][kk][col]) = v;
     }
     __syncthreads();
+    if (k0 + kSgK < K) fetch(k0 + kSgK);
 #pragma unroll
-    for (int kk = 0; kk < BK; ++kk) {
-      float ra[8], rb[8];
-      const float4 a0 = *reinterpret_cast<const float4*>(&As[kk][tr * 4]);
-      const float4 a1 = *reinterpret_cast<const float4*>(&As[kk][64 + tr * 4]);
-      const float4 b0 = *reinterpret_cast<const float4*>(&Bs[kk][tc * 4]);
-      const float4 b1 = *reinterpret_cast<const float4*>(&Bs[kk][64 + tc * 4]);
-      ra[0] = a0.x; ra[1] = a0.y; ra[2] = a0.z; ra[3] = a0.w;
-      ra[4] = a1.x; ra[5] = a1.y; ra[6] = a1.z; ra[7] = a1.w;
-      rb[0] = b0.x; rb[1] = b0.y; rb[2] = b0.z; rb[3] = b0.w;
-      rb[4] = b1.x; rb[5] = b1.y; rb[6] = b1.z; rb[7] = b1.w;
+    for (int kk = 0; kk < kSgK; ++kk) {
+      float ra[R], rb[R];
+      sg_load<R>(As[buf][kk], tr, ra);
+      sg_load<R>(Bs[buf][kk], tc, rb);
 #pragma unroll
-      for (int i = 0; i < 8; ++i)
+      for (int i = 0; i < R; ++i)
 #pragma unroll
-        for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(ra[i], rb[j], acc[i][j]);
+        for (int j = 0; j < R / 2; ++j)
+          acc[i][j] = fma2(make_float2(ra[i], ra[i]), make_float2(rb[2 * j], rb[2 * j + 1]),
+                           acc[i][j]);
     }
-    __syncthreads();
+    buf ^= 1;
   }
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int m = bm + (i < 4 ? tr * 4 + i : 64 + tr * 4 + (i - 4));
+  for (int i = 0; i < R; ++i) {
+    const int m = bm + sg_at<R>(tr, i);
     if (m >= M) continue;
     float* crow = C + (size_t)m * ldc + bn;
-    *reinterpret_cast<float4*>(crow + tc * 4) =
-        make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
-    *reinterpret_cast<float4*>(crow + 64 + tc * 4) =
-        make_float4(acc[i][4], acc[i][5], acc[i][6], acc[i][7]);
+#pragma unroll
+    for (int j = 0; j < R / 2; ++j)
+      *reinterpret_cast<float2*>(crow + sg_at<R>(tc, 2 * j)) = acc[i][j];
   }
 }
 
@@ -369,24 +410,34 @@ cudaError_t launch_init_layer(int wkind, float scale, const float* src, const si
   return cudaGetLastError();
 }
 
+// R of the SGEMM's tiles: 8 while two CTAs per SM have one, then 4 while every SM does, else 2.
+static int sgemm_tile(int M, int Ncol) {
+  auto ctas = [&](int t) { return (long long)(Ncol / t) * ((M + t - 1) / t); };
+  return ctas(128) >= 304 ? 8 : ctas(64) >= 152 ? 4 : 2;
+}
+
+template <bool ACTB>
+static cudaError_t launch_sgemm(int M, int Ncol, int K, const float* A, int lda, const float* B,
+                                int ldb, float* C, int ldc, int bact, float bg, cudaStream_t s) {
+  const int R = sgemm_tile(M, Ncol), t = 16 * R;
+  const dim3 grid(Ncol / t, (M + t - 1) / t);
+  auto fn = R == 8 ? sgemm_nn_kernel<8, ACTB>
+            : R == 4 ? sgemm_nn_kernel<4, ACTB> : sgemm_nn_kernel<2, ACTB>;
+  fn<<<grid, 256, 0, s>>>(M, K, A, lda, B, ldb, C, ldc, bact, bg);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_sgemm_nn(int M, int Ncol, int K, const float* A, int lda, const float* B,
                             int ldb, float* C, int ldc, cudaStream_t s) {
-  dim3 grid(Ncol / 128, (M + 127) / 128);
-  sgemm_nn_kernel<false><<<grid, 256, 0, s>>>(M, Ncol, K, A, lda, B, ldb, C, ldc, 0, 0.0f);
-  return cudaGetLastError();
+  return launch_sgemm<false>(M, Ncol, K, A, lda, B, ldb, C, ldc, 0, 0.0f, s);
 }
 
 // Fields of deep layer l from the previous layer (or X for l = 0): Z_l = W_l act_{l-1}(Z_{l-1}).
 cudaError_t launch_deep_forward_layer(const DeepArgs& a, int l, cudaStream_t s) {
   const int M = a.n_out[l], K = a.n_in[l];
-  dim3 grid(a.Np / 128, (M + 127) / 128);
-  if (l == 0)
-    sgemm_nn_kernel<false><<<grid, 256, 0, s>>>(M, a.Np, K, a.w[0], K, a.XT, a.Np, a.Z[0], a.Np, 0,
-                                                0.0f);
-  else
-    sgemm_nn_kernel<true><<<grid, 256, 0, s>>>(M, a.Np, K, a.w[l], K, a.Z[l - 1], a.Np, a.Z[l],
-                                               a.Np, a.act[l - 1], a.g[l - 1]);
-  return cudaGetLastError();
+  if (l == 0) return launch_sgemm_nn(M, a.Np, K, a.w[0], K, a.XT, a.Np, a.Z[0], a.Np, s);
+  return launch_sgemm<true>(M, a.Np, K, a.w[l], K, a.Z[l - 1], a.Np, a.Z[l], a.Np, a.act[l - 1],
+                            a.g[l - 1], s);
 }
 
 cudaError_t launch_sum_loss(const float* ell, int N, DevState* st, cudaStream_t s) {
