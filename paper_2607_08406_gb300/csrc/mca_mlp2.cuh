@@ -678,6 +678,42 @@ constexpr int kConsWarps = kLoopWarps - kProdWarps;
 static_assert(kLookWarp0 == kConsWarps - kWS / 32 && kWS % 32 == 0, "one lane per slot");
 constexpr int kConsThreads = kConsWarps * 32;
 
+// Warps per candidate when a batch has n live ones (n = x + 1; the last entry serves any larger n), four
+// bits each, and ceil(256 / those), nine bits each: v / w = (v ceil(256 / w)) / 256 for v < kConsWarps.
+constexpr int kWpcLast = kConsWarps / 2;
+constexpr int warps_per_cand(int x) { return x < kWpcLast ? kConsWarps / (x + 1) : 1; }
+constexpr unsigned long long wpc_table(int bits, bool inverse) {
+  unsigned long long t = 0;
+  for (int x = 0; x <= kWpcLast; ++x) {
+    const int w = warps_per_cand(x);
+    t |= (unsigned long long)(inverse ? (256 + w - 1) / w : w) << (bits * x);
+  }
+  return t;
+}
+constexpr bool wpc_exact() {
+  for (int x = 0; x <= kWpcLast; ++x)
+    for (int v = 0; v < kConsWarps; ++v) {
+      const int w = warps_per_cand(x);
+      if (((v * ((256 + w - 1) / w)) >> 8) != v / w) return false;
+    }
+  return true;
+}
+constexpr unsigned long long kWpc = wpc_table(4, false), kWpcInv = wpc_table(9, true);
+static_assert(9 * (kWpcLast + 1) <= 64 && kConsWarps < 16 && wpc_exact(), "warp split tables");
+
+// Place of the i-th set bit of a mask (a whole warp).
+__device__ __forceinline__ int nth_bit(unsigned long long mask, int i) {
+  const int lane = threadIdx.x & 31;
+  const unsigned int lt = (1u << lane) - 1u;
+  const unsigned int l0 = (unsigned int)mask, l1 = (unsigned int)(mask >> 32);
+  const int n0 = __popc(l0);
+  const unsigned int half = i < n0 ? l0 : l1;
+  const int rank = i < n0 ? i : i - n0;
+  const unsigned int hit = __ballot_sync(
+      0xffffffffu, ((half >> lane) & 1u) != 0u && __popc(half & lt) == rank);
+  return __ffs(hit) - 1 + (i < n0 ? 0 : 32);
+}
+
 // Barrier of the consumer warps only (named barrier 1).
 __device__ __forceinline__ void cons_sync() {
   asm volatile("bar.sync 1, %0;" ::"r"(kConsThreads) : "memory");
@@ -695,8 +731,8 @@ inline size_t window_smem_bytes(int RS) {
 // the fields past the class count hold -infinity, whose exponential and sigmoid are 0, instead of a
 // test per field. (One 4-byte load and one instruction per field took, per batch, 4.50 us for
 // 391-1001-7 masked nets with MSE on 12347 samples, 4.17 us for 784-2048-10 ReLU nets with
-// cross-entropy on 30000; now 3.70 and 4.03 us. 784-64-10, all of whose records fit a warp or two: 3.66
-// and 3.68.)
+// cross-entropy on 30000; with vectors 3.70 and 4.03 us. 784-64-10, all of whose records fit a warp or
+// two: 3.66 and 3.68.)
 //
 // M = 10 fields (up to 10 classes): 12 floats a sample, M = 14: 16 floats whose 16-byte parts are
 // permuted by the sample's number, so that the lanes of a warp, which read different samples, spread
@@ -1400,6 +1436,19 @@ __global__ void __launch_bounds__(kLoopThreads, 1) mlp2_window_loop(Mlp2Args a) 
           if (wk != MCA_W_FP32) (c.layer ? a.code2 : a.code1)[off] = (signed char)c.new_code;
         }
       }
+      // this warp's part of the evaluation (below), ahead of the barrier where the live candidates are
+      // known; warp 0, which ends the set-up, after it
+      int nlive = 0, wpc = 1, vi = 0, vj = 0, vk = 0;
+      auto split = [&]() {
+        const int vw = warp == 0 ? kConsWarps - 1 : warp - 1;
+        nlive = __popcll(live_mask);
+        const int x = min(max(nlive, 1) - 1, kWpcLast);
+        wpc = (int)(kWpc >> (4 * x)) & 15;
+        vi = (vw * ((int)(kWpcInv >> (9 * x)) & 511)) >> 8;
+        vj = vw - vi * wpc;
+        vk = nth_bit(live_mask, vi);
+      };
+      if (known && warp != 0) split();
       cons_sync();
       if (pend >= 0) {
         // every consumer's writes of the commit precede the new epoch that producers read
@@ -1445,6 +1494,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) mlp2_window_loop(Mlp2Args a) 
       }
       const unsigned long long t_s = timer ? globaltimer_ns() : 0ull;
       if (!known || redo) live_mask = s_live;
+      if (!known || redo || warp == 0) split();
       // ---- evaluate. A candidate's entries in this range are cut into chunks: 32 cached entries (from
       // shared memory), or a.SUB samples read from global memory. What bounds the evaluation is the
       // length of one warp's instruction sequence, so the warps share the candidates: wpc warps per
@@ -1454,11 +1504,10 @@ __global__ void __launch_bounds__(kLoopThreads, 1) mlp2_window_loop(Mlp2Args a) 
       // and added in order, whatever the number of warps. The warp that finishes a candidate adds the
       // CTA's share. The last three warps look at the slots ahead: before they evaluate when the
       // others suffice for that, else afterwards. Warp 0, which waits for the other CTAs, is the last
-      // to get work.
+      // to get work. Each warp's part comes from tables, ahead of the barrier: with three divisions after it a
+      // batch took 3.69, 4.40, 3.83, 3.71 and 4.03 us (small, wide, ternary, masked, ReLU nets), now 3.53,
+      // 4.28, 3.68, 3.52 and 3.94.
       unsigned long long* acc = a.accum + (size_t)(bidx % kAccBuffers) * kAccStride;
-      const int nlive = __popcll(live_mask);
-      const int wpc = nlive > kConsWarps / 2 ? 1 : nlive > 0 ? kConsWarps / nlive : 1;
-      const int vw = warp == 0 ? kConsWarps - 1 : warp - 1;
       const bool look_first = nlive * wpc <= kLookWarp0 - 1;
 #pragma unroll 1
       for (int ph = 0; ph < 2; ++ph) {
@@ -1507,19 +1556,8 @@ __global__ void __launch_bounds__(kLoopThreads, 1) mlp2_window_loop(Mlp2Args a) 
           continue;
         }
 #pragma unroll 1
-        for (int i = vw / wpc; i < nlive; i += kConsWarps) {   // (wpc = 1 when there are more)
-          const int j = vw - (vw / wpc) * wpc;
-          int k;                           // the i-th live candidate
-          {
-            const unsigned int lt = (1u << lane) - 1u;
-            const unsigned int l0 = (unsigned int)live_mask, l1 = (unsigned int)(live_mask >> 32);
-            const int n0 = __popc(l0);
-            const unsigned int half = i < n0 ? l0 : l1;
-            const int rank = i < n0 ? i : i - n0;
-            const unsigned int hit = __ballot_sync(
-                0xffffffffu, ((half >> lane) & 1u) != 0u && __popc(half & lt) == rank);
-            k = __ffs(hit) - 1 + (i < n0 ? 0 : 32);
-          }
+        for (int i = vi; i < nlive; i += kConsWarps) {         // (wpc = 1 when there are more)
+          const int j = vj, k = i == vi ? vk : nth_bit(live_mask, i);
           const int sl = slot_after(sl_tau, k);
           const Cand& c = s_slot[sl].c;
           const bool cached = s_slot[sl].state == 1;
