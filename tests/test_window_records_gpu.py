@@ -9,7 +9,7 @@ import pytest
 from oracle import mca_oracle as O
 from paper_2607_08406_gb300 import workloads as W
 
-from parity import TIE_REL, compare, oracle_trace
+from parity import TIE_REL, compare, forced_from_oracle, oracle_trace
 
 pytestmark = pytest.mark.gpu
 
@@ -46,6 +46,25 @@ def test_record_classes(gpu_lib, C, hidden, out, loss, N, H, beta):
     compare(gpu_lib.mca_get_trace(h, wl.n_trials), tr)
     assert np.array_equal(gpu_lib.mca_get_params(h, wl.n_params), params.flat_eff32())
     assert gpu_lib.mca_loss(h) == pytest.approx(S / wl.N, rel=TIE_REL)
+
+
+@pytest.mark.parametrize("strict,hi,K", [(False, 1.0, 16), (True, 4.0, 64)])
+def test_commit_routes(gpu_lib, strict, hi, K):
+    """Ranges of several chunks of entries: candidates whose warps hold every new loss at the commit, and
+    (wide batches of many live candidates) those with fewer warps than chunks."""
+    wl = _net(10, "tanh", "identity", "softmax_ce", 24000, 6, hi=hi)
+    wl.domain.strict, wl.K = strict, K
+    n = 400
+    tr, params, S = oracle_trace(wl, n)
+    assert tr["accept"].sum() >= 20
+    h = gpu_lib.create_from_workload(wl, trace_cap=n)
+    gpu_lib.mca_force_decisions(h, *forced_from_oracle(tr))
+    gpu_lib.mca_run(h, n, wl.seed)
+    compare(gpu_lib.mca_get_trace(h, n), tr)
+    assert np.array_equal(gpu_lib.mca_get_params(h, wl.n_params), params.flat_eff32())
+    cached = gpu_lib.mca_loss(h)
+    gpu_lib.mca_resync(h)
+    assert gpu_lib.mca_loss(h) == pytest.approx(cached, rel=TIE_REL)
 
 
 def test_hidden_fields_that_overflow(gpu_lib):
