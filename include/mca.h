@@ -133,10 +133,12 @@ typedef struct {
   size_t workspace_bytes;
   int32_t fixed_K;         /* 0: the batch width follows p, the recently observed acceptance rate
                               per trial, at most K (fewer discarded candidates while many are
-                              accepted; the trajectory is the same): ceil(2 / p) candidates for
-                              single-hidden-layer networks; for deep nets and Transformers the K
+                              accepted; the trajectory is the same): ceil(c / p) candidates for
+                              single-hidden-layer networks (c = 2, or 1.6 for large sample
+                              ranges); for deep nets and Transformers the K
                               that maximises the expected trials consumed, (1 - (1-p)^K) / p, per
-                              batch cost r + K (r about 2 candidate evaluations);
+                              cost of the batch (a fixed part, one evaluation until the candidates
+                              fill the GPU, and their share of it beyond);
                               1: every batch evaluates K candidates */
 } mca_options;
 
@@ -175,7 +177,8 @@ typedef struct {
   uint64_t alg_flops;      /* deep nets: FLOPs of the evaluated candidates' recomputation (2 per
                               multiply-add: the row update, the rank-1 layer, the dense layers) */
   uint32_t tensor_cores;   /* 1: this handle's dense recomputation runs on the tcgen05 tensor-core
-                              kernels (3xTF32): a deep net whose hidden layers are all 256 x 256,
+                              kernels (three MMAs of fp16 or tf32 parts per fp32 product): a deep
+                              net whose hidden layers are all 256 x 256,
                               or a Transformer with ctx 64, d_model 128, 4 heads, d_ff a multiple
                               of 128 up to 1024, vocab <= 128 and an even number of sequences
                               (unless the process sets MCA_TFM_TENSOR_CORES=0 before creating
@@ -241,7 +244,9 @@ mca_status mca_tfm_workspace_size(const mca_tfm_spec* spec, int64_t n_seq, const
  * host or device, in the flat order above. Every parameter is an fp32 weight (Eq. 1 replacement or
  * perturbation). mca_loss reports S / (n_seq * ctx). Errors as for mca_create.
  * Kernels: with ctx 64, d_model 128, 4 heads, d_ff a multiple of 128 up to 1024, vocab <= 128 and an
- * even n_seq the sequences run on the tensor-core kernels (3xTF32 tcgen05, two sequences per CTA);
+ * even n_seq the sequences run on the tensor-core kernels (tcgen05, three MMAs per fp32 product, of
+ * fp16 parts while every parameter is at most 4 in magnitude and of tf32 parts otherwise, two
+ * sequences per CTA);
  * for other shapes, or when the process environment has MCA_TFM_TENSOR_CORES=0, on the SIMT fp32
  * kernels. The variable is read by this call and by mca_tfm_workspace_size (the tensor-core kernels'
  * weight images are part of the workspace), so it must not change between the two. mca_run_stats
@@ -249,9 +254,10 @@ mca_status mca_tfm_workspace_size(const mca_tfm_spec* spec, int64_t n_seq, const
  * the first sub-block its parameter feeds (a block's input, its cached stream after the attention
  * sub-block for LN2, a rank-1 step for one hidden unit of the feed-forward network), the evaluation
  * of candidates k < min(K, 16) keeps what it recomputed in per-candidate scratch slots of the
- * workspace (at most 8 GiB) from which an accepted candidate is adopted, and mca_run enqueues each
+ * workspace (at most 8 GiB; SIMT kernels 1 GiB) from which an accepted candidate is adopted, and
+ * (tensor-core kernels) mca_run enqueues each
  * batch before it reads the previous decision unless resync_period > 0. MCA_ADOPT=0 in the
- * environment (read like MCA_TFM_TENSOR_CORES; it applies to deep MLPs on the tensor cores too)
+ * environment (read like MCA_TFM_TENSOR_CORES; it applies to deep MLPs too)
  * leaves out the slots: every accepted candidate is then recomputed by the commit kernels. */
 mca_status mca_create_transformer(const mca_tfm_spec* spec, const mca_domain* dom,
                                   const int32_t* tokens, int64_t n_seq, const float* init_params,

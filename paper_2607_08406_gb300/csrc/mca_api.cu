@@ -390,6 +390,8 @@ mca::Mlp2Args mlp2_args(mca_handle* h) {
   a.SUB = h->SUB;
   a.smem_records = h->smem_records;
   a.window = h->window;
+  const double per_range = (double)h->nnz / ((double)h->D * (double)h->NR);   // entries of a feature
+  a.wscale = per_range > 32.0 ? mca::kWidthMlp2Long : mca::kWidthMlp2;
   a.P = h->P;
   a.P1 = (unsigned long long)L1.n_in * L1.n_out;
   a.xs_off = h->xs_off;

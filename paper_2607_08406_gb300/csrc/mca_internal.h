@@ -24,7 +24,11 @@ constexpr int kRangeTarget = 64;
 // Batch width of the single-hidden-layer loop: ceil(c / p) candidates, p = (A + 0.5) / (T + 1) from
 // counts decayed per batch.
 constexpr float kRateDecay = 0.95f;
-constexpr float kWidthMlp2 = 2.0f;
+// In the windowed loop kWidthMlp2Long where a feature has more than one chunk of 32 entries per range: a batch
+// of seven live candidates has one warp each, which takes a round of chunks more than six with two
+// warps. 784-16384-10 on 60000 samples, trials 375k .. 1M (p = 0.29): 691k trials/s at 2, 714k at 1.6,
+// 716k at 1.4; trials 0 .. 4000 (p = 0.48): 8.11, 7.92 and 8.11 ms.
+constexpr float kWidthMlp2 = 2.0f, kWidthMlp2Long = 1.6f;
 // Host-driven batches (deep nets, the Transformer): a batch of K candidates consumes
 // (1 - (1 - p)^K) / p trials on average and costs about r + K candidate evaluations, r being its
 // fixed part (decision, adoption or commit, launch gaps, the last partial wave of CTAs). The width
@@ -117,6 +121,7 @@ struct Mlp2Args {
   int NR, RS, SUB;           // ranges, samples per range, entries per sub-chunk (multiple of 32)
   int smem_records;          // 1: each CTA keeps its range's sample records in shared memory
   int window;                // 1: run the windowed trial loop (records and window in shared memory)
+  float wscale;              // the windowed loop's batches take ceil(wscale / p) candidates
   unsigned long long P, P1;
   const int* xs_off;         // [D + 1] CSR of X by feature: entries of feature i in [off[i], off[i+1])
   const int* xs_n;           // [nnz] sample index of each entry (ascending inside a feature)
