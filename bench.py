@@ -34,9 +34,10 @@ METRIC = "MC mutation trials/sec (full-batch loss evals); fraction of HBM/TC roo
 # from one ncu capture (one pass, one launch: the first timed step, trials 200k..240k) of
 # `python bench.py --steps 20 --warmup 5 --no-e2e --no-cpu`, summarised in profiles/. It is only
 # valid for the kernel source and the workload it was measured on; anything else reports null.
-LOOP_TRAFFIC = {"source_sha1": "2502508233974700a08bab261aa72e3018dd27bb",
+LOOP_TRAFFIC = {"source_sha1": "6287e992baef9cabbf10b88d40ec38254588b001",
                 "workload": "mlp784-16384-10_ce_n60000", "bytes_per_trial": 374000.0}
-LOOP_SOURCES = ("paper_2607_08406_gb300/csrc/mca_mlp2.cu", "paper_2607_08406_gb300/csrc/mca_device.cuh")
+LOOP_SOURCES = tuple(f"paper_2607_08406_gb300/csrc/{f}" for f in (
+    "mca_mlp2.cuh", "mca_mlp2.cu", "mca_mlp2_ce.cu", "mca_mlp2_mse.cu", "mca_device.cuh"))
 
 
 def loop_source_sha1() -> str:
@@ -357,12 +358,12 @@ def run_ours(args):
                 bf16, bf16_kind = float(json.load(open(pk))["bf16_tflops_sustained"]), "measured"
             else:
                 bf16, bf16_kind = 1700.0, "fallback"
-            peak = bf16 * 0.5 / 3.0
-            peak_kind = (f"{bf16_kind} bf16 sustained x 1/2 (nominal tf32 : bf16 dense rate) / 3 "
-                         "(3xTF32: three tf32 MMAs per fp32 product)")
+            peak = bf16 / 3.0
+            peak_kind = (f"{bf16_kind} bf16 sustained / 3 (three fp16 MMAs per fp32 product, at the "
+                         "bf16 rate)")
             roofline = {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                         "frac": achieved / peak, "traffic": None,
-                        "kernel": "tfm_tc_kernel" if is_tfm(wl) else "deep_chain_tc_kernel",
+                        "kernel": "tfm_f16_kernel" if is_tfm(wl) else "deep_chain_tc_kernel",
                         "peak_kind": peak_kind,
                         "flops": "2 x fp32 multiply-adds of the evaluated chains (not x3), over "
                                  "the evaluation kernel's event-timed duration"}

@@ -96,7 +96,8 @@ bool deep_tc_ok(const std::vector<mca_layer>& layers) {
   return true;
 }
 
-// Accepted candidates are adopted from scratch slots written by their evaluation unless the process sets MCA_ADOPT=0: then the commit kernels
+// Accepted candidates are adopted from scratch slots written by their evaluation unless the process sets
+// MCA_ADOPT=0: then the commit kernels
 // recompute them. Read by the workspace-size calls and creation, so it must not change between them.
 bool adopt_enabled() {
   const char* e = std::getenv("MCA_ADOPT");

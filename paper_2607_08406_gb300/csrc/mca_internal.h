@@ -239,7 +239,7 @@ struct DeepArgs {
   const float* ex_new;
   double* ex_out;
   ExTail* ex_tail;           // nullable
-  // tensor-core evaluation of candidate k < nscr with a dense chain (layer <= L-3): every field it
+  // evaluation of candidate k < nscr (on the tensor cores with a dense chain, layer <= L-3): every field it
   // computes goes to scr[k * (L + 1) + m] (layer m: row j of the mutated layer, the full layers
   // after it; m = L: the per-sample losses), so that an accepted candidate's fields are adopted
   // by swapping pointers instead of recomputing them
@@ -317,8 +317,8 @@ struct TfmArgs {
   void* wimg16;              // the images with fp16 parts, kept beside them
   int f16;                   // tc = 1: run the kernels with fp16 parts (every parameter, and every
                              //   candidate's, at most kTfmF16Max in magnitude)
-  // scratch slots (tc = 1, trial loop only): candidate k < nscr of a batch writes the residual
-  // streams it recomputes to slot k of scrX ([nscr][(2 nL + 1) x B x T x d]: X, then Xmid) and its
+  // scratch slots (trial loop only): candidate k < nscr of a batch writes the residual streams it
+  // recomputes to slot k of scrX ([nscr][(2 nL + 1) x B x T x d]: X, then Xmid; SIMT: X alone) and its
   // sequence losses to scr_ell ([nscr][B]); an accepted candidate with a slot is adopted from it
   float* scrX;
   float* scr_ell;
@@ -395,7 +395,8 @@ cudaError_t launch_propose(const ProposeArgs& a, cudaStream_t s);
 
 // Fields of a layer on the tensor cores (mca_gemm_tc.cu): Z[M x Np] = W[M x K] act(B)[K x Np]
 // (act < 0: B as it is), three MMAs per product of fp16 or tf32 parts. img: scratch of
-// gemm_tc_image_bytes(M, K, Np) bytes, 256-byte aligned; err: device status word (MCA_ERR_TIMEOUT when a bounded wait ran out).
+// gemm_tc_image_bytes(M, K, Np) bytes, 256-byte aligned; err: device status word (MCA_ERR_TIMEOUT when a
+// bounded wait ran out).
 bool gemm_tc_ok(int M, int K, int Np);
 size_t gemm_tc_image_bytes(int M, int K, int Np);
 cudaError_t launch_gemm_tc(const float* W, int M, int K, const float* B, int act, float g,
@@ -472,7 +473,7 @@ struct mca_handle {
     mca::ExTail tail;
   }* ev_host = nullptr;
   float* gimg = nullptr;                 // operand images of the tensor-core forward pass
-  int nscr = 0;                          // tensor-core paths: candidate scratch slots
+  int nscr = 0;                          // host-driven batches: candidate scratch slots
   std::vector<float*> scr;               // [nscr x (L + 1)] layer m of slot k (m = L: losses)
   float** scr_dev = nullptr;             // the same table in device memory
   cudaEvent_t ev_c[2] = {nullptr, nullptr};   // around the adoption / commit after a decision
@@ -503,10 +504,10 @@ struct mca_handle {
   float* params = nullptr;               // [P] flat parameters
   int* tokens = nullptr;                 // [B x (ctx + 1)]
   float* X = nullptr;                    // cached residual stream at every stage
-  float* tfm_img = nullptr;
+  float* tfm_img = nullptr;              // split-weight images of the tensor-core kernels (tc)
   void* tfm_img16 = nullptr;             // the same with fp16 operand parts
   float pmax = 0.0f;                     // tensor-core Transformer: largest parameter magnitude
   float* tfm_Xmid = nullptr;             // its mid streams (after each block's attention)
-  float* tfm_scrX = nullptr;             // Transformer tensor-core path: candidate scratch slots
-  float* tfm_scr_ell = nullptr;          // (h->nscr of them)              // split-weight images of the tensor-core kernels (tc)
+  float* tfm_scrX = nullptr;             // Transformer: candidate scratch slots
+  float* tfm_scr_ell = nullptr;          // (h->nscr of them)
 };

@@ -1198,7 +1198,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) mlp2_window_loop(Mlp2Args a) 
   __shared__ unsigned int s_redo_head, s_redo_tail;
   __shared__ unsigned long long s_bbytes, s_tau_hi, s_next, s_limit;
   // CTA 0's statistics, here rather than in 20 registers of every thread (with them the kernels spilled, and
-  // a batch of the wide, ternary and ReLU nets took 4.07, 3.57 and 3.74 us, now 3.89, 3.52 and 3.67)
+  // a batch of the wide, ternary and ReLU nets took 4.07, 3.57 and 3.74 us, with them here 3.89, 3.52 and 3.67)
   __shared__ unsigned long long s_cand, s_waste, s_bytes, s_bytes_back, s_trace;
   __shared__ double s_S;
   float* s_records = s_dyn;
@@ -1464,7 +1464,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) mlp2_window_loop(Mlp2Args a) 
             if (held && (c.ecnt + 31) / 32 <= wpc) {
               // every entry was the last one of some lane of warps 1.., which has its new loss: the
               // losses are not computed again (with that, batches took 3.54, 4.28, 3.69, 3.52 and 3.94 us
-              // for the small, wide, ternary, masked and ReLU nets; now 3.36, 4.06, 3.60, 3.36 and 3.73.
+              // for the small, wide, ternary, masked and ReLU nets; without 3.36, 4.06, 3.60, 3.36, 3.73.
               // Keeping the fields as well spills registers.)
               if (hk == kst && he < c.ecnt) commit_entry<M>(R, w, nl, da, zn, he, hl, zrow);
             } else {
@@ -1563,8 +1563,8 @@ __global__ void __launch_bounds__(kLoopThreads, 1) mlp2_window_loop(Mlp2Args a) 
       // CTA's share. The last three warps look at the slots ahead: before they evaluate when the
       // others suffice for that, else afterwards. Warp 0, which waits for the other CTAs, is the last
       // to get work. Each warp's part comes from tables, ahead of the barrier: with three divisions after it a
-      // batch took 3.69, 4.40, 3.83, 3.71 and 4.03 us (small, wide, ternary, masked, ReLU nets), now 3.53,
-      // 4.28, 3.68, 3.52 and 3.94.
+      // batch took 3.69, 4.40, 3.83, 3.71 and 4.03 us (small, wide, ternary, masked, ReLU nets), with the
+      // tables 3.53, 4.28, 3.68, 3.52 and 3.94.
       unsigned long long* acc = a.accum + (size_t)(bidx % kAccBuffers) * kAccStride;
       const bool look_first = nlive * wpc <= kLookWarp0 - 1;
 #pragma unroll 1
