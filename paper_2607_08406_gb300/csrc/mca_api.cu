@@ -467,9 +467,9 @@ mca::DeepArgs deep_args(mca_handle* h) {
   }
   a.tc = h->tc ? 1 : 0;
   a.tc_f16 = h->tc_f16 ? 1 : 0;
-  if (h->tc_f16) {                   // the dense weights' bound to at most 2^15
+  if (h->tc_f16) {                   // the scale of the weight images: their bound to at most 2^15
     int e = 0;
-    std::frexp(h->wbound, &e);
+    std::frexp(h->wsplit, &e);
     e = std::max(-90, e);
     a.tc_wscale = std::ldexp(1.0f, 15 - e);
     a.tc_dscale = std::ldexp(1.0f / mca::kDeepDScale, e - 15);
@@ -499,6 +499,15 @@ mca::DeepArgs deep_args(mca_handle* h) {
   return a;
 }
 
+// The weight images of the dense chain, scaled for weights up to h->wbound. The only place that changes
+// the scale deep_args hands to the kernels.
+mca_status deep_split(mca_handle* h) {
+  h->wsplit = h->wbound;
+  CUDA_TRY(h, mca::launch_deep_split(deep_args(h), h->stream));
+  h->launches += 1;
+  return MCA_OK;
+}
+
 // Full forward pass: every cached field, every sample's loss, and S (Section 2.4's cache).
 mca::TfmArgs tfm_args(mca_handle* h);
 
@@ -517,11 +526,11 @@ mca_status resync(mca_handle* h) {
     return MCA_OK;
   }
   if (h->deep) {
-    const mca::DeepArgs a = deep_args(h);
-    if (a.tc) {
-      CUDA_TRY(h, mca::launch_deep_split(a, h->stream));
-      h->launches += 1;
+    if (h->tc) {
+      const mca_status rc = deep_split(h);
+      if (rc != MCA_OK) return rc;
     }
+    const mca::DeepArgs a = deep_args(h);
     // With tanh layers throughout, one launch runs every layer after the first, a tile's activations
     // staying on chip from layer to layer, and the losses: 24 layers of 256 on 10000 samples took
     // 765 us as one product (and its operand images) per layer, 254 us as one chain.
@@ -1280,14 +1289,14 @@ mca_status mca_run(mca_handle* h, uint64_t n_trials, uint64_t seed, mca_run_stat
           h->ev_c_pending = false;
         }
       }
-      if (h->tc_f16 && ctl.kstar >= 0 && std::fabs(ctl.acc.neww) > h->wbound) {
-        // a kept weight beyond the operands' scale (perturbations): split again with a larger one
-        h->wbound = pow2_above(std::fabs(ctl.acc.neww));
+      if (h->tc_f16 && ctl.kstar >= 0 && std::fabs(ctl.acc.neww) > h->wsplit) {
+        // a kept weight beyond the images' scale (perturbations): split again with a larger one
+        h->wbound = std::max(h->wbound, pow2_above(std::fabs(ctl.acc.neww)));
+        const mca_status rc = deep_split(h);
+        if (rc != MCA_OK) return rc;
         const uint64_t sd = a.seed;
         a = deep_args(h);
         a.seed = sd;
-        CUDA_TRY(h, mca::launch_deep_split(a, h->stream));
-        h->launches += 1;
       }
       if (h->tfm && ctl.kstar >= 0) {
         h->pmax = std::max(h->pmax, std::fabs(ctl.acc.neww));
@@ -1757,8 +1766,6 @@ mca_status mca_run_channels(mca_handle* h, uint64_t n_trials, uint64_t seed, int
                                 h->stream));
     CUDA_TRY(h, cudaStreamSynchronize(h->stream));
   }
-  for (int m = 0; m < L; ++m)         // He values
-    h->wbound = std::max(h->wbound, pow2_above((float)std::sqrt(6.0 / (double)h->layers[m].n_in)));
   std::vector<int> node(L + 1);
   std::vector<float> oldw(L), neww(L);
   std::vector<float*> at(L);
@@ -1766,6 +1773,9 @@ mca_status mca_run_channels(mca_handle* h, uint64_t n_trials, uint64_t seed, int
   mca_status rc = read_state(h, &ds);
   if (rc != MCA_OK) return rc;
   double S = ds.S;
+  if (h->tc_f16 && n_trials > 0 && scheme == MCA_CHANNEL_HE)
+    for (int m = 1; m + 1 < L; ++m)   // He values in the dense layers; the first trial's resync splits
+      h->wbound = std::max(h->wbound, pow2_above((float)std::sqrt(6.0 / (double)h->layers[m].n_in)));
   for (uint64_t t = 0; t < n_trials; ++t) {
     const uint64_t tau = h->tau;
     for (int m = 0; m <= L; ++m) {

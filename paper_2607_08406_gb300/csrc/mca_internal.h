@@ -446,8 +446,9 @@ struct mca_handle {
   bool deep = false;
   bool tc = false;                   // deep: dense chain on the tensor cores; Transformer: the
                                      // tensor-core sequence kernels
-  bool tc_f16 = false;               // deep: the chain's operands as fp16 parts, scaled for weights
-  float wbound = 1.0f;               //   of magnitude at most wbound
+  bool tc_f16 = false;               // deep: the chain's operands as fp16 parts
+  float wbound = 1.0f;               //   bound of the dense weights' magnitude
+  float wsplit = 1.0f;               //   the bound that the weight images are scaled for
   std::vector<float*> Z;
   std::vector<float*> whi;           // split-weight images of layers 1 .. L-2 (tensor-core chain)
   float* ell = nullptr;

@@ -5,6 +5,7 @@ import dataclasses
 import numpy as np
 import pytest
 
+from oracle import mca_oracle as O
 from paper_2607_08406_gb300 import workloads as W
 
 from parity import TIE_REL, compare, forced_from_oracle, oracle_trace
@@ -30,3 +31,41 @@ def test_deep_perturbations_beyond_the_operand_scale(gpu_lib, scale, delta):
     gpu_lib.mca_resync(h)
     assert gpu_lib.mca_loss(h) == pytest.approx(cached, rel=TIE_REL)
     assert cached == pytest.approx(S / wl.N, rel=TIE_REL)
+
+
+def _check_candidates(gpu_lib, wl, h, new_amp=1.0, n=32):
+    """dS of n candidates in the layers ahead of a dense one, against the fp64 oracle."""
+    flat = gpu_lib.mca_get_params(h, wl.n_params)
+    rng = np.random.default_rng(11)
+    off = np.cumsum([0] + [ly.n_in * ly.n_out for ly in wl.layers])
+    idx = np.concatenate([rng.integers(off[0], off[1], n // 2),
+                          rng.integers(off[1], off[2], n // 2)]).astype(np.uint32)
+    new = rng.uniform(-new_amp, new_amp, n).astype(np.float32)
+    got = gpu_lib.mca_eval_candidates(h, idx, new)
+    X = wl.X.T.astype(np.float64)
+
+    def total(f):
+        return O.total_loss(O.Params(wl.layers, f), X, wl.y, wl.loss)
+
+    S = total(flat)
+    for k in range(n):
+        f = flat.copy()
+        f[idx[k]] = new[k]
+        want = total(f) - S
+        assert abs(got[k] - want) <= TIE_REL * max(S, S + want), k
+    return got
+
+
+def test_channel_call_without_trials_changes_nothing(gpu_lib):
+    """The operands' scale may only grow together with the images: a channel call with no trials on
+    weights below the He amplitude leaves every loss change as it was."""
+    wl = W.mlp_deep(N=300, width=256, depth=4, n_trials=16, K=16)
+    wl.domain = dataclasses.replace(wl.domain, op="perturb", delta=0.01)
+    h = gpu_lib.create_from_workload(wl)
+    before = _check_candidates(gpu_lib, wl, h)
+    for scheme in ("he", "zero"):
+        acc, dS = gpu_lib.mca_run_channels(h, 0, 3, scheme)
+        assert len(acc) == 0 and len(dS) == 0
+        assert np.array_equal(_check_candidates(gpu_lib, wl, h), before)
+    gpu_lib.mca_run_channels(h, 3, 3, "he")
+    _check_candidates(gpu_lib, wl, h)
