@@ -466,8 +466,8 @@ mca::DeepArgs deep_args(mca_handle* h) {
     a.whi[l] = h->tc && l >= 1 && l + 1 < a.L ? h->whi[l - 1] : nullptr;
   }
   a.tc = h->tc ? 1 : 0;
-  a.tc_f16 = h->tc_f16 ? 1 : 0;
-  if (h->tc_f16) {                   // the scale of the weight images: their bound to at most 2^15
+  a.tc_f16 = h->split_f16 ? 1 : 0;
+  if (h->split_f16) {                // the scale of the weight images: their bound to at most 2^15
     int e = 0;
     std::frexp(h->wsplit, &e);
     e = std::max(-90, e);
@@ -499,12 +499,35 @@ mca::DeepArgs deep_args(mca_handle* h) {
   return a;
 }
 
-// The weight images of the dense chain, scaled for weights up to h->wbound. The only place that changes
-// the scale deep_args hands to the kernels.
+// The weight images of the dense chain, in the parts and for the bound that the handle wants now. The only
+// place that changes what deep_args tells the kernels of them.
 mca_status deep_split(mca_handle* h) {
   h->wsplit = h->wbound;
+  h->split_f16 = h->parts_f16;
   CUDA_TRY(h, mca::launch_deep_split(deep_args(h), h->stream));
   h->launches += 1;
+  return MCA_OK;
+}
+
+// Dense weights up to `bound`, a power of two, are to come: the next split takes it for its scale, or the tf32
+// parts if that leaves too many of the present weights out of range.
+mca_status deep_raise(mca_handle* h, float bound) {
+  if (bound <= h->wbound) return MCA_OK;
+  h->wbound = bound;
+  if (!h->parts_f16) return MCA_OK;
+  int* dflag = nullptr;
+  int wide = 0;
+  cudaError_t e = cudaMalloc(&dflag, sizeof(int));
+  if (e == cudaSuccess) e = cudaMemsetAsync(dflag, 0, sizeof(int), h->stream);
+  if (e == cudaSuccess)
+    e = mca::launch_deep_wide(deep_args(h), nullptr, 0.0f, 0.5f * bound, dflag, h->stream);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(&wide, dflag, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+  cudaFree(dflag);
+  CUDA_TRY(h, e);
+  h->launches += 1;
+  if (wide) h->parts_f16 = false;
   return MCA_OK;
 }
 
@@ -534,7 +557,7 @@ mca_status resync(mca_handle* h) {
     // With tanh layers throughout, one launch runs every layer after the first, a tile's activations
     // staying on chip from layer to layer, and the losses: 24 layers of 256 on 10000 samples took
     // 765 us as one product (and its operand images) per layer, 254 us as one chain.
-    const bool chain = h->tc_f16 && h->layers[0].act == MCA_ACT_TANH && forward_tc_enabled();
+    const bool chain = a.tc_f16 && h->layers[0].act == MCA_ACT_TANH && forward_tc_enabled();
     const int by_layer = chain ? 1 : a.L;
     for (int l = 0; l < by_layer; ++l) {
       if (h->gimg && forward_tc_layer(h->layers, (size_t)l, h->Np)) {
@@ -595,10 +618,10 @@ mca_status load_params(mca_handle* h, const float* params, const signed char* co
   const float* src = pdev ? params : tmp;
   const signed char* csrc = codes ? (cdev ? codes : ctmp) : nullptr;
   // [0] a non-finite value; [1] the largest magnitude of a deep net's dense weights, or of the
-  // Transformer's parameters
+  // Transformer's parameters; [2] dense weights out of the fp16 parts' range
   int* dflag = nullptr;
-  cudaError_t e = cudaMalloc(&dflag, 2 * sizeof(int));
-  if (e == cudaSuccess) e = cudaMemsetAsync(dflag, 0, 2 * sizeof(int), h->stream);
+  cudaError_t e = cudaMalloc(&dflag, 3 * sizeof(int));
+  if (e == cudaSuccess) e = cudaMemsetAsync(dflag, 0, 3 * sizeof(int), h->stream);
   if (e == cudaSuccess) e = mca::launch_count_nonfinite(src, P, dflag, h->stream);
   if (e == cudaSuccess && h->tc_f16)
     e = mca::launch_abs_max(src + h->off[1], h->off[h->layers.size() - 1] - h->off[1], dflag + 1,
@@ -611,7 +634,18 @@ mca_status load_params(mca_handle* h, const float* params, const signed char* co
                                n, h->w_eff[l], h->code[l], h->wfix[l], h->stream);
     h->launches++;
   }
-  int hflag[2] = {0, 0};
+  // the dense weights' magnitude is at most max(their largest now times sc, reach)
+  float sc = 1.0f, reach = 0.0f;
+  if (h->tc_f16) {
+    for (const mca_layer& L : h->layers)   // ternary layers hold codes
+      if (L.wkind == MCA_W_TERNARY_I8) sc = std::max(sc, std::fabs(L.scale));
+    reach = h->dom.op == MCA_OP_REPLACE ? std::max(std::fabs(h->dom.lo), std::fabs(h->dom.hi))
+                                        : std::fabs(h->dom.delta);
+    if (e == cudaSuccess)
+      e = mca::launch_deep_wide(deep_args(h), dflag + 1, sc, reach, dflag + 2, h->stream);
+    h->launches++;
+  }
+  int hflag[3] = {0, 0, 0};
   if (e == cudaSuccess) e = cudaMemcpyAsync(hflag, dflag, sizeof(hflag), cudaMemcpyDeviceToHost,
                                             h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
@@ -624,13 +658,11 @@ mca_status load_params(mca_handle* h, const float* params, const signed char* co
   std::memcpy(&top, &hflag[1], sizeof(top));
   h->pmax = top;
   if (h->tc_f16) {
-    float sc = 1.0f;                 // ternary layers hold codes
+    h->wbound = pow2_above(std::max(top * sc, reach));
+    h->parts_f16 = hflag[2] == 0;
     for (const mca_layer& L : h->layers)
-      if (L.wkind == MCA_W_TERNARY_I8) sc = std::max(sc, std::fabs(L.scale));
-    top *= sc;
-    if (h->dom.op == MCA_OP_REPLACE)
-      top = std::max(top, std::max(std::fabs(h->dom.lo), std::fabs(h->dom.hi)));
-    h->wbound = pow2_above(top);
+      if (L.wkind == MCA_W_TERNARY_I8 && std::fabs(L.scale) < std::ldexp(h->wbound, -mca::kWideGap))
+        h->parts_f16 = false;
   }
   return MCA_OK;
 }
@@ -1289,10 +1321,11 @@ mca_status mca_run(mca_handle* h, uint64_t n_trials, uint64_t seed, mca_run_stat
           h->ev_c_pending = false;
         }
       }
-      if (h->tc_f16 && ctl.kstar >= 0 && std::fabs(ctl.acc.neww) > h->wsplit) {
-        // a kept weight beyond the images' scale (perturbations): split again with a larger one
-        h->wbound = std::max(h->wbound, pow2_above(std::fabs(ctl.acc.neww)));
-        const mca_status rc = deep_split(h);
+      if (a.tc_f16 && ctl.kstar >= 0 && ctl.acc.layer >= 1 && ctl.acc.layer + 1 < a.L &&
+          std::fabs(ctl.acc.neww) > h->wsplit) {
+        // a kept dense weight beyond the images' scale (perturbations): split again with a larger one
+        mca_status rc = deep_raise(h, pow2_above(std::fabs(ctl.acc.neww)));
+        if (rc == MCA_OK) rc = deep_split(h);
         if (rc != MCA_OK) return rc;
         const uint64_t sd = a.seed;
         a = deep_args(h);
@@ -1774,8 +1807,10 @@ mca_status mca_run_channels(mca_handle* h, uint64_t n_trials, uint64_t seed, int
   if (rc != MCA_OK) return rc;
   double S = ds.S;
   if (h->tc_f16 && n_trials > 0 && scheme == MCA_CHANNEL_HE)
-    for (int m = 1; m + 1 < L; ++m)   // He values in the dense layers; the first trial's resync splits
-      h->wbound = std::max(h->wbound, pow2_above((float)std::sqrt(6.0 / (double)h->layers[m].n_in)));
+    for (int m = 1; m + 1 < L; ++m) {   // He values in the dense layers; the first trial's resync splits
+      rc = deep_raise(h, pow2_above((float)std::sqrt(6.0 / (double)h->layers[m].n_in)));
+      if (rc != MCA_OK) return rc;
+    }
   for (uint64_t t = 0; t < n_trials; ++t) {
     const uint64_t tau = h->tau;
     for (int m = 0; m <= L; ++m) {

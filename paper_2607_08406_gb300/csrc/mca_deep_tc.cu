@@ -9,7 +9,8 @@
 //   D = A_lo W_hi^T + A_hi W_lo^T + A_hi W_hi^T      (the A_lo W_lo^T term, ~2^-22 relative, dropped)
 // Tanh layers use fp16 parts (kind::f16, K = 16 per MMA): |change| <= 2 and the largest weight's
 // magnitude are scaled by powers of two to at most 2^15, so that an element x is represented to 2^-22 of
-// itself or 2^-40 of the largest, whichever is larger, and D is scaled back exactly. Layers whose
+// itself or 2^-40 of the largest, whichever is larger, and D is scaled back exactly. Weights of which
+// too many lie that far below the largest (deep_wide_kernel), layers whose
 // changes have no bound (ReLU, GELU, identity) or another function use tf32 parts (K = 8 per MMA,
 // the same time per MMA, hence half the rate).
 //
@@ -644,7 +645,34 @@ __global__ void deep_split_kernel(DeepArgs a) {
     deep_tc_image_store(a, m, e / kTcW, e % kTcW, a.w[m][e]);
 }
 
+// One warp per row of a dense layer: are more than wide_allowance of its weights below 2^-kWideGap of the
+// bound? (Masked layers: of the weights behind the masks.)
+__global__ void deep_wide_kernel(DeepArgs a, const int* top, float sc, float floor, int* out) {
+  const int m = blockIdx.y + 1, lane = threadIdx.x & 31;
+  const int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (m > a.L - 2 || r >= kTcW) return;
+  const float b = fmaxf(floor, top ? __int_as_float(*top) * sc : 0.0f);
+  const int limit = (__float_as_int(b) >> 23) + 1 - kWideGap;   // exponents below it
+  const float* w = (a.wk[m] == MCA_W_MASKED_FP32 ? a.wfix[m] : a.w[m]) + (size_t)r * kTcW;
+  unsigned int n = 0, low = 0;
+#pragma unroll
+  for (int k = lane; k < kTcW; k += 32) {
+    const float v = fabsf(w[k]);
+    n += v != 0.0f;
+    low += v != 0.0f && (__float_as_int(v) >> 23) < limit;
+  }
+  n = __reduce_add_sync(0xffffffffu, n);
+  low = __reduce_add_sync(0xffffffffu, low);
+  if (lane == 0 && low > wide_allowance(n)) *out = 1;
+}
+
 }  // namespace
+
+cudaError_t launch_deep_wide(const DeepArgs& a, const int* top, float sc, float floor, int* out,
+                             cudaStream_t s) {
+  deep_wide_kernel<<<dim3(kTcW / 8, a.L - 2), 256, 0, s>>>(a, top, sc, floor, out);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_deep_split(const DeepArgs& a, cudaStream_t s) {
   if (a.L < 3) return cudaSuccess;

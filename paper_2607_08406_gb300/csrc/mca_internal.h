@@ -179,6 +179,12 @@ constexpr int kDeepThreads = 256;
 constexpr int kDeepMaxWidth = 256; // widths of the layers inside the dense chain
 constexpr int kDeepKC = 16;        // weight-tile depth of the chain GEMM
 constexpr float kDeepDScale = 16384.0f;   // tanh changes (at most 2) as fp16 operands: scale
+// Two fp16 parts of a value hold its 22 leading bits, like two tf32 parts, down to 2^-17 of the power of two
+// that its operand is scaled for; below, their error is absolute, 2^-40 of that power. So an operand is
+// taken as fp16 parts only while at most wide_allowance of a row's n non-zero entries lie below 2^-17:
+// of uniform values 2^-17 do, 0.03 in a row of 256 weights of +-0.1 under a bound of 2.
+constexpr int kWideGap = 17;
+constexpr unsigned int wide_allowance(unsigned int n) { return 3u + n / 2048u; }
 constexpr int kDeepScrSlots = 16;  // candidates whose fields the tensor-core evaluation keeps
 constexpr float kTfmF16Max = 4.0f;   // largest parameter magnitude of the fp16 Transformer kernels
 constexpr int kTfmScrSlots = 16;   // candidates whose residual streams the evaluation keeps
@@ -254,6 +260,10 @@ cudaError_t launch_deep_commit(const DeepArgs& a, cudaStream_t s);  // grid ntil
 cudaError_t launch_deep_forward_layer(const DeepArgs& a, int l, cudaStream_t s);
 cudaError_t launch_deep_losses(const DeepArgs& a, cudaStream_t s);
 cudaError_t launch_deep_split(const DeepArgs& a, cudaStream_t s);     // W_hi / W_lo of all layers
+// *out = 1 if the dense weights are out of the fp16 parts' range under the bound pow2_above(max(*top
+// sc, floor)); top: bits of a float >= 0, or null. (*out is left alone otherwise.)
+cudaError_t launch_deep_wide(const DeepArgs& a, const int* top, float sc, float floor, int* out,
+                             cudaStream_t s);
 cudaError_t launch_deep_eval_tc(const DeepArgs& a, cudaStream_t s);   // grid (Kb, ntiles)
 cudaError_t launch_deep_commit_tc(const DeepArgs& a, cudaStream_t s); // grid ntiles
 cudaError_t launch_deep_forward_tc(const DeepArgs& a, cudaStream_t s);  // grid ntiles
@@ -446,9 +456,12 @@ struct mca_handle {
   bool deep = false;
   bool tc = false;                   // deep: dense chain on the tensor cores; Transformer: the
                                      // tensor-core sequence kernels
-  bool tc_f16 = false;               // deep: the chain's operands as fp16 parts
-  float wbound = 1.0f;               //   bound of the dense weights' magnitude
-  float wsplit = 1.0f;               //   the bound that the weight images are scaled for
+  // deep: the chain's operands may be fp16 parts (tanh layers); the bound of the dense weights' magnitude,
+  // and whether the weights are in the range of fp16 parts under it; both as the weight images
+  // were split, which is what the kernels are told
+  bool tc_f16 = false;
+  float wbound = 1.0f, wsplit = 1.0f;
+  bool parts_f16 = false, split_f16 = false;
   std::vector<float*> Z;
   std::vector<float*> whi;           // split-weight images of layers 1 .. L-2 (tensor-core chain)
   float* ell = nullptr;

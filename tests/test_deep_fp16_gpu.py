@@ -69,3 +69,40 @@ def test_channel_call_without_trials_changes_nothing(gpu_lib):
         assert np.array_equal(_check_candidates(gpu_lib, wl, h), before)
     gpu_lib.mca_run_channels(h, 3, 3, "he")
     _check_candidates(gpu_lib, wl, h)
+
+
+@pytest.mark.parametrize("case", ["outlier", "domain", "perturb_outlier", "he_over_tiny"])
+def test_deep_weights_of_a_wide_range(gpu_lib, case):
+    """Weights far below the scale of the fp16 operands (one huge dense weight, a wide replacement domain,
+    a step that makes one weight huge, He values over tiny weights) take the tf32 parts."""
+    wl = W.mlp_deep(N=300, width=256, depth=4, n_trials=16, K=16)
+    dense = wl.layers[0].n_in * 256
+    if case == "outlier":
+        wl.init[dense + 256 * 7 + 3] = np.float32(1e10)
+        wl.domain = dataclasses.replace(wl.domain, op="perturb", delta=0.01)
+        h = gpu_lib.create_from_workload(wl)
+    elif case == "domain":
+        wl.domain = dataclasses.replace(wl.domain, lo=-2.0 ** 31, hi=2.0 ** 31)
+        h = gpu_lib.create_from_workload(wl)
+    elif case == "perturb_outlier":
+        wl.domain = dataclasses.replace(wl.domain, op="perturb", delta=1e11)
+        h = gpu_lib.create_from_workload(wl, trace_cap=40)
+        tau = np.arange(40, dtype=np.uint64)
+        gpu_lib.mca_force_decisions(h, tau, tau % 2 == 0)
+        gpu_lib.mca_run(h, 40, 3)
+        moved = np.abs(gpu_lib.mca_get_params(h, wl.n_params)[dense:dense + 256 * 256 * 3]) > 1e8
+        assert moved.any()
+    else:
+        wl.init = (wl.init * np.float32(2.0 ** -30)).astype(np.float32)
+        wl.init[:dense] *= np.float32(2.0 ** 30)
+        wl.domain = dataclasses.replace(wl.domain, op="perturb", delta=2.0 ** -31)
+        h = gpu_lib.create_from_workload(wl)
+        gpu_lib.mca_force_decisions(h, [0, 1], [True, False])
+        gpu_lib.mca_run_channels(h, 2, 5, "he")
+        st = gpu_lib.mca_get_params(h, wl.n_params)
+        assert (np.abs(st[dense:dense + 256 * 256 * 3]) > 1e-4).sum() == 3
+    assert gpu_lib.mca_get_stats(h)["tensor_cores"] == 1
+    _check_candidates(gpu_lib, wl, h)
+    cached = gpu_lib.mca_loss(h)
+    gpu_lib.mca_resync(h)
+    assert gpu_lib.mca_loss(h) == pytest.approx(cached, rel=TIE_REL)
