@@ -257,21 +257,28 @@ __device__ __forceinline__ float act_compact(float z, float g, int act_runtime) 
   }
 }
 
-// Per-sample loss of the output fields z[0..C) with label y.
+// Cross-entropy from the largest field m, the sum of e^(field - m) and the label's field.
+__device__ __forceinline__ float ce_loss(float m, float sum, float zy) {
+  return __fsub_rn(__fadd_rn(__logf(sum), m), zy);
+}
+
+// Per-sample loss of the output fields z[0..C) with label y. Fields of even and of odd index are added
+// apart and then together, the order of the windowed loop's pairs of fields: the loss of the same fields
+// is the same number wherever it is computed, and a change that reaches no field has dS = 0 exactly.
 template <int ACT2, int LOSS, int MAXC>
 __device__ __forceinline__ float sample_loss(const float (&z)[MAXC], int C, int y, float g2,
                                              int act2_rt, int loss_rt) {
   const int loss = LOSS < 0 ? loss_rt : LOSS;
   if (loss == MCA_LOSS_MSE_ONEHOT) {
-    float s = 0.0f;
+    float s[2] = {0.0f, 0.0f};
 #pragma unroll
     for (int k = 0; k < MAXC; ++k) {
       if (k < C) {
         const float d = act_compact<ACT2>(z[k], g2, act2_rt) - (k == y ? 1.0f : 0.0f);
-        s = fmaf(d, d, s);
+        s[k & 1] = fmaf(d, d, s[k & 1]);
       }
     }
-    return s;
+    return s[0] + s[1];
   }
   float a[MAXC];
   float m = -INFINITY;
@@ -282,15 +289,15 @@ __device__ __forceinline__ float sample_loss(const float (&z)[MAXC], int C, int 
       m = fmaxf(m, a[k]);
     }
   }
-  float s = 0.0f, ay = 0.0f;
+  float s[2] = {0.0f, 0.0f}, ay = 0.0f;
 #pragma unroll
   for (int k = 0; k < MAXC; ++k) {
     if (k < C) {
-      s += exp_fast(a[k] - m);
+      s[k & 1] += exp_fast(a[k] - m);
       if (k == y) ay = a[k];
     }
   }
-  return (__logf(s) + m) - ay;
+  return ce_loss(m, s[0] + s[1], ay);
 }
 
 // ------------------------------------------------------------------------------------------------

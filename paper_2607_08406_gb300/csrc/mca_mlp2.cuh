@@ -776,7 +776,8 @@ struct VRecs {
   }
 };
 
-// Loss of the fields z with label y; zy: field y; onehot: -[k == y] per field (MSE).
+// Loss of the fields z with label y; zy: field y; onehot: -[k == y] per field (MSE). The same operations on
+// each field and the same order of sums as sample_loss: records come from it in the forward pass.
 template <int ACT2, int LOSS, int M>
 __device__ __forceinline__ float vloss(const Mlp2Args& a, const float2 (&z)[M / 2], int y, float zy,
                                        const float* onehot) {
@@ -790,7 +791,7 @@ __device__ __forceinline__ float vloss(const Mlp2Args& a, const float2 (&z)[M / 
       const float2 t = mul2(add2(z[q], make_float2(-m, -m)), make_float2(kLog2e, kLog2e));
       s = add2(s, make_float2(ex2_ftz(t.x), ex2_ftz(t.y)));
     }
-    return (__logf(s.x + s.y) + m) - zy;
+    return ce_loss(m, s.x + s.y, zy);
   } else if constexpr (ACT2 == MCA_ACT_SIGMOID && LOSS == MCA_LOSS_MSE_ONEHOT) {
     const float* oh = onehot + 16 * y;
     float2 s = make_float2(0.0f, 0.0f);

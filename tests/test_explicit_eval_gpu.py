@@ -60,3 +60,45 @@ def test_explicit_candidates(gpu_lib, C, hidden, out, loss, N, H, n, grid):
         assert np.array_equal(rec["dS"].astype(np.float64), again)
         assert np.all(np.abs(rec["S"] - S) <= TIE_REL * S)
         gpu_lib.mca_run(h, 50, wl.seed)
+
+
+@pytest.mark.parametrize("C,hidden,out,loss", [
+    (10, "tanh", "identity", "softmax_ce"),
+    (10, "tanh", "sigmoid", "mse_onehot"),
+    (7, "gaussian", "sigmoid", "mse_onehot"),
+    (13, "relu", "identity", "softmax_ce"),
+    (10, "gelu", "tanh", "mse_onehot"),
+])
+def test_changes_that_reach_no_output_field_are_zero(gpu_lib, C, hidden, out, loss):
+    """A hidden neuron without outgoing weights: its activation changes, no output field does, and the loss
+    change is exactly 0 (a neutral trial), in the evaluation kernel and in the windowed loop, before
+    and after commits."""
+    N, D, H = 3001, 20, 9
+    rng = np.random.default_rng(C)
+    layers = [W.Layer(D, H, hidden, 0.7), W.Layer(H, C, out)]
+    init = W.uniform_init(rng, layers, 0.3)
+    init[D * H:].reshape(C, H)[:, ::2] = 0.0            # neurons 0, 2, ..: no outgoing weight
+    wl = W.MLPWorkload("neutral", layers, loss, W.synth_images(rng, N, D, 0.4),
+                       rng.integers(0, C, N).astype(np.int32), init, 300, 16)
+    h = gpu_lib.create_from_workload(wl, trace_cap=300)
+    idx = np.array([j * D + i for j in range(0, H, 2) for i in range(0, D, 3)], np.uint32)
+    new = rng.uniform(-1, 1, len(idx)).astype(np.float32)
+    assert np.all(gpu_lib.mca_eval_candidates(h, idx, new) == 0.0)
+    gpu_lib.mca_run(h, 300, 5)
+    tr = gpu_lib.mca_get_trace(h, 300)
+    live = init[D * H:].reshape(C, H) != 0.0
+    seen = 0
+    for t in tr:
+        i = int(t["idx"])
+        if i < D * H:
+            if not live[:, i // D].any():
+                assert t["dS"] == 0.0 and t["accept"] == 1
+                seen += 1
+        elif t["accept"]:
+            live[(i - D * H) // H, (i - D * H) % H] = t["new_w"] != 0.0
+    assert seen > 15 and tr["accept"].sum() > 60
+    got = gpu_lib.mca_get_params(h, wl.n_params)[D * H:].reshape(C, H)
+    dead = [j for j in range(H) if not got[:, j].any()]
+    idx = np.array([j * D + 1 for j in dead], np.uint32)
+    if dead:
+        assert np.all(gpu_lib.mca_eval_candidates(h, idx, np.full(len(idx), 0.9, np.float32)) == 0.0)
