@@ -805,8 +805,9 @@ TfmMem tfm_plan(const mca_tfm_spec& t, long long B, int trace_cap, bool tc, int 
 
 // The Transformer's parameters, and those of any trial drawn now, are within the range of the fp16
 // operands. Perturbations: the decision of the batch in flight may move a parameter by delta before
-// a trial moves it by delta again.
+// a trial moves it by delta again. A Gaussian feed-forward activation exp(-g u^2) with g < 0 has no bound.
 bool tfm_f16_range(const mca_handle* h) {
+  if (h->tspec.act == MCA_ACT_GAUSSIAN && h->tspec.act_param < 0.0f) return false;
   const bool move = h->dom.op == MCA_OP_PERTURB;
   const float step = move ? 2.0f * std::fabs(h->dom.delta) : 0.0f;
   const float drawn = move ? 0.0f : std::max(std::fabs(h->dom.lo), std::fabs(h->dom.hi));

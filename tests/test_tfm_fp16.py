@@ -68,6 +68,29 @@ def test_tfm_perturbations_leave_the_fp16_range(gpu_lib):
     assert np.array_equal(gpu_lib.mca_get_params(h, wl.n_params), flat)
 
 
+@pytest.mark.gpu
+def test_tfm_growing_feed_forward_activation(gpu_lib):
+    """exp(-g u^2) with g < 0 has no bound that the fp16 operands could hold."""
+    spec = W.TfmSpec(n_layer=1, d_ff=128, act="gaussian", act_param=-0.25)
+    wl = W.char_transformer(batch=2, text_len=4000, spec=spec, n_trials=8, K=8)
+    rng = np.random.default_rng(1)
+    wl.init, o = wl.init.copy(), 0
+    for name, shape in spec.blocks():
+        m = int(np.prod(shape))
+        if name == "b0.b1":
+            wl.init[o:o + 3] = np.float32(3.0)
+        if name == "b0.w1":                          # u up to about 8: activations up to 1e7
+            wl.init[o:o + m] = rng.normal(0.0, 0.2, m)
+        if name == "b0.w2":
+            wl.init[o:o + m] = rng.normal(0.0, 1e-3, m)
+        o += m
+    flat = wl.init.astype(np.float64)
+    S0 = T.tfm_seq_losses(spec, flat, wl.tokens).sum()
+    h = gpu_lib.create_from_tfm_workload(wl)
+    assert gpu_lib.mca_get_stats(h)["tensor_cores"] == 1
+    assert gpu_lib.mca_loss(h) * 2 * spec.ctx == pytest.approx(S0, rel=TIE_REL)
+
+
 PROBE = r"""
 #include <cstdio>
 #include <cstdlib>
