@@ -149,7 +149,8 @@ typedef struct {
   uint64_t batches;
   uint64_t wasted;         /* candidates evaluated after the accepted one in their batch */
   uint64_t forced;         /* decisions taken from mca_force_decisions */
-  uint64_t resyncs;
+  uint64_t resyncs;        /* full recomputations: each resync_period, mca_resync, and where growing
+                              Transformer parameters take the trials to other kernels */
   uint64_t launches;       /* kernels this handle launched */
   uint64_t tau;            /* next trial counter */
   double S;                /* current loss sum */
@@ -245,8 +246,8 @@ mca_status mca_tfm_workspace_size(const mca_tfm_spec* spec, int64_t n_seq, const
  * perturbation). mca_loss reports S / (n_seq * ctx). Errors as for mca_create.
  * Kernels: with ctx 64, d_model 128, 4 heads, d_ff a multiple of 128 up to 1024, vocab <= 128 and an
  * even n_seq the sequences run on the tensor-core kernels (tcgen05, three MMAs per fp32 product, of
- * fp16 parts while every parameter is at most 4 in magnitude and of tf32 parts otherwise, two
- * sequences per CTA);
+ * fp16 parts while every parameter, and any that a trial may draw, is at most 4 in magnitude and of tf32
+ * parts otherwise, two sequences per CTA);
  * for other shapes, or when the process environment has MCA_TFM_TENSOR_CORES=0, on the SIMT fp32
  * kernels. The variable is read by this call and by mca_tfm_workspace_size (the tensor-core kernels'
  * weight images are part of the workspace), so it must not change between the two. mca_run_stats

@@ -803,15 +803,22 @@ TfmMem tfm_plan(const mca_tfm_spec& t, long long B, int trace_cap, bool tc, int 
   return M;
 }
 
-// The Transformer's parameters, and those of any trial drawn now, are within the range of the fp16
-// operands. Perturbations: the decision of the batch in flight may move a parameter by delta before
-// a trial moves it by delta again. A Gaussian feed-forward activation exp(-g u^2) with g < 0 has no bound.
-bool tfm_f16_range(const mca_handle* h) {
+// Bound of the Transformer's parameters after `moves` more trials, the last one's own value included.
+float tfm_reach(const mca_handle* h, int moves) {
+  const mca_domain& d = h->dom;
+  float v = d.op == MCA_OP_PERTURB ? h->pmax : std::max(std::fabs(d.lo), std::fabs(d.hi));
+  for (int m = 0; m < moves && d.op == MCA_OP_PERTURB; ++m) v += std::fabs(d.delta);  // as the trials round
+  if (d.bound > 0.0f) v = std::min(v, d.bound);     // proposals beyond it are not evaluated
+  return std::max(h->pmax, v);
+}
+
+// Whether a trial runs on the fp16 kernels: the parameters, with any value it may draw, are within
+// their range. It follows from the trials before it alone (not from how they fell into batches), so that
+// the trajectory does not depend on the batch width. A Gaussian feed-forward activation exp(-g u^2)
+// with g < 0 has no bound.
+bool tfm_f16_range(const mca_handle* h, int moves = 1) {
   if (h->tspec.act == MCA_ACT_GAUSSIAN && h->tspec.act_param < 0.0f) return false;
-  const bool move = h->dom.op == MCA_OP_PERTURB;
-  const float step = move ? 2.0f * std::fabs(h->dom.delta) : 0.0f;
-  const float drawn = move ? 0.0f : std::max(std::fabs(h->dom.lo), std::fabs(h->dom.hi));
-  return h->pmax + step <= mca::kTfmF16Max && drawn <= mca::kTfmF16Max;
+  return tfm_reach(h, moves) <= mca::kTfmF16Max;
 }
 
 mca::TfmArgs tfm_args(mca_handle* h) {
@@ -873,6 +880,16 @@ mca::TfmArgs tfm_args(mca_handle* h) {
   return a;
 }
 
+// An accepted parameter of magnitude w. Where it takes the trials to the tf32 kernels, the cached state is
+// recomputed by them: loss changes compare losses that the same kernels computed.
+mca_status tfm_grow(mca_handle* h, float w) {
+  const bool f16 = tfm_f16_range(h);
+  h->pmax = std::max(h->pmax, w);
+  if (!h->tc || tfm_f16_range(h) == f16) return MCA_OK;
+  h->resyncs += 1;
+  return resync(h);
+}
+
 // Transformer tensor-core batches with the host one batch ahead of the decisions: the kernels of
 // batch i + 1 are enqueued before the host reads batch i's decision. The batch's first trial lives
 // on the device (the decision advances it by the trials it consumed), so the GPU does not wait for
@@ -922,8 +939,12 @@ mca_status run_tfm_pipelined(mca_handle* h, mca::TfmArgs ta, uint64_t n_trials) 
   if (rc != MCA_OK) return rc;
   for (int i = 0;; ++i) {
     NvtxRange nv_batch("mca batch (transformer, one ahead)");
-    rc = launch(i + 1);
-    if (rc != MCA_OK) return rc;
+    // not ahead where the decision in flight may take the next batch to other kernels
+    const bool ahead = tfm_f16_range(h, 1) == tfm_f16_range(h, 2);
+    if (ahead) {
+      rc = launch(i + 1);
+      if (rc != MCA_OK) return rc;
+    }
     const int p = i & 1;
     CUDA_TRY(h, cudaEventSynchronize(h->ev_p[p][2]));
     float ms_eval = 0.0f, ms_rest = 0.0f;
@@ -937,13 +958,20 @@ mca_status run_tfm_pipelined(mca_handle* h, mca::TfmArgs ta, uint64_t n_trials) 
       h->broken = true;
       return fail(h, MCA_ERR_NUMERIC, "non-finite loss change");
     }
-    if (ctl.kstar >= 0) h->pmax = std::max(h->pmax, std::fabs(ctl.acc.neww));
+    if (ctl.kstar >= 0) {
+      rc = tfm_grow(h, std::fabs(ctl.acc.neww));
+      if (rc != MCA_OK) return rc;
+    }
     done += (uint64_t)ctl.consumed;
     h->rate_acc = h->rate_acc * mca::kRateDecay + (ctl.kstar >= 0 ? 1.0f : 0.0f);
     h->rate_trials = h->rate_trials * mca::kRateDecay + (float)ctl.consumed;
     if (done >= n_trials) break;
+    if (!ahead) {
+      rc = launch(i + 1);
+      if (rc != MCA_OK) return rc;
+    }
   }
-  // the batch enqueued last starts at the run's end and does nothing; let it finish
+  // a batch enqueued ahead starts at the run's end and does nothing; let it finish
   CUDA_TRY(h, cudaStreamSynchronize(h->stream));
   h->tau += done;
   return MCA_OK;
@@ -1333,7 +1361,8 @@ mca_status mca_run(mca_handle* h, uint64_t n_trials, uint64_t seed, mca_run_stat
         a.seed = sd;
       }
       if (h->tfm && ctl.kstar >= 0) {
-        h->pmax = std::max(h->pmax, std::fabs(ctl.acc.neww));
+        const mca_status rc = tfm_grow(h, std::fabs(ctl.acc.neww));
+        if (rc != MCA_OK) return rc;
         ta.f16 = h->tc && tfm_f16_range(h) ? 1 : 0;
       }
       h->tau += (uint64_t)ctl.consumed;

@@ -52,20 +52,77 @@ def test_tfm_parameter_range(gpu_lib, layers, ff, vocab, big):
             assert abs(d - want) <= TIE_REL * max(S0, S0 + want)
 
 
-@pytest.mark.gpu
-def test_tfm_perturbations_leave_the_fp16_range(gpu_lib):
-    """A run whose parameters grow past the fp16 kernels' bound continues on the tf32 kernels."""
+def _growing(n, top=3.5, delta=0.45):
+    """A perturbing workload whose largest parameters grow past 4 - delta within n trials: some at
+    +-top."""
     spec = W.TfmSpec(n_layer=1, d_ff=128)
-    wl = W.char_transformer(batch=2, text_len=4000, spec=spec, n_trials=60, K=8)
-    wl.domain = dataclasses.replace(wl.domain, op="perturb", delta=1.2)
+    wl = W.char_transformer(batch=2, text_len=4000, spec=spec, n_trials=n, K=8)
+    wl.domain = dataclasses.replace(wl.domain, op="perturb", delta=delta)
+    rng = np.random.default_rng(2)
     wl.init = wl.init.copy()
-    wl.init[::97] = np.float32(1.5)
-    tr, flat, S = T.run_full_tfm(spec, wl.tokens, wl.init, 60, 1, wl.domain)
-    h = gpu_lib.create_from_tfm_workload(wl, trace_cap=60)
+    big = rng.random(wl.init.size) < 0.15
+    o = 0
+    for name, shape in spec.blocks():            # (not the matrices of the attention scores)
+        m = int(np.prod(shape))
+        if name[-2:] in ("wq", "wk", "bq", "bk"):
+            big[o:o + m] = False
+        o += m
+    wl.init[big] = (top * rng.choice([-1.0, 1.0], big.sum())).astype(np.float32)
+    return wl
+
+
+def _crossing(tr, init, domain):
+    """Trials ahead of which the largest parameter plus a step lies within 4, and accepted trials
+    on either side."""
+    top = float(np.abs(init).max())
+    inside = []
+    for k in range(len(tr["tau"])):
+        inside.append(top + domain.delta <= 4.0)
+        if tr["accept"][k]:
+            top = max(top, abs(float(np.float32(tr["new"][k]))))
+    inside = np.array(inside)
+    return inside, tr["accept"] & inside, tr["accept"] & ~inside
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("period", [0, 25])
+def test_tfm_perturbations_leave_the_fp16_range(gpu_lib, period):
+    """A run whose parameters grow past the fp16 kernels' bound continues on the tf32 kernels: with
+    batches enqueued one ahead, and in round trips (resync period). Accepted trials on both sides."""
+    n = 60
+    wl = _growing(n)
+    tr, flat, S = T.run_full_tfm(wl.spec, wl.tokens, wl.init, n, 1, wl.domain)
+    inside, before, after = _crossing(tr, wl.init, wl.domain)
+    assert 3 <= inside.sum() <= n - 20 and before.sum() >= 2 and after.sum() >= 5
+    h = gpu_lib.create_from_tfm_workload(wl, trace_cap=n, resync_period=period)
     gpu_lib.mca_force_decisions(h, *forced_from_oracle(tr))
-    gpu_lib.mca_run(h, 60, 1)
-    compare(gpu_lib.mca_get_trace(h, 60), tr)
+    st = gpu_lib.mca_run(h, n, 1)
+    assert st["resyncs"] == 1 + (n // period if period else 0)        # one for the change of kernels
+    compare(gpu_lib.mca_get_trace(h, n), tr)
     assert np.array_equal(gpu_lib.mca_get_params(h, wl.n_params), flat)
+    cached = gpu_lib.mca_loss(h)
+    gpu_lib.mca_resync(h)
+    assert gpu_lib.mca_loss(h) == pytest.approx(cached, rel=TIE_REL)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("top,delta", [(3.5, 0.45), (3.05, 0.45), (0.9, 0.15), (0.05, 0.8)])
+def test_tfm_trajectory_does_not_depend_on_the_batch_width(gpu_lib, top, delta):
+    """Perturbed parameters that cross 4 (fp16 to tf32 kernels) or powers of two below (the operands' scales)
+    on the way: the same trace, bit for bit, for every batch width and split of the run."""
+    n = 120
+    wl = _growing(n, top, delta)
+    out = []
+    for K, fixed, parts in ((1, True, (n,)), (16, True, (n,)), (5, False, (n,)), (64, False, (7, 40, n - 47))):
+        h = gpu_lib.create_from_tfm_workload(wl, trace_cap=n, K=K, fixed_K=fixed)
+        for m in parts:
+            gpu_lib.mca_run(h, m, 3)
+        out.append((gpu_lib.mca_get_trace(h, n), gpu_lib.mca_get_params(h, wl.n_params),
+                    gpu_lib.mca_loss(h)))
+    assert out[0][0]["accept"].sum() > 10
+    for o in out[1:]:
+        assert np.array_equal(o[0], out[0][0])
+        assert np.array_equal(o[1], out[0][1]) and o[2] == out[0][2]
 
 
 @pytest.mark.gpu
