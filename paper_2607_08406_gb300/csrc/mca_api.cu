@@ -515,17 +515,11 @@ mca_status deep_raise(mca_handle* h, float bound) {
   if (bound <= h->wbound) return MCA_OK;
   h->wbound = bound;
   if (!h->parts_f16) return MCA_OK;
-  int* dflag = nullptr;
   int wide = 0;
-  cudaError_t e = cudaMalloc(&dflag, sizeof(int));
-  if (e == cudaSuccess) e = cudaMemsetAsync(dflag, 0, sizeof(int), h->stream);
-  if (e == cudaSuccess)
-    e = mca::launch_deep_wide(deep_args(h), nullptr, 0.0f, 0.5f * bound, dflag, h->stream);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(&wide, dflag, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-  cudaFree(dflag);
-  CUDA_TRY(h, e);
+  CUDA_TRY(h, cudaMemsetAsync(h->flag, 0, sizeof(int), h->stream));
+  CUDA_TRY(h, mca::launch_deep_wide(deep_args(h), nullptr, 0.0f, 0.5f * bound, h->flag, h->stream));
+  CUDA_TRY(h, cudaMemcpyAsync(&wide, h->flag, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+  CUDA_TRY(h, cudaStreamSynchronize(h->stream));
   h->launches += 1;
   if (wide) h->parts_f16 = false;
   return MCA_OK;
@@ -533,10 +527,13 @@ mca_status deep_raise(mca_handle* h, float bound) {
 
 // Full forward pass: every cached field, every sample's loss, and S (Section 2.4's cache).
 mca::TfmArgs tfm_args(mca_handle* h);
+float tfm_level(const mca_handle* h, int moves);
+mca_status tfm_check_small(mca_handle* h);
 
 mca_status resync(mca_handle* h) {
   NvtxRange nv("mca resync");
   if (h->tfm) {
+    h->tfm_q = tfm_level(h, 1);
     const mca::TfmArgs a = tfm_args(h);
     if (a.tc) {
       CUDA_TRY(h, mca::launch_tfm_tc_split(a, h->stream));
@@ -664,7 +661,7 @@ mca_status load_params(mca_handle* h, const float* params, const signed char* co
       if (L.wkind == MCA_W_TERNARY_I8 && std::fabs(L.scale) < std::ldexp(h->wbound, -mca::kWideGap))
         h->parts_f16 = false;
   }
-  return MCA_OK;
+  return h->tfm && h->tc ? tfm_check_small(h) : MCA_OK;
 }
 
 mca_status read_state(mca_handle* h, DevState* out) {
@@ -812,13 +809,45 @@ float tfm_reach(const mca_handle* h, int moves) {
   return std::max(h->pmax, v);
 }
 
-// Whether a trial runs on the fp16 kernels: the parameters, with any value it may draw, are within
-// their range. It follows from the trials before it alone (not from how they fell into batches), so that
-// the trajectory does not depend on the batch width. A Gaussian feed-forward activation exp(-g u^2)
-// with g < 0 has no bound.
-bool tfm_f16_range(const mca_handle* h, int moves = 1) {
-  if (h->tspec.act == MCA_ACT_GAUSSIAN && h->tspec.act_param < 0.0f) return false;
-  return tfm_reach(h, moves) <= mca::kTfmF16Max;
+// The smallest power of two >= x > 0.
+float pow2_ceil(float x) {
+  int e = 0;
+  return std::frexp(x, &e) == 0.5f ? x : std::ldexp(1.0f, e);
+}
+
+// The level that the scales of the fp16 kernels' operands follow for the next trial: a power of two that no
+// parameter and no value the trial may draw exceeds, 0 beyond the kernels' range (tf32 kernels). It
+// follows from the trials before it alone (not from how they fell into batches), so that the
+// trajectory does not depend on the batch width. A Gaussian feed-forward activation exp(-g u^2) with g < 0
+// has no bound.
+float tfm_level(const mca_handle* h, int moves) {
+  if (!h->tc || h->tfm_small ||
+      (h->tspec.act == MCA_ACT_GAUSSIAN && h->tspec.act_param < 0.0f))
+    return 0.0f;
+  const float r = tfm_reach(h, moves);
+  return r <= mca::kTfmF16Max ? pow2_ceil(std::max(r, mca::kTfmF16Min)) : 0.0f;
+}
+
+// Bound of attention outputs and feed-forward activations of parameters up to q: 2 q sqrt(128) q sqrt(128) + q
+// (1 for a Gaussian).
+float tfm_act_bound(const mca_handle* h, float q) {
+  return std::max(256.0f * q * q + q, h->tspec.act == MCA_ACT_GAUSSIAN ? 1.0f : 0.0f);
+}
+
+// The kernels and scales for weight images of the handle's level and parameters up to qx (a candidate's
+// own, if it is beyond the level). A layer-norm output is at most qx (sqrt(127) + 1) < 12.3 qx. Scaled, the
+// bounds and the level are below fp16's 65504, and within a factor of four of it.
+void tfm_f16_args(const mca_handle* h, mca::TfmArgs* a, float qx = 0.0f) {
+  a->f16 = h->tfm_q > 0.0f && qx <= mca::kTfmF16Max ? 1 : 0;
+  const float q = h->tfm_q > 0.0f ? h->tfm_q : mca::kTfmF16Max;
+  qx = qx > q && a->f16 ? pow2_ceil(qx) : q;
+  int e = 0;
+  std::frexp(tfm_act_bound(h, qx), &e);
+  a->f16_w = 32768.0f / q;
+  a->f16_ln = 4096.0f / qx;
+  a->f16_act = std::ldexp(1.0f, 16 - e);
+  a->f16_dln = 1.0f / (a->f16_ln * a->f16_w);
+  a->f16_dact = 1.0f / (a->f16_act * a->f16_w);
 }
 
 mca::TfmArgs tfm_args(mca_handle* h) {
@@ -876,16 +905,32 @@ mca::TfmArgs tfm_args(mca_handle* h) {
   a.tc = h->tc ? 1 : 0;
   a.wimg = h->tfm_img;
   a.wimg16 = h->tfm_img16;
-  a.f16 = h->tc && tfm_f16_range(h) ? 1 : 0;
+  tfm_f16_args(h, &a);
   return a;
 }
 
-// An accepted parameter of magnitude w. Where it takes the trials to the tf32 kernels, the cached state is
-// recomputed by them: loss changes compare losses that the same kernels computed.
+// Whether the present parameters are too small for the fp16 kernels at their level (then it is 0).
+mca_status tfm_check_small(mca_handle* h) {
+  h->tfm_small = false;
+  const float q = tfm_level(h, 1);
+  if (q == 0.0f) return MCA_OK;
+  int small = 0;
+  CUDA_TRY(h, cudaMemsetAsync(h->flag, 0, sizeof(int), h->stream));
+  CUDA_TRY(h, mca::launch_tfm_f16_range(tfm_args(h), q, tfm_act_bound(h, q), h->flag, h->stream));
+  CUDA_TRY(h, cudaMemcpyAsync(&small, h->flag, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+  CUDA_TRY(h, cudaStreamSynchronize(h->stream));
+  h->launches += 1;
+  h->tfm_small = small != 0;
+  return MCA_OK;
+}
+
+// An accepted parameter of magnitude w. Where it takes the trials to another level, the weight images are
+// split and the cached state is recomputed: loss changes compare losses of the same arithmetic.
 mca_status tfm_grow(mca_handle* h, float w) {
-  const bool f16 = tfm_f16_range(h);
   h->pmax = std::max(h->pmax, w);
-  if (!h->tc || tfm_f16_range(h) == f16) return MCA_OK;
+  if (!h->tc || tfm_level(h, 1) == h->tfm_q) return MCA_OK;
+  const mca_status rc = tfm_check_small(h);
+  if (rc != MCA_OK) return rc;
   h->resyncs += 1;
   return resync(h);
 }
@@ -917,7 +962,7 @@ mca_status run_tfm_pipelined(mca_handle* h, mca::TfmArgs ta, uint64_t n_trials) 
                                   : mca::batch_width_waves(h->rate_acc, h->rate_trials, h->wave,
                                                            mca::kWaveTailTfm, h->opt.K);
     ta.Kb = (int)std::min<uint64_t>(n_trials, (uint64_t)Kw);
-    ta.f16 = tfm_f16_range(h) ? 1 : 0;
+    tfm_f16_args(h, &ta);
     ta.ctl = h->ctl2 + p;
     CUDA_TRY(h, cudaEventRecord(h->ev_p[p][0], h->stream));
     CUDA_TRY(h, mca::launch_tfm_eval(ta, h->stream));
@@ -939,8 +984,8 @@ mca_status run_tfm_pipelined(mca_handle* h, mca::TfmArgs ta, uint64_t n_trials) 
   if (rc != MCA_OK) return rc;
   for (int i = 0;; ++i) {
     NvtxRange nv_batch("mca batch (transformer, one ahead)");
-    // not ahead where the decision in flight may take the next batch to other kernels
-    const bool ahead = tfm_f16_range(h, 1) == tfm_f16_range(h, 2);
+    // not ahead where the decision in flight may take the next batch to another level
+    const bool ahead = tfm_level(h, 1) == tfm_level(h, 2);
     if (ahead) {
       rc = launch(i + 1);
       if (rc != MCA_OK) return rc;
@@ -1159,6 +1204,7 @@ mca_status mca_create(const mca_layer* layers, int32_t n_layers, int32_t loss,
   h->ex_new = reinterpret_cast<float*>(base + L.ex_new);
   h->gimg = L.gimg != SIZE_MAX ? reinterpret_cast<float*>(base + L.gimg) : nullptr;
   int* scratch = reinterpret_cast<int*>(base + L.scratch);
+  h->flag = scratch;
   CTRY(cudaMemsetAsync(h->st, 0, sizeof(DevState), h->stream));
   CTRY(cudaMemsetAsync(h->bar, 0, sizeof(GridBarrier), h->stream));
   CTRY(cudaMemsetAsync(h->partial, 0, L.st - L.partial, h->stream));
@@ -1363,7 +1409,7 @@ mca_status mca_run(mca_handle* h, uint64_t n_trials, uint64_t seed, mca_run_stat
       if (h->tfm && ctl.kstar >= 0) {
         const mca_status rc = tfm_grow(h, std::fabs(ctl.acc.neww));
         if (rc != MCA_OK) return rc;
-        ta.f16 = h->tc && tfm_f16_range(h) ? 1 : 0;
+        tfm_f16_args(h, &ta);
       }
       h->tau += (uint64_t)ctl.consumed;
       remaining -= (uint64_t)ctl.consumed;
@@ -1540,7 +1586,7 @@ mca_status eval_explicit(mca_handle* h, size_t n, float wmax) {
   auto* ev = h->ev_host;
   if (h->tfm) {
     mca::TfmArgs a = tfm_args(h);
-    if (wmax > mca::kTfmF16Max) a.f16 = 0;
+    tfm_f16_args(h, &a, wmax);
     a.n_explicit = (int)n;
     a.ex_idx = h->ex_idx;
     a.ex_new = h->ex_new;
@@ -1638,7 +1684,7 @@ mca_status mca_eval_trials(mca_handle* h, uint64_t seed, uint64_t tau, size_t n,
   a.ex_new = h->ex_new;
   CUDA_TRY(h, mca::launch_propose(a, h->stream));
   h->launches++;
-  const mca_status rc = eval_explicit(h, n, 0.0f);    // proposals are within tfm_f16_range's bound
+  const mca_status rc = eval_explicit(h, n, 0.0f);    // proposals are within the level
   if (rc != MCA_OK) return rc;
   const double S = h->ev_host->tail.S;
   for (size_t k = 0; k < n; ++k) {
@@ -1768,6 +1814,7 @@ mca_status mca_create_transformer(const mca_tfm_spec* spec, const mca_domain* do
   h->tfm_Xmid = h->tc ? reinterpret_cast<float*>(base + M.Xmid) : nullptr;
   h->ctl2 = reinterpret_cast<mca::DeepCtl*>(base + M.ctl2);
   h->tau_dev = reinterpret_cast<unsigned long long*>(base + M.tau_dev);
+  h->flag = reinterpret_cast<int*>(base + M.scratch);
   h->nscr = M.nscr;
   h->tfm_scrX = reinterpret_cast<float*>(base + M.scrX);
   h->tfm_scr_ell = reinterpret_cast<float*>(base + M.scr_ell);

@@ -187,6 +187,7 @@ constexpr int kWideGap = 17;
 constexpr unsigned int wide_allowance(unsigned int n) { return 3u + n / 2048u; }
 constexpr int kDeepScrSlots = 16;  // candidates whose fields the tensor-core evaluation keeps
 constexpr float kTfmF16Max = 4.0f;   // largest parameter magnitude of the fp16 Transformer kernels
+constexpr float kTfmF16Min = 0x1p-10f;   // ... and the smallest that their scales follow
 constexpr int kTfmScrSlots = 16;   // candidates whose residual streams the evaluation keeps
 constexpr size_t kSimtScrBytes = (size_t)1 << 30;   // all slots of a SIMT evaluation
 
@@ -326,7 +327,9 @@ struct TfmArgs {
   float* wimg;               // their split-weight images (mca_tc_layout.h), tc = 1 only
   void* wimg16;              // the images with fp16 parts, kept beside them
   int f16;                   // tc = 1: run the kernels with fp16 parts (every parameter, and every
-                             //   candidate's, at most kTfmF16Max in magnitude)
+                             //   candidate's, at most kTfmF16Max in magnitude), with
+  float f16_w, f16_ln, f16_act;   //   these scales (powers of two) of the weights in wimg16, of layer-norm
+  float f16_dln, f16_dact;        //   outputs and of other activations; the products' scales back
   // scratch slots (trial loop only): candidate k < nscr of a batch writes the residual streams it
   // recomputes to slot k of scrX ([nscr][(2 nL + 1) x B x T x d]: X, then Xmid; SIMT: X alone) and its
   // sequence losses to scr_ell ([nscr][B]); an accepted candidate with a slot is adopted from it
@@ -350,6 +353,8 @@ cudaError_t launch_tfm_forward(const TfmArgs& a, cudaStream_t s);   // grid B, w
 // parameters, the three sequence modes, and the image entry of the accepted parameter after a commit.
 cudaError_t launch_tfm_tc_split(const TfmArgs& a, cudaStream_t s);
 cudaError_t launch_tfm_f16_split(const TfmArgs& a, cudaStream_t s);
+// *out = 1 if parameters are too small for the fp16 parts at level q (bound: of the activations there).
+cudaError_t launch_tfm_f16_range(const TfmArgs& a, float q, float bound, int* out, cudaStream_t s);
 cudaError_t launch_tfm_f16(const TfmArgs& a, int mode, cudaStream_t s);   // the three modes, fp16 parts
 cudaError_t launch_tfm_tc_eval(const TfmArgs& a, cudaStream_t s);      // grid (Kb, B / 2)
 cudaError_t launch_tfm_tc_commit(const TfmArgs& a, cudaStream_t s);    // grid B / 2
@@ -486,6 +491,7 @@ struct mca_handle {
     mca_trace_rec prop[mca::kKmax];
     mca::ExTail tail;
   }* ev_host = nullptr;
+  int* flag = nullptr;                   // a device word for checks that the host waits for
   float* gimg = nullptr;                 // operand images of the tensor-core forward pass
   int nscr = 0;                          // host-driven batches: candidate scratch slots
   std::vector<float*> scr;               // [nscr x (L + 1)] layer m of slot k (m = L: losses)
@@ -521,6 +527,8 @@ struct mca_handle {
   float* tfm_img = nullptr;              // split-weight images of the tensor-core kernels (tc)
   void* tfm_img16 = nullptr;             // the same with fp16 operand parts
   float pmax = 0.0f;                     // tensor-core Transformer: largest parameter magnitude
+  float tfm_q = 0.0f;                    //   level of the fp16 operands' scales, 0: tf32 kernels
+  bool tfm_small = false;                //   parameters too small for them: tf32 kernels
   float* tfm_Xmid = nullptr;             // its mid streams (after each block's attention)
   float* tfm_scrX = nullptr;             // Transformer: candidate scratch slots
   float* tfm_scr_ell = nullptr;          // (h->nscr of them)

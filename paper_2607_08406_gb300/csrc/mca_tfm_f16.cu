@@ -1,10 +1,14 @@
 // Character-level Transformer on the tensor cores with fp16 operand parts: the recomputation of
 // mca_tfm_tc.cu (the same rows, restarts, rank-1 terms and cached streams), with every dense
-// projection as three kind::f16 MMAs per product, D = A_lo W_hi^T + A_hi W_lo^T + A_hi W_hi^T. A part has the
-// 11-bit significand of a tf32 part, and an fp16 MMA covers K = 16 in the time a tf32 MMA takes for
-// K = 8, so the projections cost half. fp16 has less range: the operands are scaled by powers of two from
-// bounds that follow from the largest parameter magnitude, and the host takes these kernels only while
-// it is at most kTfmF16Max; mca_tfm_tc.cu has no such bound.
+// projection as three kind::f16 MMAs per product, D = A_lo W_hi^T + A_hi W_lo^T + A_hi W_hi^T. An fp16 MMA
+// covers K = 16 in the time a tf32 MMA takes for K = 8, so the projections cost half. The two parts of a
+// value hold its 22 leading bits, like two tf32 parts, but fp16 has less range: the operands are
+// scaled by powers of two from bounds that follow from the largest parameter magnitude q (a power of two
+// at or above it), and below some size the error is absolute. With q = 1: weights down to 2^-18, 2^-40
+// below; layer-norm outputs down to 2^-15, 2^-37 below; attention outputs and feed-forward activations
+// (of up to 257) down to 2^-10, 2^-32 below; for q in general q, q and about q^2 times that. All of them enter the
+// residual stream through a weight and a sum in fp32. The host takes these kernels only while q is at most
+// kTfmF16Max; mca_tfm_tc.cu has no such bound.
 //
 // What bounded the tf32 kernel was not the tensor pipe but one thread deciding each MMA's operands at
 // run time (155 cycles per MMA whose arithmetic takes 64), and every phase waiting for the previous
@@ -312,7 +316,7 @@ __device__ __forceinline__ void ln_to_a(const TfmArgs& a, const Ctx& c, unsigned
     for (int i = 0; i < 32; ++i)
       if (32 * c.g + i == stash) s_acol[c.r] = x[i];
   }
-  store_parts<32>(c, x, kTfmF16Ln, kColA + 16u * (uint32_t)c.g, kAlo);
+  store_parts<32>(c, x, a.f16_ln, kColA + 16u * (uint32_t)c.g, kAlo);
 }
 
 template <int MODE>
@@ -468,8 +472,7 @@ __global__ void __launch_bounds__(kThreads, 1) tfm_f16_kernel(const __grid_const
     if (elect_one()) control(a, c, B, fail);
     __syncwarp();
   } else {
-    constexpr float dln = 1.0f / (kTfmF16Ln * kTfmF16W);      // scales of the products
-    constexpr float dact = 1.0f / (kTfmF16Act * kTfmF16W);
+    const float dln = a.f16_dln, dact = a.f16_dact;           // scales of the products
     uint32_t pm = 0u;            // phases of mdone
     int gh = 0;                  // halves of all feed-forward networks so far
     const int nh = a.F / kHc;
@@ -547,7 +550,7 @@ __global__ void __launch_bounds__(kThreads, 1) tfm_f16_kernel(const __grid_const
             for (int i = 0; i < 32; ++i)
               if (32 * c.g + i == c.tg.col) s_acol[c.r] = o[i];
           }
-          store_parts<32>(c, o, kTfmF16Act, kColA + 16u * (uint32_t)c.g, kAlo);
+          store_parts<32>(c, o, a.f16_act, kColA + 16u * (uint32_t)c.g, kAlo);
         }
         publish(&B.aready);        // also: this warp is done with K and V
         rows_sync();
@@ -598,7 +601,7 @@ __global__ void __launch_bounds__(kThreads, 1) tfm_f16_kernel(const __grid_const
           wait_phase(&B.a2empty[h & 1], (ph - 1u) & 1u, fail);
           tc_fence_after();
         }
-        store_parts<16>(c, u, kTfmF16Act, kColA2 + u2 + 8u * (uint32_t)c.g, kA2lo);
+        store_parts<16>(c, u, a.f16_act, kColA2 + u2 + 8u * (uint32_t)c.g, kA2lo);
         publish(&B.a2full[h & 1]);
       }
       product_done();
@@ -696,6 +699,50 @@ __global__ void tfm_f16_split_kernel(TfmArgs a) {
   }
 }
 
+// Are some of the operands so far below their scales that fp16 parts hold fewer bits than tf32 parts? One
+// warp per row of a weight matrix (blockIdx.y as in tfm_f16_split_kernel): the absolute error of its parts is
+// 2^-40 q, below 2^-26 of the row's largest weight from 2^-14 q on. The last x block of Wv and of W1
+// compares the bound of the activations that it produces with the one that their scale follows from: typical
+// ones lie about 2^-9 below their bound and keep 22 bits down to 2^-17 below the scale's.
+__global__ void __launch_bounds__(256) tfm_f16_range_kernel(TfmArgs a, float q, float bound, int* out) {
+  const int slot = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int b = slot / 6, mat = slot == 6 * a.nL ? (int)kTcHead : slot % 6;
+  const unsigned long long base = a.o_blk0 + (unsigned long long)b * a.blk_size;
+  const unsigned int off[6] = {a.r_wq, a.r_wk, a.r_wv, a.r_wo, a.r_w1, a.r_w2};
+  const float* w = a.params + (mat == kTcHead ? a.o_wh : base + off[mat]);
+  const int rows = mat == kTcHead ? a.V : mat == kTcW1 ? a.F : kD;
+  const int cols = mat == kTcW2 ? a.F : kD;
+  if (blockIdx.x + 1 < gridDim.x) {
+    for (int r = blockIdx.x * 8 + warp; r < rows; r += 8 * (gridDim.x - 1)) {
+      float m = 0.0f;
+      for (int k = lane; k < cols; k += 32) m = fmaxf(m, fabsf(w[(size_t)r * cols + k]));
+      m = __int_as_float(__reduce_max_sync(0xffffffffu, __float_as_int(m)));
+      if (lane == 0 && m > 0.0f && m < q * 0x1p-14f) *out = 1;
+    }
+    return;
+  }
+  if (mat != kTcV && mat != kTcW1) return;
+  __shared__ int s_m[3];                // bits of the largest weight, layer-norm gain or bias, own bias
+  if (threadIdx.x < 3) s_m[threadIdx.x] = 0;
+  __syncthreads();
+  const float* ln = a.params + base + (mat == kTcV ? a.r_ln1g : a.r_ln2g);
+  const float* lb = a.params + base + (mat == kTcV ? a.r_ln1b : a.r_ln2b);
+  const float* bi = a.params + base + (mat == kTcV ? a.r_bv : a.r_b1);
+  int m[3] = {0, 0, 0};
+  for (int e = threadIdx.x; e < rows * cols; e += 256) m[0] = max(m[0], __float_as_int(fabsf(w[e])));
+  for (int e = threadIdx.x; e < kD; e += 256)
+    m[1] = max(m[1], __float_as_int(fmaxf(fabsf(ln[e]), fabsf(lb[e]))));
+  for (int e = threadIdx.x; e < rows; e += 256) m[2] = max(m[2], __float_as_int(fabsf(bi[e])));
+  for (int i = 0; i < 3; ++i) {
+    m[i] = __reduce_max_sync(0xffffffffu, m[i]);
+    if (lane == 0) atomicMax(&s_m[i], m[i]);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0 && 256.0f * __int_as_float(s_m[1]) * __int_as_float(s_m[0]) +
+                                  __int_as_float(s_m[2]) < bound * 0x1p-8f)
+    *out = 1;
+}
+
 template <int MODE>
 cudaError_t launch_f16(const TfmArgs& a, dim3 grid, cudaStream_t s) {
   cudaError_t e = cudaFuncSetAttribute((const void*)tfm_f16_kernel<MODE>,
@@ -709,6 +756,11 @@ cudaError_t launch_f16(const TfmArgs& a, dim3 grid, cudaStream_t s) {
 
 cudaError_t launch_tfm_f16_split(const TfmArgs& a, cudaStream_t s) {
   tfm_f16_split_kernel<<<dim3(32, 6 * a.nL + 1), 256, 0, s>>>(a);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_tfm_f16_range(const TfmArgs& a, float q, float bound, int* out, cudaStream_t s) {
+  tfm_f16_range_kernel<<<dim3(17, 6 * a.nL + 1), 256, 0, s>>>(a, q, bound, out);
   return cudaGetLastError();
 }
 

@@ -21,11 +21,6 @@ constexpr int kHc = kTcTfmHc;
 constexpr int kXLd = kD + 4;                     // residual row stride: conflict-free row access
 constexpr int kTfmWorkers = 512;                 // threads that own token rows
 
-// Scales of the fp16 operands. While every parameter is at most kTfmF16Max = 4 in magnitude, a layer-norm
-// output is at most 4 sqrt(127) + 4 < 50, and an attention output or a feed-forward unit's activation at
-// most (4 + 4) sqrt(128) 4 sqrt(128) + 4 = 4100: scaled, all stay below fp16's 65504.
-constexpr float kTfmF16Ln = 1024.0f, kTfmF16Act = 8.0f, kTfmF16W = 8192.0f;
-
 // Barrier of the threads that own token rows (the control warp of the fp16 kernel takes no part).
 __device__ __forceinline__ void rows_sync() {
   asm volatile("bar.sync 1, %0;" ::"r"(kTfmWorkers) : "memory");
@@ -282,7 +277,7 @@ __device__ __forceinline__ void tfm_f16_image_store(const TfmArgs& a, int mat, i
                                                     float w) {
   __half* img = reinterpret_cast<__half*>(a.wimg16);
   const size_t o = tfm_f16_image_offset(mat, b, r, k, a.F, a.nL);
-  const float x = w * kTfmF16W;
+  const float x = w * a.f16_w;
   const __half h = __float2half_rn(x);
   img[o] = h;
   img[o + kTfmF16Chunk / 4] = __float2half_rn(x - __half2float(h));

@@ -148,6 +148,24 @@ def test_tfm_growing_feed_forward_activation(gpu_lib):
     assert gpu_lib.mca_loss(h) * 2 * spec.ctx == pytest.approx(S0, rel=TIE_REL)
 
 
+@pytest.mark.gpu
+@pytest.mark.parametrize("v", [1e-2, 1e-3, 1e-4, 1e-5, 1e-6])
+def test_tfm_small_activations(gpu_lib, v):
+    """Attention outputs and feed-forward activations of size v that the residual stream consists of (tiny
+    embeddings, an epsilon below the stream's variance): in fp16 parts or, if those lose bits, in tf32 parts."""
+    spec = W.TfmSpec(n_layer=1, d_ff=128, ln_eps=1e-30)
+    wl = W.char_transformer(batch=2, text_len=4000, spec=spec, n_trials=8, K=8)
+    rng = np.random.default_rng(3)
+    amp = {"tok_emb": 1e-6 * v, "pos_emb": 1e-6 * v, "b0.wq": 0.05, "b0.wk": 0.05, "b0.wv": v / 4,
+           "b0.wo": 0.3, "b0.w1": v / 11, "b0.w2": 0.3, "w_head": 0.5}
+    wl.init = np.concatenate([
+        (np.ones(shape) if name.endswith(".g") else rng.normal(0.0, amp.get(name, 0.0) or 1e-30, shape)
+         ).ravel() for name, shape in spec.blocks()]).astype(np.float32)
+    S0 = T.tfm_seq_losses(spec, wl.init.astype(np.float64), wl.tokens).sum()
+    h = gpu_lib.create_from_tfm_workload(wl)
+    assert gpu_lib.mca_loss(h) * 2 * spec.ctx == pytest.approx(S0, rel=TIE_REL)
+
+
 PROBE = r"""
 #include <cstdio>
 #include <cstdlib>
