@@ -325,7 +325,7 @@ __global__ void __launch_bounds__(kOutWarps * 32, 2) mlp2_outputs_kernel(
       }
     }
     const int yn = y[n];
-    const float ln = sample_loss<-1, -1, kMaxC>(zz, C, yn, a.g2, a.act2, a.loss);
+    const float ln = sample_loss<-1, -1, kMaxC, true>(zz, C, yn, a.g2, a.act2, a.loss);
     store_srec(a.srec, a.Np, n, zz, ln, yn);
   }
 }

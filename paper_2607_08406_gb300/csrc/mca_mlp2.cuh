@@ -106,7 +106,7 @@ __device__ __forceinline__ float entry_l1(const Mlp2Args& a, Recs R, float delta
 #pragma unroll
   for (int k = 0; k < M; ++k)
     if (k < C) zz[k] = fmaf(w[k], da, zz[k]);
-  const float ln = sample_loss<ACT2, LOSS, M>(zz, C, y, a.g2, a.act2, a.loss);
+  const float ln = sample_loss<ACT2, LOSS, M, true>(zz, C, y, a.g2, a.act2, a.loss);
   if (COMMIT) store_srec(R.rec, R.pitch, nl, zz, ln, y);
   return ln - ell;
 }
@@ -131,7 +131,7 @@ __device__ __forceinline__ float entry_l2(const Mlp2Args& a, Recs R, float delta
 #pragma unroll
   for (int k = 0; k < M; ++k)
     if (k == o) zz[k] = zon;
-  const float ln = sample_loss<ACT2, LOSS, M>(zz, C, y, a.g2, a.act2, a.loss);
+  const float ln = sample_loss<ACT2, LOSS, M, true>(zz, C, y, a.g2, a.act2, a.loss);
   if (COMMIT) store_srec(R.rec, R.pitch, nl, zz, ln, y);
   return ln - ell;
 }
@@ -777,7 +777,7 @@ struct VRecs {
 };
 
 // Loss of the fields z with label y; zy: field y; onehot: -[k == y] per field (MSE). The same operations on
-// each field and the same order of sums as sample_loss: records come from it in the forward pass.
+// each field and the same order of sums as sample_loss with PAIRS, which the forward pass calls.
 template <int ACT2, int LOSS, int M>
 __device__ __forceinline__ float vloss(const Mlp2Args& a, const float2 (&z)[M / 2], int y, float zy,
                                        const float* onehot) {
@@ -811,7 +811,7 @@ __device__ __forceinline__ float vloss(const Mlp2Args& a, const float2 (&z)[M / 
       zz[2 * q] = z[q].x;
       zz[2 * q + 1] = z[q].y;
     }
-    return sample_loss<-1, -1, M>(zz, a.C, y, a.g2, a.act2, a.loss);
+    return sample_loss<-1, -1, M, true>(zz, a.C, y, a.g2, a.act2, a.loss);
   }
 }
 
@@ -852,7 +852,7 @@ __device__ __noinline__ float vdelta_any(const Mlp2Args& a, VRecs<M> R, const fl
     zz[f] = o >= 0 ? (f == o ? fmaf(delta, da, z) : z) : f < a.C ? fmaf(w2c[f], da, z) : z;
   }
   const float ell = R.at(nl, M);
-  const float ln = sample_loss<-1, -1, M>(zz, a.C, __float_as_int(R.at(nl, M + 1)), a.g2, a.act2,
+  const float ln = sample_loss<-1, -1, M, true>(zz, a.C, __float_as_int(R.at(nl, M + 1)), a.g2, a.act2,
                                           a.loss);
   if (COMMIT) {
 #pragma unroll
