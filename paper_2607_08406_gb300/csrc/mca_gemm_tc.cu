@@ -8,11 +8,9 @@
 //    A and every feature's row of W is scaled by a power of two that brings its largest magnitude to
 //    [2^14, 2^15), taken back when the fields are written; then |x - hi - lo| <= 2^-22 |x| for values down
 //    to 2^-17 of their row's largest, as with tf32, and 2^-39 of the largest below.
-//  - tf32 for products too small to pay for finding the scales (kF16Macs) and for rows of so wide a
-//    range that values below 2^-17 of the largest may matter: where the non-zero magnitudes of any row
-//    lie more than kMaxGap binary orders below its largest on average, or are not finite. Images
-//    of pixels and weights drawn uniformly lie 1 to 3 orders below. The scale kernels set a flag that the
-//    later kernels read.
+//  - tf32 for products too small to pay for finding the scales (kF16Macs), and where any row has
+//    non-finite values, or more than wide_allowance of its non-zero values below 2^-17 of its largest: a field may
+//    read only those. The scale kernels set a flag that the later kernels read.
 //
 // The operands are first written as split images in core-matrix order (mca_tc_layout.h; two fp16
 // in the place of one tf32): A by blocks of 128 samples, W by blocks of 256 rows, both cut into K
@@ -62,7 +60,6 @@ constexpr uint32_t kGIdesc16 = tc_idesc_f16(kGM, kGN), kGIdesc32 = tc_idesc_tf32
 // samples, H = 1024 (3.2e9) 91 us with tf32 parts, 90 us with fp16; 10000 samples (8e9) 160 and 147 us;
 // 30000 samples, H = 2048 (4.8e10) 478 and 375 us; 4000 samples, H = 256 (8e8) 80 and 86 us.
 constexpr double kF16Macs = 4294967296.0;
-constexpr unsigned int kMaxGap = 8;
 
 __device__ __forceinline__ void expect_tx(uint64_t* bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
@@ -85,23 +82,17 @@ __device__ __forceinline__ int row_exponent(unsigned int bits) {
 }
 __device__ __forceinline__ float pow2(int e) { return __int_as_float((127 + e) << 23); }
 
-// Magnitudes of a row: the largest (as bits), the sum of the non-zero ones' exponents, their number.
+// Of a row's values: how many are non-zero, and how many of these lie more than kWideGap binary orders
+// below the largest (whose bits are top).
 struct RowRange {
-  unsigned int top, sum, n;             // (K < 2^24: the sum stays below 2^32)
-  __device__ __forceinline__ void add(float v) {
+  unsigned int n, low;
+  __device__ __forceinline__ void add(float v, unsigned int top) {
     const unsigned int m = __float_as_uint(fabsf(v));
-    top = max(top, m);
-    sum += m >> 23;
     n += m != 0u;
+    low += m != 0u && (m >> 23) + (unsigned int)kWideGap < (top >> 23);
   }
-  __device__ __forceinline__ void add(const RowRange& o) {
-    top = max(top, o.top);
-    sum += o.sum;
-    n += o.n;
-  }
-  __device__ __forceinline__ bool wide() const {
-    const unsigned int E = top >> 23;
-    return E == 255u || E * n - sum > kMaxGap * n;
+  __device__ __forceinline__ bool wide(unsigned int top) const {
+    return top >> 23 == 255u || low > wide_allowance(n);
   }
 };
 
@@ -148,37 +139,54 @@ __device__ __forceinline__ float act_value(const float* __restrict__ B, int k, i
   return act >= 0 ? act_rt(act, v, g) : v;
 }
 
-// Scale exponents of the samples: 32 samples per CTA, 8 slices of k.
+// Scale exponents of the samples: 32 samples per CTA, 8 slices of k. (The second pass over a CTA's rows finds
+// them in L2.)
 __global__ void act_scale_kernel(const float* __restrict__ B, int K, int Np, int act, float g,
                                  int* __restrict__ ex, int* wide) {
-  __shared__ RowRange s_m[8][32];
+  __shared__ unsigned int s_top[8][32];
+  __shared__ RowRange s_r[8][32];
   const int lane = threadIdx.x & 31, p = threadIdx.x >> 5, n = blockIdx.x * 32 + lane;
-  RowRange m{0u, 0u, 0u};
+  unsigned int top = 0u;
 #pragma unroll 4
-  for (int k = p; k < K; k += 8) m.add(act_value(B, k, n, Np, act, g));
-  s_m[p][lane] = m;
+  for (int k = p; k < K; k += 8)
+    top = max(top, __float_as_uint(fabsf(act_value(B, k, n, Np, act, g))));
+  s_top[p][lane] = top;
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < 8; ++q) top = max(top, s_top[q][lane]);
+  RowRange r{0u, 0u};
+#pragma unroll 4
+  for (int k = p; k < K; k += 8) r.add(act_value(B, k, n, Np, act, g), top);
+  s_r[p][lane] = r;
   __syncthreads();
   if (p != 0) return;
 #pragma unroll
-  for (int q = 1; q < 8; ++q) m.add(s_m[q][lane]);
-  ex[n] = row_exponent(m.top);
-  if (m.wide()) *wide = 1;
+  for (int q = 1; q < 8; ++q) {
+    r.n += s_r[q][lane].n;
+    r.low += s_r[q][lane].low;
+  }
+  ex[n] = row_exponent(top);
+  if (r.wide(top)) *wide = 1;
 }
 
 // Scale exponents of W's rows: one warp per row.
 __global__ void w_scale_kernel(const float* __restrict__ W, int M, int K, int* __restrict__ ex,
                                int* wide) {
-  const int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (r >= M) return;
-  RowRange m{0u, 0u, 0u};
+  const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (row >= M) return;
+  unsigned int top = 0u;
 #pragma unroll 4
-  for (int k = lane; k < K; k += 32) m.add(W[(size_t)r * K + k]);
-  m.top = __reduce_max_sync(0xffffffffu, m.top);
-  m.sum = __reduce_add_sync(0xffffffffu, m.sum);
-  m.n = __reduce_add_sync(0xffffffffu, m.n);
+  for (int k = lane; k < K; k += 32)
+    top = max(top, __float_as_uint(fabsf(W[(size_t)row * K + k])));
+  top = __reduce_max_sync(0xffffffffu, top);
+  RowRange r{0u, 0u};
+#pragma unroll 4
+  for (int k = lane; k < K; k += 32) r.add(W[(size_t)row * K + k], top);
+  r.n = __reduce_add_sync(0xffffffffu, r.n);
+  r.low = __reduce_add_sync(0xffffffffu, r.low);
   if (lane == 0) {
-    ex[r] = row_exponent(m.top);
-    if (m.wide()) *wide = 1;
+    ex[row] = row_exponent(top);
+    if (r.wide(top)) *wide = 1;
   }
 }
 

@@ -39,3 +39,24 @@ def test_forward_fields(gpu_lib, N, H, D, spread):
     h = gpu_lib.create_from_workload(wl)
     S = O.total_loss(O.Params(layers, init), X.T.astype(np.float64), wl.y, wl.loss)
     assert gpu_lib.mca_loss(h) == pytest.approx(S / N, rel=TIE_REL)
+
+
+@pytest.mark.parametrize("n_small,down", [(150, 34), (24, 40), (4, 40)])
+def test_forward_fields_of_a_few_small_features(gpu_lib, n_small, down):
+    """Features far below the others, and hidden units that read only those: a minority of small entries
+    in the samples' rows must not lose their bits. Few distinct samples, so that the errors of
+    the fields do not average out in the loss."""
+    N, H, D = 22000, 256, 784
+    rng = np.random.default_rng(n_small)
+    layers = [W.Layer(D, H, "tanh"), W.Layer(H, 10, "identity")]
+    base = rng.uniform(0.5, 1.0, (4, D)).astype(np.float32)
+    base[:, :n_small] *= np.float32(2.0 ** -down)
+    X = np.ascontiguousarray(base[np.arange(N) % 4])
+    W1 = np.zeros((H, D), np.float32)
+    W1[:, :n_small] = rng.uniform(-1, 1, (H, n_small)) * 2.0 ** down / np.sqrt(n_small)
+    init = np.concatenate([W1.ravel(), rng.uniform(-0.5, 0.5, H * 10)]).astype(np.float32)
+    wl = W.MLPWorkload("fields", layers, "softmax_ce", X, (np.arange(N) % 7).astype(np.int32), init, 8,
+                       8)
+    h = gpu_lib.create_from_workload(wl)
+    S = O.total_loss(O.Params(layers, init), X.T.astype(np.float64), wl.y, wl.loss)
+    assert gpu_lib.mca_loss(h) == pytest.approx(S / N, rel=TIE_REL)
