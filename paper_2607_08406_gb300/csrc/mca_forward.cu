@@ -291,10 +291,10 @@ __global__ void __launch_bounds__(kOutWarps * 32, 2) mlp2_outputs_kernel(
     for (int h = 0; h < kOutRows; h += 16) {
       float v[16];
 #pragma unroll
-      for (int q = 0; q < 16; ++q)                   // rows past the last carry weight 0
-        v[q] = z[(size_t)min(j0 + h + q, a.H - 1) * a.Np];
+      for (int q = 0; q < 16; ++q) v[q] = z[(size_t)min(j0 + h + q, a.H - 1) * a.Np];
 #pragma unroll
-      for (int q = 0; q < 16; ++q) v[q] = act<ACT1>(v[q], a.g1, a.act1);
+      for (int q = 0; q < 16; ++q)                   // (rows past the last: 0 times infinity is not 0)
+        v[q] = j0 + h + q < a.H ? act<ACT1>(v[q], a.g1, a.act1) : 0.0f;
 #pragma unroll
       for (int k = 0; k < M; ++k) {
         if (k < C) {

@@ -60,3 +60,22 @@ def test_forward_fields_of_a_few_small_features(gpu_lib, n_small, down):
     h = gpu_lib.create_from_workload(wl)
     S = O.total_loss(O.Params(layers, init), X.T.astype(np.float64), wl.y, wl.loss)
     assert gpu_lib.mca_loss(h) == pytest.approx(S / N, rel=TIE_REL)
+
+
+def test_forward_last_hidden_field_overflows(gpu_lib):
+    """An infinite activation of the last hidden neuron (33 neurons: the rows past it are padding)
+    saturates a sigmoid output and nothing else."""
+    N, D, H = 70, 5, 33
+    rng = np.random.default_rng(0)
+    layers = [W.Layer(D, H, "relu"), W.Layer(H, 4, "sigmoid")]
+    X = W.synth_images(rng, N, D, 0.6)
+    X[:, :2] = 0.0
+    X[::9, :2] = 1.0
+    init = W.uniform_init(rng, layers, 0.3)
+    init[(H - 1) * D:(H - 1) * D + 2] = np.float32(3e38)
+    wl = W.MLPWorkload("overflow", layers, "mse_onehot", X, rng.integers(0, 4, N).astype(np.int32),
+                       init, 8, 8)
+    with np.errstate(over="ignore"):
+        S = O.total_loss(O.Params(layers, init), X.T.astype(np.float64), wl.y, wl.loss)
+    h = gpu_lib.create_from_workload(wl)
+    assert gpu_lib.mca_loss(h) == pytest.approx(S / N, rel=TIE_REL)
