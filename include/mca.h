@@ -129,7 +129,11 @@ typedef struct {
                               only to rounding */
   void* workspace;         /* NULL: the library allocates its device memory itself; otherwise a
                               caller-owned device buffer of >= mca_workspace_size() bytes,
-                              256-byte aligned, that must outlive the handle */
+                              256-byte aligned, that must outlive the handle. Scratch slots for
+                              accepted candidates are left out where device memory is short, and
+                              on the SIMT kernels where the buffer is too small for them (down to
+                              its size without slots, that under MCA_ADOPT=0): a little slower,
+                              the same results */
   size_t workspace_bytes;
   int32_t fixed_K;         /* 0: the batch width follows p, the recently observed acceptance rate
                               per trial, at most K (fewer discarded candidates while many are

@@ -768,7 +768,7 @@ int tfm_scratch_slots(const mca_tfm_spec& t, long long B, int K, bool tc) {
   return (int)std::min<size_t>((size_t)std::min(K, mca::kTfmScrSlots), cap / slot);
 }
 
-TfmMem tfm_plan(const mca_tfm_spec& t, long long B, int trace_cap, bool tc, int K) {
+TfmMem tfm_plan(const mca_tfm_spec& t, long long B, int trace_cap, bool tc, int nscr) {
   TfmMem M;
   size_t o = 0;
   auto take = [&](size_t bytes) {
@@ -791,7 +791,7 @@ TfmMem tfm_plan(const mca_tfm_spec& t, long long B, int trace_cap, bool tc, int 
   M.wimg = tc ? take(sizeof(float) * mca::tfm_tc_image_floats(t.d_ff, t.n_layer)) : 0;
   M.wimg16 = tc ? take(mca::tfm_f16_image_bytes(t.d_ff, t.n_layer)) : 0;
   M.Xmid = take(tc ? sizeof(float) * (size_t)t.n_layer * B * t.ctx * t.d_model : 0);
-  M.nscr = tfm_scratch_slots(t, B, K, tc);
+  M.nscr = nscr;
   M.scrX = take(sizeof(float) * (size_t)M.nscr * tfm_streams(t, tc) * B * t.ctx * t.d_model);
   M.scr_ell = take(sizeof(float) * (size_t)M.nscr * B);
   M.ctl2 = take(2 * sizeof(mca::DeepCtl));
@@ -1149,8 +1149,11 @@ mca_status mca_create(const mca_layer* layers, int32_t n_layers, int32_t loss,
     h->window = R.window;
   }
   h->nscr = deep_scratch_slots(ls, h->N, o.K);
-  const Layout L = plan(ls, h->N, h->D, h->nnz, o.trace_cap, h->NR, h->nscr);
+  Layout L = plan(ls, h->N, h->D, h->nnz, o.trace_cap, h->NR, h->nscr);
   if (o.workspace) {
+    // the SIMT kernels take fewer slots where the workspace was sized without (all of) them
+    while (!h->tc && h->nscr > 0 && o.workspace_bytes < L.total)
+      L = plan(ls, h->N, h->D, h->nnz, o.trace_cap, h->NR, --h->nscr);
     if (o.workspace_bytes < L.total)
       return bail(fail(h, MCA_ERR_OOM, "workspace of %zu bytes < %zu needed", o.workspace_bytes,
                        L.total));
@@ -1159,7 +1162,14 @@ mca_status mca_create(const mca_layer* layers, int32_t n_layers, int32_t loss,
     h->ws = o.workspace;
     h->ws_bytes = o.workspace_bytes;
   } else {
-    CTRY(cudaMalloc(&h->ws, L.total));
+    cudaError_t e = cudaMalloc(&h->ws, L.total);
+    if (e == cudaErrorMemoryAllocation && h->nscr > 0) {   // without slots, then
+      cudaGetLastError();
+      h->nscr = 0;
+      L = plan(ls, h->N, h->D, h->nnz, o.trace_cap, h->NR, 0);
+      e = cudaMalloc(&h->ws, L.total);
+    }
+    CTRY(e);
     h->ws_owned = true;
     h->ws_bytes = L.total;
   }
@@ -1723,7 +1733,8 @@ mca_status mca_tfm_workspace_size(const mca_tfm_spec* spec, int64_t n_seq, const
   if (rc != MCA_OK) return rc;
   if (!bytes) return fail(nullptr, MCA_ERR_INVALID, "bytes is NULL");
   const mca_options o = opt ? *opt : default_options();
-  *bytes = tfm_plan(*spec, n_seq, o.trace_cap, tfm_use_tc(*spec, n_seq), o.K).total;
+  const bool tc = tfm_use_tc(*spec, n_seq);
+  *bytes = tfm_plan(*spec, n_seq, o.trace_cap, tc, tfm_scratch_slots(*spec, n_seq, o.K, tc)).total;
   return MCA_OK;
 }
 
@@ -1780,8 +1791,15 @@ mca_status mca_create_transformer(const mca_tfm_spec* spec, const mca_domain* do
     e = cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, h->device);
   if (e != cudaSuccess) return bail(fail(h, MCA_ERR_CUDA, "%s", cudaGetErrorString(e)));
   h->tc = tfm_use_tc(*spec, n_seq);
-  const TfmMem M = tfm_plan(*spec, n_seq, o.trace_cap, h->tc, o.K);
+  TfmMem M = tfm_plan(*spec, n_seq, o.trace_cap, h->tc,
+                      tfm_scratch_slots(*spec, n_seq, o.K, h->tc));
   if (o.workspace) {
+    // fewer slots where the workspace was sized without (all of) them: SIMT kernels, or without the fp16
+    // images: tensor-core kernels
+    const size_t least =
+        h->tc ? M.total - mca::tfm_f16_image_bytes(spec->d_ff, spec->n_layer) : 0;
+    while (M.nscr > 0 && o.workspace_bytes >= least && o.workspace_bytes < M.total)
+      M = tfm_plan(*spec, n_seq, o.trace_cap, h->tc, M.nscr - 1);
     if (o.workspace_bytes < M.total)
       return bail(fail(h, MCA_ERR_OOM, "workspace of %zu bytes < %zu needed", o.workspace_bytes,
                        M.total));
@@ -1791,6 +1809,11 @@ mca_status mca_create_transformer(const mca_tfm_spec* spec, const mca_domain* do
     h->ws_bytes = o.workspace_bytes;
   } else {
     e = cudaMalloc(&h->ws, M.total);
+    if (e == cudaErrorMemoryAllocation && M.nscr > 0) {    // without slots, then
+      cudaGetLastError();
+      M = tfm_plan(*spec, n_seq, o.trace_cap, h->tc, 0);
+      e = cudaMalloc(&h->ws, M.total);
+    }
     if (e != cudaSuccess) return bail(fail(h, MCA_ERR_OOM, "%s", cudaGetErrorString(e)));
     h->ws_owned = true;
     h->ws_bytes = M.total;

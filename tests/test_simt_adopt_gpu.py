@@ -56,3 +56,40 @@ def test_simt_adoption_matches_commit(gpu_lib, monkeypatch, case, fixed_K):
     assert np.array_equal(out[0][0], out[1][0])
     assert np.array_equal(out[0][1], out[1][1])
     assert out[0][2] == out[1][2]
+
+
+@pytest.mark.parametrize("case", ["narrow", "tfm"])
+def test_workspace_without_room_for_slots(gpu_lib, monkeypatch, case):
+    """The slots of the SIMT paths are taken as far as the caller's workspace reaches: a workspace of the size
+    without slots, or with room for some, gives the same run; a smaller one is refused."""
+    import torch
+    wl = CASES[case]()
+    tfm = case == "tfm"
+    create = gpu_lib.create_from_tfm_workload if tfm else gpu_lib.create_from_workload
+
+    def size():
+        if tfm:
+            return gpu_lib.mca_tfm_workspace_size(wl.spec, len(wl.tokens), 32, 200)
+        return gpu_lib.mca_workspace_size(wl.layers, wl.loss, wl.X, wl.y, 32, 200)
+
+    full = size()
+    monkeypatch.setenv("MCA_ADOPT", "0")
+    least = size()
+    monkeypatch.delenv("MCA_ADOPT")
+    assert least < full
+    name = "mca_tfm_workspace_size" if tfm else "mca_workspace_size"
+    out = []
+    for nbytes in (full, least + (full - least) // 3, least, least - 256):
+        with monkeypatch.context() as m:
+            m.setattr(gpu_lib, name, lambda *a, **k: nbytes)
+            if nbytes < least:
+                with pytest.raises(gpu_lib.MCAError, match="workspace"):
+                    create(wl, trace_cap=200, K=32)
+                continue
+            h = create(wl, trace_cap=200, K=32, fixed_K=True)
+        gpu_lib.mca_run(h, 200, 4)
+        out.append((gpu_lib.mca_get_trace(h, 200), gpu_lib.mca_get_params(h, wl.n_params)))
+        h.close()
+    assert len(out) == 3
+    for o in out[1:]:
+        assert np.array_equal(o[0], out[0][0]) and np.array_equal(o[1], out[0][1])
