@@ -4,6 +4,7 @@
 #include <chrono>
 #include <cmath>
 #include <cstdarg>
+#include <cstddef>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -77,7 +78,7 @@ bool is_device_ptr(const void* p) {
 
 struct Layout {
   size_t XT, y, xs_off, xs_n, xs_v, xs_sect, xs_roff, z1, srec, partial, accum, bar, st, trace,
-      ex_idx, ex_new, scratch, ell, ctl, gimg, scr_tab, total;
+      ex, scratch, ell, ctl, gimg, scr_tab, total;
   std::vector<size_t> w_eff, code, wfix, Z, whi, scr;
 };
 
@@ -191,8 +192,7 @@ Layout plan(const std::vector<mca_layer>& layers, long long N, int D, long long 
   L.bar = take(sizeof(GridBarrier));
   L.st = take(sizeof(DevState));
   L.trace = take(sizeof(mca_trace_rec) * (size_t)std::max(trace_cap, 0));
-  L.ex_idx = take(sizeof(unsigned int) * mca::kKmax);
-  L.ex_new = take(sizeof(float) * mca::kKmax);
+  L.ex = take(sizeof(mca::ExCands));
   L.scratch = take(sizeof(int) * (size_t)(D + 8));
   const size_t gb = forward_tc_image_bytes(layers, Np);
   L.gimg = gb ? take(gb) : SIZE_MAX;
@@ -742,7 +742,7 @@ mca_status tfm_check(const mca_tfm_spec* t, int64_t n_seq) {
 }
 
 struct TfmMem {
-  size_t params, tokens, X, ell, partial, st, ctl, trace, ex_idx, ex_new, scratch,
+  size_t params, tokens, X, ell, partial, st, ctl, trace, ex, scratch,
       wimg, wimg16, Xmid, scrX, scr_ell, ctl2, tau_dev, total;
   int nscr;
 };
@@ -785,8 +785,7 @@ TfmMem tfm_plan(const mca_tfm_spec& t, long long B, int trace_cap, bool tc, int 
   M.st = take(sizeof(DevState));
   M.ctl = take(sizeof(mca::DeepCtl));
   M.trace = take(sizeof(mca_trace_rec) * (size_t)std::max(trace_cap, 0));
-  M.ex_idx = take(sizeof(unsigned int) * mca::kKmax);
-  M.ex_new = take(sizeof(float) * mca::kKmax);
+  M.ex = take(sizeof(mca::ExCands));
   M.scratch = take(sizeof(int) * 8);
   M.wimg = tc ? take(sizeof(float) * mca::tfm_tc_image_floats(t.d_ff, t.n_layer)) : 0;
   M.wimg16 = tc ? take(mca::tfm_f16_image_bytes(t.d_ff, t.n_layer)) : 0;
@@ -1210,8 +1209,7 @@ mca_status mca_create(const mca_layer* layers, int32_t n_layers, int32_t loss,
   h->bar = reinterpret_cast<GridBarrier*>(base + L.bar);
   h->st = reinterpret_cast<DevState*>(base + L.st);
   h->trace = o.trace_cap > 0 ? reinterpret_cast<mca_trace_rec*>(base + L.trace) : nullptr;
-  h->ex_idx = reinterpret_cast<unsigned int*>(base + L.ex_idx);
-  h->ex_new = reinterpret_cast<float*>(base + L.ex_new);
+  h->ex = reinterpret_cast<mca::ExCands*>(base + L.ex);
   h->gimg = L.gimg != SIZE_MAX ? reinterpret_cast<float*>(base + L.gimg) : nullptr;
   int* scratch = reinterpret_cast<int*>(base + L.scratch);
   h->flag = scratch;
@@ -1588,7 +1586,7 @@ mca_status mca_force_decisions(mca_handle* h, const uint64_t* tau, const uint8_t
 
 namespace {
 
-// Loss changes of the n candidates in h->ex_idx / h->ex_new against the current state, no commit,
+// Loss changes of the n candidates in h->ex against the current state, no commit,
 // into h->ev_host; wmax: the candidates' largest magnitude. The evaluation kernels of mca_run's
 // evaluation step. The kernels write the results to pinned memory, so one synchronisation ends the
 // call.
@@ -1598,8 +1596,8 @@ mca_status eval_explicit(mca_handle* h, size_t n, float wmax) {
     mca::TfmArgs a = tfm_args(h);
     tfm_f16_args(h, &a, wmax);
     a.n_explicit = (int)n;
-    a.ex_idx = h->ex_idx;
-    a.ex_new = h->ex_new;
+    a.ex_idx = h->ex->idx;
+    a.ex_new = h->ex->new_w;
     a.ex_out = ev->dS;
     a.ex_tail = &ev->tail;
     CUDA_TRY(h, mca::launch_tfm_eval(a, h->stream));
@@ -1608,8 +1606,8 @@ mca_status eval_explicit(mca_handle* h, size_t n, float wmax) {
   } else if (h->deep) {
     mca::DeepArgs a = deep_args(h);
     a.n_explicit = (int)n;
-    a.ex_idx = h->ex_idx;
-    a.ex_new = h->ex_new;
+    a.ex_idx = h->ex->idx;
+    a.ex_new = h->ex->new_w;
     a.ex_out = ev->dS;
     a.ex_tail = &ev->tail;
     CUDA_TRY(h, mca::launch_deep_eval(a, h->stream));
@@ -1618,8 +1616,8 @@ mca_status eval_explicit(mca_handle* h, size_t n, float wmax) {
   } else {
     mca::Mlp2Args a = mlp2_args(h);
     a.n_explicit = (int)n;
-    a.ex_idx = h->ex_idx;
-    a.ex_new = h->ex_new;
+    a.ex_idx = h->ex->idx;
+    a.ex_new = h->ex->new_w;
     a.ex_out = ev->dS;
     a.ex_tail = &ev->tail;
     if (!h->smem_records)            // the trial loop's grid barrier counts generations from 0
@@ -1649,12 +1647,11 @@ mca_status mca_eval_candidates(mca_handle* h, const uint32_t* flat_idx, const fl
     if (!std::isfinite(new_w[m])) return fail(h, MCA_ERR_INVALID, "new_w[%zu] not finite", m);
     wmax = std::max(wmax, std::fabs(new_w[m]));
   }
-  std::memcpy(h->ev_host->idx, flat_idx, sizeof(unsigned int) * n);
-  std::memcpy(h->ev_host->new_w, new_w, sizeof(float) * n);
-  // ex_idx and ex_new lie one after the other, as in EvalHost
-  CUDA_TRY(h, cudaMemcpyAsync(h->ex_idx, h->ev_host->idx,
-                              sizeof(h->ev_host->idx) + sizeof(float) * n, cudaMemcpyHostToDevice,
-                              h->stream));
+  mca::ExCands& in = h->ev_host->in;
+  std::memcpy(in.idx, flat_idx, sizeof(unsigned int) * n);
+  std::memcpy(in.new_w, new_w, sizeof(float) * n);
+  CUDA_TRY(h, cudaMemcpyAsync(h->ex, &in, offsetof(mca::ExCands, new_w) + sizeof(float) * n,
+                              cudaMemcpyHostToDevice, h->stream));
   const mca_status rc = eval_explicit(h, n, wmax);
   if (rc != MCA_OK) return rc;
   std::memcpy(dS, h->ev_host->dS, sizeof(double) * n);
@@ -1690,8 +1687,8 @@ mca_status mca_eval_trials(mca_handle* h, uint64_t seed, uint64_t tau, size_t n,
   a.seed = seed;
   a.tau0 = tau;
   a.rec = h->ev_host->prop;
-  a.ex_idx = h->ex_idx;
-  a.ex_new = h->ex_new;
+  a.ex_idx = h->ex->idx;
+  a.ex_new = h->ex->new_w;
   CUDA_TRY(h, mca::launch_propose(a, h->stream));
   h->launches++;
   const mca_status rc = eval_explicit(h, n, 0.0f);    // proposals are within the level
@@ -1830,8 +1827,7 @@ mca_status mca_create_transformer(const mca_tfm_spec* spec, const mca_domain* do
   h->st = reinterpret_cast<DevState*>(base + M.st);
   h->ctl = reinterpret_cast<mca::DeepCtl*>(base + M.ctl);
   h->trace = o.trace_cap > 0 ? reinterpret_cast<mca_trace_rec*>(base + M.trace) : nullptr;
-  h->ex_idx = reinterpret_cast<unsigned int*>(base + M.ex_idx);
-  h->ex_new = reinterpret_cast<float*>(base + M.ex_new);
+  h->ex = reinterpret_cast<mca::ExCands*>(base + M.ex);
   h->tfm_img = h->tc ? reinterpret_cast<float*>(base + M.wimg) : nullptr;
   h->tfm_img16 = h->tc ? base + M.wimg16 : nullptr;
   h->tfm_Xmid = h->tc ? reinterpret_cast<float*>(base + M.Xmid) : nullptr;

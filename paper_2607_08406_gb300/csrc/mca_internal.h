@@ -108,6 +108,12 @@ struct DevState {
   int pad;
 };
 
+// The candidates of an explicit evaluation, copied to the device in one piece.
+struct ExCands {
+  unsigned int idx[kKmax];
+  float new_w[kKmax];
+};
+
 // What an explicit evaluation reports beside its loss changes.
 struct ExTail {
   double S;                  // loss sum of the cached state
@@ -480,13 +486,11 @@ struct mca_handle {
   mca::DevState* st = nullptr;
   mca_trace_rec* trace = nullptr;
   int trace_cap = 0;
-  unsigned int* ex_idx = nullptr;
-  float* ex_new = nullptr;
+  mca::ExCands* ex = nullptr;
   // explicit evaluations: pinned host memory that the candidates are copied from and the kernels
   // write the results to
   struct EvalHost {
-    unsigned int idx[mca::kKmax];
-    float new_w[mca::kKmax];
+    mca::ExCands in;
     double dS[mca::kKmax];
     mca_trace_rec prop[mca::kKmax];
     mca::ExTail tail;
