@@ -1258,17 +1258,17 @@ __global__ void __launch_bounds__(kLoopThreads, 1) mlp2_window_loop(Mlp2Args a) 
         unsigned int spins = 0;
         for (;;) {
           const unsigned int tl = *(volatile unsigned int*)&s_redo_tail;
-          unsigned long long* q = &s_redo_q[tl % kRedoLen];
-          // (0: empty, or its writer is between two stores; looked at again after a new trial, or
-          // in the bounded wait below)
-          const unsigned long long e = tl != *(volatile unsigned int*)&s_redo_head
-                                           ? ld_acquire_cta_shared_u64(q) : 0ull;
+          // 0: no entry, or its writer is between two stores (looked at again after a new trial, or in the
+          // bounded wait below)
+          const unsigned long long e = ld_acquire_cta_shared_u64(&s_redo_q[tl % kRedoLen]);
           if (e != 0ull) {
-            if (atomicCAS(&s_redo_tail, tl, tl + 1u) != tl) continue;   // another producer took it
-            t = e - 1ull;
-            st_release_cta_shared_u64(q, 0ull);
-            ++n_again;
-            break;
+            if (atomicCAS(&s_redo_tail, tl, tl + 1u) == tl) {
+              t = e - 1ull;
+              st_release_cta_shared_u64(&s_redo_q[tl % kRedoLen], 0ull);
+              ++n_again;
+              break;
+            }
+            continue;                  // another producer took it
           }
           if (!have) {
             tn = atomicAdd(&s_next, 1ull);
