@@ -254,8 +254,8 @@ struct DeepArgs {
   ExTail* ex_tail;           // nullable
   // evaluation of candidate k < nscr (on the tensor cores with a dense chain, layer <= L-3): every field it
   // computes goes to scr[k * (L + 1) + m] (layer m: row j of the mutated layer, the full layers
-  // after it; m = L: the per-sample losses), so that an accepted candidate's fields are adopted
-  // by swapping pointers instead of recomputing them
+  // after it; m = L: the per-sample losses), so that an accepted candidate's fields are adopted instead
+  // of recomputed (tensor-core chain: by swapping pointers, SIMT chain: by a copy)
   float* const* scr;
   int nscr;
 };

@@ -10,8 +10,8 @@ size_t mlp2_window_smem_bytes(int RS) { return window_smem_bytes(RS); }
 // fixed at compile time; everything else takes run-time switches, which cost most in the windowed
 // loop, whose batch is one long instruction sequence: with them a batch took 14.6 us for a 7-class
 // Gaussian net of 1001 hidden neurons and 17.0 us for 2048 ReLU neurons under the Metropolis rule;
-// the variants (with the producers computing the rule's threshold) take 4.5 and 4.2 us. The
-// variants of each loss are compiled in their own file.
+// the variants (with the producers computing the rule's threshold) took 4.5 and 4.2 us, and take 3.3 and
+// 3.7 with what came since. The variants of each loss are compiled in their own file.
 static LoopKind loop_kind(const Mlp2Args& a) {
   if (a.n_explicit > 0) return a.smem_records ? kLoopEval : kLoopTrial;
   return a.window ? kLoopWindow : kLoopTrial;

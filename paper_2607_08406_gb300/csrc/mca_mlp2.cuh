@@ -638,11 +638,12 @@ __global__ void __launch_bounds__(kLoopThreads, 1) mlp2_trial_loop(Mlp2Args a) {
 // 64 hidden neurons every second slot goes stale before its batch; prepared again by the batch itself,
 // one after another, that took 8.9 us per batch, against 3.6.)
 //
-// A batch takes 3.3 to 3.9 us. Time stamps of 784-16384-10 on 60000 samples (an instrumented build, 4.6 us
-// a batch): 0.2 us is the CTAs' skew, 0.9 set-up beside the commit, 0.3 the barrier, 1.2 the evaluation,
-// 0.3 adding the shares, and 1.9 from there to the next batch: the slowest CTA's share reaching L2, the
-// poll, the decision and two barriers. Inside, registers are the limit: variants that spill a hundred bytes are
-// 5 to 10 % slower.
+// In the first thousands of trials a batch takes 3.3 to 3.9 us by network; in trials 200k to 1M of
+// 784-16384-10 on 60000 samples (29 % accepted, about seven candidates) 4.1 us. Time stamps of a batch of
+// that net near its start (an instrumented build; us since the first CTA began it): set-up and
+// commit done 1.05, barrier 1.37, the warps know their chunks 1.68, last chunk 2.62, shares added 2.92, next batch
+// 4.78. The last step, the slowest CTA's share reaching L2, the poll, the decision and two barriers, is the
+// longest. Inside, registers are the limit: variants that spill a hundred bytes are 5 to 10 % slower.
 // ------------------------------------------------------------------------------------------------
 struct WSlot {
   Cand c;
@@ -735,10 +736,8 @@ inline size_t window_smem_bytes(int RS) {
 // of instructions that one warp has to execute one after another, so a record is a vector per sample
 // (read with three or four 16-byte loads), output fields come in pairs (one instruction for two), and
 // the fields past the class count hold -infinity, whose exponential and sigmoid are 0, instead of a
-// test per field. (One 4-byte load and one instruction per field took, per batch, 4.50 us for
-// 391-1001-7 masked nets with MSE on 12347 samples, 4.17 us for 784-2048-10 ReLU nets with
-// cross-entropy on 30000; with vectors 3.70 and 4.03 us. 784-64-10, all of whose records fit a warp or
-// two: 3.66 and 3.68.)
+// test per field. (A batch of 391-1001-7 masked nets with MSE on 12347 samples: 4.50 us with one 4-byte load
+// and one instruction per field, 3.70 with vectors, all else as it was then.)
 //
 // M = 10 fields (up to 10 classes): 12 floats a sample, M = 14: 16 floats whose 16-byte parts are
 // permuted by the sample's number, so that the lanes of a warp, which read different samples, spread
@@ -1198,8 +1197,8 @@ __global__ void __launch_bounds__(kLoopThreads, 1) mlp2_window_loop(Mlp2Args a) 
   __shared__ unsigned long long s_redo_q[kRedoLen];
   __shared__ unsigned int s_redo_head, s_redo_tail;
   __shared__ unsigned long long s_bbytes, s_tau_hi, s_next, s_limit;
-  // CTA 0's statistics, here rather than in 20 registers of every thread (with them the kernels spilled, and
-  // a batch of the wide, ternary and ReLU nets took 4.07, 3.57 and 3.74 us, with them here 3.89, 3.52 and 3.67)
+  // CTA 0's statistics, here rather than in 20 registers of every thread: with them the kernels spill, and a
+  // batch of the wide net took 4.07 us instead of 3.89
   __shared__ unsigned long long s_cand, s_waste, s_bytes, s_bytes_back, s_trace;
   __shared__ double s_S;
   float* s_records = s_dyn;
@@ -1464,9 +1463,8 @@ __global__ void __launch_bounds__(kLoopThreads, 1) mlp2_window_loop(Mlp2Args a) 
             load_column<M>(s_w2c[sl], w);
             if (held && (c.ecnt + 31) / 32 <= wpc) {
               // every entry was the last one of some lane of warps 1.., which has its new loss: the
-              // losses are not computed again (with that, batches took 3.54, 4.28, 3.69, 3.52 and 3.94 us
-              // for the small, wide, ternary, masked and ReLU nets; without 3.36, 4.06, 3.60, 3.36, 3.73.
-              // Keeping the fields as well spills registers.)
+              // losses are not computed again (a batch of the wide net 4.28 us with, 4.06 without
+              // computing them; keeping the fields as well spills registers)
               if (hk == kst && he < c.ecnt) commit_entry<M>(R, w, nl, da, zn, he, hl, zrow);
             } else {
 #pragma unroll 1
@@ -1557,15 +1555,14 @@ __global__ void __launch_bounds__(kLoopThreads, 1) mlp2_window_loop(Mlp2Args a) 
       // ---- evaluate. A candidate's entries in this range are cut into chunks: 32 cached entries (from
       // shared memory), or a.SUB samples read from global memory. What bounds the evaluation is the
       // length of one warp's instruction sequence, so the warps share the candidates: wpc warps per
-      // candidate, warp j of them taking chunks j, j + wpc, ... (with the 80
-      // entries of the wide net on one warp, three per lane, a batch of 4096 Gaussian neurons took
-      // 4.24 us, with two to four warps 3.79 at the time). The chunks are fixed by the candidate
-      // and added in order, whatever the number of warps. The warp that finishes a candidate adds the
-      // CTA's share. The last three warps look at the slots ahead: before they evaluate when the
-      // others suffice for that, else afterwards. Warp 0, which waits for the other CTAs, is the last
-      // to get work. Each warp's part comes from tables, ahead of the barrier: with three divisions after it a
-      // batch took 3.69, 4.40, 3.83, 3.71 and 4.03 us (small, wide, ternary, masked, ReLU nets), with the
-      // tables 3.53, 4.28, 3.68, 3.52 and 3.94.
+      // candidate, warp j of them taking chunks j, j + wpc, ... (a batch of 4096 Gaussian neurons,
+      // 80 entries a candidate: 4.24 us with one warp per candidate, 3.79 with two to four). The chunks
+      // are fixed by the candidate and added in order, whatever the number of warps. The warp that
+      // finishes a candidate adds the CTA's share. The last three warps look at the slots ahead: before
+      // they evaluate when the others suffice for that, else afterwards. Warp 0, which waits for the
+      // other CTAs, is the last to get work. Each warp's part comes from tables, ahead of the
+      // barrier: with three divisions after it a batch of the wide net took 4.40 us, with the tables
+      // 4.28.
       unsigned long long* acc = a.accum + (size_t)(bidx % kAccBuffers) * kAccStride;
       const bool look_first = nlive * wpc <= kLookWarp0 - 1;
 #pragma unroll 1

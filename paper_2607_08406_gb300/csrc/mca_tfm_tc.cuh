@@ -271,8 +271,7 @@ __device__ __forceinline__ void attention(const RowCtx& c, const float (&q)[32],
   }
 }
 
-// The image entry of the accepted weight-matrix parameter (after the commit kernel, which reads the
-// old one).
+// Weight w, element (r, k) of a matrix, into its image with fp16 parts.
 __device__ __forceinline__ void tfm_f16_image_store(const TfmArgs& a, int mat, int b, int r, int k,
                                                     float w) {
   __half* img = reinterpret_cast<__half*>(a.wimg16);
@@ -283,6 +282,8 @@ __device__ __forceinline__ void tfm_f16_image_store(const TfmArgs& a, int mat, i
   img[o + kTfmF16Chunk / 4] = __float2half_rn(x - __half2float(h));
 }
 
+// The image entries of the accepted weight-matrix parameter (after the commit kernel, which reads the
+// old one).
 __device__ __forceinline__ void image_update(const TfmArgs& a, const DeepCand& c) {
   const Target tg = tc_target(a, c.idx, c.layer);
   if (tg.mat == kTcMatNone) return;
