@@ -34,7 +34,7 @@ METRIC = "MC mutation trials/sec (full-batch loss evals); fraction of HBM/TC roo
 # from one ncu capture (one pass, one launch: the first timed step, trials 200k..240k) of
 # `python bench.py --steps 20 --warmup 5 --no-e2e --no-cpu`, summarised in profiles/. It is only
 # valid for the kernel source and the workload it was measured on; anything else reports null.
-LOOP_TRAFFIC = {"source_sha1": "6287e992baef9cabbf10b88d40ec38254588b001",
+LOOP_TRAFFIC = {"source_sha1": "dfa8301bc3729353be5c4f8e47cacfbebf8b1bb8",
                 "workload": "mlp784-16384-10_ce_n60000", "bytes_per_trial": 374000.0}
 LOOP_SOURCES = tuple(f"paper_2607_08406_gb300/csrc/{f}" for f in (
     "mca_mlp2.cuh", "mca_mlp2.cu", "mca_mlp2_ce.cu", "mca_mlp2_mse.cu", "mca_device.cuh"))

@@ -639,7 +639,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1) mlp2_trial_loop(Mlp2Args a) {
 // one after another, that took 8.9 us per batch, against 3.6.)
 //
 // In the first thousands of trials a batch takes 3.3 to 3.9 us by network; in trials 200k to 1M of
-// 784-16384-10 on 60000 samples (29 % accepted, about seven candidates) 4.1 us. Time stamps of a batch of
+// 784-16384-10 on 60000 samples (29 % accepted, six candidates) 4.1 us. Time stamps of a batch of
 // that net near its start (an instrumented build; us since the first CTA began it): set-up and
 // commit done 1.05, barrier 1.37, the warps know their chunks 1.68, last chunk 2.62, shares added 2.92, next batch
 // 4.78. The last step, the slowest CTA's share reaching L2, the poll, the decision and two barriers, is the
