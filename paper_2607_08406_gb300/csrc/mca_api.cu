@@ -517,7 +517,7 @@ mca_status deep_raise(mca_handle* h, float bound) {
   if (!h->parts_f16) return MCA_OK;
   int wide = 0;
   CUDA_TRY(h, cudaMemsetAsync(h->flag, 0, sizeof(int), h->stream));
-  CUDA_TRY(h, mca::launch_deep_wide(deep_args(h), nullptr, 0.0f, 0.5f * bound, h->flag, h->stream));
+  CUDA_TRY(h, mca::launch_deep_wide(deep_args(h), nullptr, 0.5f * bound, h->flag, h->stream));
   CUDA_TRY(h, cudaMemcpyAsync(&wide, h->flag, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
   CUDA_TRY(h, cudaStreamSynchronize(h->stream));
   h->launches += 1;
@@ -597,6 +597,58 @@ float pow2_above(float x) {
   return std::ldexp(1.0f, std::min(e, 126));
 }
 
+// The largest magnitude that a trial may give a dense weight (perturbations: from 0).
+float deep_reach(const mca_handle* h) {
+  float v = h->dom.op == MCA_OP_REPLACE ? std::max(std::fabs(h->dom.lo), std::fabs(h->dom.hi))
+                                        : std::fabs(h->dom.delta);
+  for (size_t m = 1; m + 1 < h->layers.size(); ++m)
+    if (h->layers[m].wkind == MCA_W_TERNARY_I8) v = std::max(v, std::fabs(h->layers[m].scale));
+  return v;
+}
+
+// What the fp16 operands' scales follow from, of the parameters on the device: out[0] the largest magnitude of a
+// deep net's dense weights or of the Transformer's parameters (bits), out[1] dense weights out of the
+// fp16 parts' range. out: zeroed device memory.
+cudaError_t enqueue_bounds(mca_handle* h, int* out) {
+  if (h->tfm) return h->tc ? mca::launch_abs_max(h->params, h->P, out, h->stream) : cudaSuccess;
+  if (!h->tc_f16) return cudaSuccess;
+  const mca::DeepArgs a = deep_args(h);
+  h->launches += 2;
+  const cudaError_t e = mca::launch_deep_top(a, out, h->stream);
+  return e == cudaSuccess ? mca::launch_deep_wide(a, out, deep_reach(h), out + 1, h->stream) : e;
+}
+
+mca_status apply_bounds(mca_handle* h, const int* out) {
+  float top = 0.0f;
+  std::memcpy(&top, &out[0], sizeof(top));
+  if (h->tc_f16) {
+    h->wbound = pow2_above(std::max(top, deep_reach(h)));
+    h->parts_f16 = out[1] == 0;
+    for (size_t m = 1; m + 1 < h->layers.size(); ++m)
+      if (h->layers[m].wkind == MCA_W_TERNARY_I8 &&
+          std::fabs(h->layers[m].scale) < std::ldexp(h->wbound, -mca::kWideGap))
+        h->parts_f16 = false;
+  }
+  if (!h->tfm || !h->tc) return MCA_OK;
+  h->pmax = top;
+  return tfm_check_small(h);
+}
+
+// A resync that forgets what the parameters were: afterwards the handle is the one that mca_set_params
+// would make of them, so that a run resumed there goes on as this one does.
+mca_status resync_boundary(mca_handle* h) {
+  if (h->tc_f16 || (h->tfm && h->tc)) {
+    int out[2] = {0, 0};
+    CUDA_TRY(h, cudaMemsetAsync(h->flag, 0, sizeof(out), h->stream));
+    CUDA_TRY(h, enqueue_bounds(h, h->flag));
+    CUDA_TRY(h, cudaMemcpyAsync(out, h->flag, sizeof(out), cudaMemcpyDeviceToHost, h->stream));
+    CUDA_TRY(h, cudaStreamSynchronize(h->stream));
+    const mca_status rc = apply_bounds(h, out);
+    if (rc != MCA_OK) return rc;
+  }
+  return resync(h);
+}
+
 // Load parameters in the init format into the per-layer weight arrays.
 mca_status load_params(mca_handle* h, const float* params, const signed char* codes) {
   const bool pdev = is_device_ptr(params);
@@ -614,16 +666,11 @@ mca_status load_params(mca_handle* h, const float* params, const signed char* co
   }
   const float* src = pdev ? params : tmp;
   const signed char* csrc = codes ? (cdev ? codes : ctmp) : nullptr;
-  // [0] a non-finite value; [1] the largest magnitude of a deep net's dense weights, or of the
-  // Transformer's parameters; [2] dense weights out of the fp16 parts' range
+  // [0] a non-finite value; [1], [2] enqueue_bounds
   int* dflag = nullptr;
   cudaError_t e = cudaMalloc(&dflag, 3 * sizeof(int));
   if (e == cudaSuccess) e = cudaMemsetAsync(dflag, 0, 3 * sizeof(int), h->stream);
   if (e == cudaSuccess) e = mca::launch_count_nonfinite(src, P, dflag, h->stream);
-  if (e == cudaSuccess && h->tc_f16)
-    e = mca::launch_abs_max(src + h->off[1], h->off[h->layers.size() - 1] - h->off[1], dflag + 1,
-                            h->stream);
-  if (e == cudaSuccess && h->tfm && h->tc) e = mca::launch_abs_max(src, P, dflag + 1, h->stream);
   for (size_t l = 0; e == cudaSuccess && l < h->layers.size(); ++l) {
     const mca_layer& L = h->layers[l];
     const size_t n = (size_t)L.n_in * L.n_out;
@@ -631,17 +678,7 @@ mca_status load_params(mca_handle* h, const float* params, const signed char* co
                                n, h->w_eff[l], h->code[l], h->wfix[l], h->stream);
     h->launches++;
   }
-  // the dense weights' magnitude is at most max(their largest now times sc, reach)
-  float sc = 1.0f, reach = 0.0f;
-  if (h->tc_f16) {
-    for (const mca_layer& L : h->layers)   // ternary layers hold codes
-      if (L.wkind == MCA_W_TERNARY_I8) sc = std::max(sc, std::fabs(L.scale));
-    reach = h->dom.op == MCA_OP_REPLACE ? std::max(std::fabs(h->dom.lo), std::fabs(h->dom.hi))
-                                        : std::fabs(h->dom.delta);
-    if (e == cudaSuccess)
-      e = mca::launch_deep_wide(deep_args(h), dflag + 1, sc, reach, dflag + 2, h->stream);
-    h->launches++;
-  }
+  if (e == cudaSuccess) e = enqueue_bounds(h, dflag + 1);
   int hflag[3] = {0, 0, 0};
   if (e == cudaSuccess) e = cudaMemcpyAsync(hflag, dflag, sizeof(hflag), cudaMemcpyDeviceToHost,
                                             h->stream);
@@ -651,17 +688,7 @@ mca_status load_params(mca_handle* h, const float* params, const signed char* co
   if (ctmp) cudaFree(ctmp);
   CUDA_TRY(h, e);
   if (hflag[0]) return fail(h, MCA_ERR_NUMERIC, "non-finite parameter value");
-  float top = 0.0f;
-  std::memcpy(&top, &hflag[1], sizeof(top));
-  h->pmax = top;
-  if (h->tc_f16) {
-    h->wbound = pow2_above(std::max(top * sc, reach));
-    h->parts_f16 = hflag[2] == 0;
-    for (const mca_layer& L : h->layers)
-      if (L.wkind == MCA_W_TERNARY_I8 && std::fabs(L.scale) < std::ldexp(h->wbound, -mca::kWideGap))
-        h->parts_f16 = false;
-  }
-  return h->tfm && h->tc ? tfm_check_small(h) : MCA_OK;
+  return apply_bounds(h, &hflag[1]);
 }
 
 mca_status read_state(mca_handle* h, DevState* out) {
@@ -1424,9 +1451,12 @@ mca_status mca_run(mca_handle* h, uint64_t n_trials, uint64_t seed, mca_run_stat
       h->rate_acc = h->rate_acc * mca::kRateDecay + (ctl.kstar >= 0 ? 1.0f : 0.0f);
       h->rate_trials = h->rate_trials * mca::kRateDecay + (float)ctl.consumed;
       if (R > 0 && h->tau % R == 0) {
-        mca_status rc = resync(h);
+        mca_status rc = resync_boundary(h);
         if (rc != MCA_OK) return rc;
         h->resyncs++;
+        if (h->deep) a = deep_args(h);
+        a.seed = seed;
+        if (h->tfm) tfm_f16_args(h, &ta);
       }
     }
   }
@@ -1531,7 +1561,7 @@ mca_status mca_set_params(mca_handle* h, const float* params, const int8_t* code
 mca_status mca_resync(mca_handle* h) {
   if (!h) return fail(nullptr, MCA_ERR_INVALID, "NULL handle");
   if (h->broken) return fail(h, MCA_ERR_CUDA, "handle unusable after an earlier device error");
-  mca_status rc = resync(h);
+  mca_status rc = resync_boundary(h);
   if (rc != MCA_OK) return rc;
   DevState ds;
   rc = read_state(h, &ds);

@@ -645,15 +645,32 @@ __global__ void deep_split_kernel(DeepArgs a) {
     deep_tc_image_store(a, m, e / kTcW, e % kTcW, a.w[m][e]);
 }
 
-// One warp per row of a dense layer: are more than wide_allowance of its weights below 2^-kWideGap of the
-// bound? (Masked layers: of the weights behind the masks.)
-__global__ void deep_wide_kernel(DeepArgs a, const int* top, float sc, float floor, int* out) {
+// Row r of dense layer m: the weights, or those behind the masks.
+__device__ __forceinline__ const float* dense_row(const DeepArgs& a, int m, int r) {
+  return (a.wk[m] == MCA_W_MASKED_FP32 ? a.wfix[m] : a.w[m]) + (size_t)r * kTcW;
+}
+
+__global__ void deep_top_kernel(DeepArgs a, int* top) {
   const int m = blockIdx.y + 1, lane = threadIdx.x & 31;
   const int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (m > a.L - 2 || r >= kTcW) return;
-  const float b = fmaxf(floor, top ? __int_as_float(*top) * sc : 0.0f);
+  const float* w = dense_row(a, m, r);
+  int v = 0;                         // the bits of non-negative floats order like the floats
+#pragma unroll
+  for (int k = lane; k < kTcW; k += 32) v = max(v, __float_as_int(fabsf(w[k])));
+  v = __reduce_max_sync(0xffffffffu, v);
+  if (lane == 0) atomicMax(top, v);
+}
+
+// One warp per row of a dense layer: are more than wide_allowance of its weights below 2^-kWideGap of the
+// bound?
+__global__ void deep_wide_kernel(DeepArgs a, const int* top, float floor, int* out) {
+  const int m = blockIdx.y + 1, lane = threadIdx.x & 31;
+  const int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (m > a.L - 2 || r >= kTcW) return;
+  const float b = fmaxf(floor, top ? __int_as_float(*top) : 0.0f);
   const int limit = (__float_as_int(b) >> 23) + 1 - kWideGap;   // exponents below it
-  const float* w = (a.wk[m] == MCA_W_MASKED_FP32 ? a.wfix[m] : a.w[m]) + (size_t)r * kTcW;
+  const float* w = dense_row(a, m, r);
   unsigned int n = 0, low = 0;
 #pragma unroll
   for (int k = lane; k < kTcW; k += 32) {
@@ -668,9 +685,14 @@ __global__ void deep_wide_kernel(DeepArgs a, const int* top, float sc, float flo
 
 }  // namespace
 
-cudaError_t launch_deep_wide(const DeepArgs& a, const int* top, float sc, float floor, int* out,
+cudaError_t launch_deep_top(const DeepArgs& a, int* top, cudaStream_t s) {
+  deep_top_kernel<<<dim3(kTcW / 8, a.L - 2), 256, 0, s>>>(a, top);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_deep_wide(const DeepArgs& a, const int* top, float floor, int* out,
                              cudaStream_t s) {
-  deep_wide_kernel<<<dim3(kTcW / 8, a.L - 2), 256, 0, s>>>(a, top, sc, floor, out);
+  deep_wide_kernel<<<dim3(kTcW / 8, a.L - 2), 256, 0, s>>>(a, top, floor, out);
   return cudaGetLastError();
 }
 

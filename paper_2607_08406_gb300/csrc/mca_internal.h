@@ -267,9 +267,11 @@ cudaError_t launch_deep_commit(const DeepArgs& a, cudaStream_t s);  // grid ntil
 cudaError_t launch_deep_forward_layer(const DeepArgs& a, int l, cudaStream_t s);
 cudaError_t launch_deep_losses(const DeepArgs& a, cudaStream_t s);
 cudaError_t launch_deep_split(const DeepArgs& a, cudaStream_t s);     // W_hi / W_lo of all layers
-// *out = 1 if the dense weights are out of the fp16 parts' range under the bound pow2_above(max(*top
-// sc, floor)); top: bits of a float >= 0, or null. (*out is left alone otherwise.)
-cudaError_t launch_deep_wide(const DeepArgs& a, const int* top, float sc, float floor, int* out,
+// *top = bits of the dense weights' largest magnitude (of those behind the masks), at least its old value.
+cudaError_t launch_deep_top(const DeepArgs& a, int* top, cudaStream_t s);
+// *out = 1 if the dense weights are out of the fp16 parts' range under the bound pow2_above(max(*top,
+// floor)); top: bits of a float >= 0, or null. (*out is left alone otherwise.)
+cudaError_t launch_deep_wide(const DeepArgs& a, const int* top, float floor, int* out,
                              cudaStream_t s);
 cudaError_t launch_deep_eval_tc(const DeepArgs& a, cudaStream_t s);   // grid (Kb, ntiles)
 cudaError_t launch_deep_commit_tc(const DeepArgs& a, cudaStream_t s); // grid ntiles

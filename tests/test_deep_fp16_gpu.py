@@ -106,3 +106,43 @@ def test_deep_weights_of_a_wide_range(gpu_lib, case):
     cached = gpu_lib.mca_loss(h)
     gpu_lib.mca_resync(h)
     assert gpu_lib.mca_loss(h) == pytest.approx(cached, rel=TIE_REL)
+
+
+@pytest.mark.parametrize("kind", ["deep", "tfm"])
+def test_resume_where_a_large_weight_has_gone(gpu_lib, kind):
+    """A run that starts with one large weight (tf32 parts of the deep chain, a larger scale of the
+    Transformer's operands), which an accepted trial replaces: from the next resync on it is the run
+    that mca_set_params starts from the parameters there, bit for bit."""
+    n, period = 60, 20
+    if kind == "deep":
+        wl = W.mlp_deep(N=300, width=256, depth=4, n_trials=n, K=8)
+        lo, hi, big = 784 * 256, 784 * 256 + 3 * 65536, 1e10
+        create = gpu_lib.create_from_workload
+    else:
+        wl = W.char_transformer(batch=2, text_len=4000, n_trials=n, K=8,
+                                spec=W.TfmSpec(n_layer=1, d_ff=128))
+        lo, hi, big = 0, wl.n_params, 4.0
+        create = gpu_lib.create_from_tfm_workload
+    seed = 2
+    h = create(wl, trace_cap=n)
+    gpu_lib.mca_run(h, n, seed)
+    tr = gpu_lib.mca_get_trace(h, n)[:period]
+    k = int(np.flatnonzero((tr["idx"] >= lo) & (tr["idx"] < hi))[0])
+    wl.init = wl.init.copy()
+    wl.init[tr["idx"][k]] = np.float32(big)
+    full = create(wl, trace_cap=n, resync_period=period)
+    gpu_lib.mca_force_decisions(full, [k], [True])
+    gpu_lib.mca_run(full, n, seed)
+    part = create(wl, trace_cap=n, resync_period=period)
+    gpu_lib.mca_force_decisions(part, [k], [True])
+    gpu_lib.mca_run(part, period, seed)
+    params = gpu_lib.mca_get_params(part, wl.n_params)
+    assert np.abs(params[lo:hi]).max() < 2.0
+    again = create(wl, trace_cap=n, resync_period=period)
+    gpu_lib.mca_set_params(again, params, tau=period)
+    gpu_lib.mca_run(again, n - period, seed)
+    assert np.array_equal(gpu_lib.mca_get_trace(again, n), gpu_lib.mca_get_trace(full, n)[period:])
+    assert gpu_lib.mca_loss(again) == gpu_lib.mca_loss(full)
+    gpu_lib.mca_resync(part)
+    gpu_lib.mca_run(part, n - period, seed)
+    assert gpu_lib.mca_loss(part) == gpu_lib.mca_loss(full)
